@@ -33,7 +33,7 @@
 #include <type_traits>
 
 #include "check.cuh"
-#include "ops.cuh"
+#include "kmer.cuh"
 
 namespace sg {
 
@@ -73,44 +73,6 @@ struct Bloom {
     }
 };
 
-// Batches: the job prefix of a window, from the base offset of each job's first read (jpos[b] =
-// off[ro[b]], jpos[njobs] = total). A window lies in the last job b with jpos[b] <= its position
-// (windows never cross reads, and empty jobs start where the next one does). The cursor keeps the
-// last job's range, so increasing positions search only when they leave it.
-struct JobPos {
-    const int64_t *jpos;  // nullptr: one read set, no prefix
-    int64_t njobs;
-    int kbits;  // 2k
-};
-
-struct JobPosCursor {
-    JobPos m;
-    int64_t jb = 0, jlo = 0, jhi = -1;
-    __device__ __forceinline__ uint64_t prefix(int64_t q) {
-        if (!m.jpos) return 0;
-        if (q < jlo || q >= jhi) {
-            int64_t lo = 0, hi = m.njobs;
-            while (hi - lo > 1) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (m.jpos[mid] <= q) lo = mid; else hi = mid;
-            }
-            jb = lo;
-            jlo = m.jpos[lo];
-            jhi = m.jpos[lo + 1];
-        }
-        return (uint64_t)jb << m.kbits;
-    }
-};
-
-__global__ void job_pos_kernel(const int64_t *__restrict__ ro, int64_t njobs, const int64_t *__restrict__ off,
-                               int64_t n, int64_t *__restrict__ jpos) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > njobs) return;
-    int64_t r = ro[b];
-    r = r < 0 ? 0 : (r > n ? n : r);
-    jpos[b] = off[r];
-}
-
 // Staged bases: the block's chunk as 32-bit words (4 bases each), one pad word after every 8, so
 // that thread t's 32-base segment starts at word 9t and a warp reading the j-th word of its
 // segments hits 32 distinct banks. Bytes past the end of the sequence read as 'N'.
@@ -145,7 +107,6 @@ __device__ __forceinline__ void load_chunk(uint32_t *smw, const uint8_t *__restr
 // (window_key). Thread t of block b covers windows and bases b * KM_CHUNK + t * KM_W + j, j < KM_W,
 // reading bases [t * KM_W, t * KM_W + KM_W + k - 1) of the block's chunk. K > 0 makes k a
 // compile-time constant (K == 0: k taken from k_rt).
-constexpr uint64_t WC_STRAND = 1ull << 63;
 constexpr uint32_t H_NONE = 0xFFFFFFFFu;
 constexpr uint32_t B1_SEED = 0x9e3779b9u, B2_SEED = 0x7f4a7c15u;
 static_assert(KM_W == 32, "one packed word per thread");
@@ -218,22 +179,6 @@ __global__ void __launch_bounds__(KM_NT) pack_kernel(const uint8_t *__restrict__
         }
     }
     P[qs >> 5] = pw;
-}
-
-// Key of window q = 32g + lane from P[g] = w0 and P[g + 1] = w1 (a valid window): the canonical
-// code (with the job prefix) | strand << 63. The 2k bits from
-// bit 2 * lane of w1:w0 hold the window's bases, first base lowest; complementing them gives the
-// reverse complement's code (last base's complement highest), and reversing the order of the
-// 2-bit groups gives the forward code (first base highest).
-__device__ __forceinline__ uint64_t window_key(uint64_t w0, uint64_t w1, int lane, int k, JobPosCursor &jc,
-                                               int64_t q) {
-    const int sh = 2 * lane;
-    const uint64_t x = sh ? (w0 >> sh) | (w1 << (64 - sh)) : w0;
-    const uint64_t rc = ~x & ((1ull << (2 * k)) - 1);  // k <= 31
-    uint64_t y = __brevll(x);
-    y = ((y >> 1) & 0x5555555555555555ull) | ((y & 0x5555555555555555ull) << 1);
-    const uint64_t fw = y >> (64 - 2 * k);
-    return jc.prefix(q) | (fw < rc ? fw : rc) | (rc < fw ? WC_STRAND : 0ull);
 }
 
 // One launch per slice [w_lo, w_hi) of B1's words: every launch streams all window hashes but
@@ -635,21 +580,6 @@ __global__ void resolve_kernel(uint64_t *__restrict__ val, int64_t nc, const int
     val[i] = resolve_pos(val[i], off, n, lut, nb);
 }
 
-__global__ void validate_offsets_kernel(const int64_t *__restrict__ off, int64_t n, int64_t total,
-                                        uint32_t *__restrict__ err) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > n) return;
-    int64_t a = off[i];
-    bool bad = false;
-    if (i == 0 && a != 0) bad = true;
-    if (i == n && a != total) bad = true;
-    if (i < n) {
-        int64_t b = off[i + 1];
-        if (b < a || b - a >= ((int64_t)1 << 31)) bad = true;
-    }
-    if (bad) atomicOr(err, (uint32_t)DEV_INVALID);
-}
-
 // head[i] = 1 where a new code starts.
 __global__ void seg_head_kernel(const uint64_t *__restrict__ key, int64_t nc, uint32_t *__restrict__ head) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -699,15 +629,14 @@ __global__ void keep_kernel(const uint32_t *__restrict__ head, const int64_t *__
     keep[i] = (rel[s] && first) ? 1u : 0u;
 }
 
-// Writes At's entries, its row pointers, the column codes, and the (read, col|val) pairs that
-// are sorted into A.
+// Writes At's entries, its row pointers and the column codes.
 __global__ void emit_at_kernel(const uint32_t *__restrict__ head, const int64_t *__restrict__ seg_excl,
                                const uint32_t *__restrict__ rel, const int64_t *__restrict__ col_of_seg,
                                const uint32_t *__restrict__ keep, const int64_t *__restrict__ out_pos,
                                const uint64_t *__restrict__ key, const uint64_t *__restrict__ val, int64_t nc,
                                int64_t m, int64_t nnz, int32_t *__restrict__ at_col, uint32_t *__restrict__ at_val,
                                int64_t *__restrict__ at_rp, uint64_t *__restrict__ codes,
-                               uint32_t *__restrict__ a_key, uint64_t *__restrict__ a_val, int kbits,
+                               int kbits,
                                unsigned long long *__restrict__ job_ncols) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) at_rp[m] = nnz;
@@ -726,8 +655,6 @@ __global__ void emit_at_kernel(const uint32_t *__restrict__ head, const int64_t 
         uint32_t r = (uint32_t)(val[i] >> 32), v = (uint32_t)val[i];
         at_col[o] = (int32_t)r;
         at_val[o] = v;
-        a_key[o] = r;
-        a_val[o] = ((uint64_t)col_of_seg[s] << 32) | v;
     }
 }
 
@@ -781,14 +708,13 @@ __global__ void seg_flags_kernel(const uint64_t *__restrict__ key, const uint64_
     if (threadIdx.x == 0 && s_kept) atomicAdd(nkeep, (unsigned long long)s_kept);
 }
 
-// Writes At's entries, its row pointers, the column codes and the (read, col|val) pairs sorted
-// into A, from the exclusive scan of the fused flags (low 31 bits: reliable segments before, high
+// Writes At's entries, its row pointers and the column codes, from the exclusive scan of the fused flags (low 31 bits: reliable segments before, high
 // bits: kept entries before; pre[nc] = the totals). Entry i's own flags are pre[i + 1] - pre[i].
 __global__ void emit_fused_kernel(const uint64_t *__restrict__ pre,
                                   const uint64_t *__restrict__ key, const uint64_t *__restrict__ val, int64_t nc,
                                   int64_t m, int64_t nnz, int32_t *__restrict__ at_col, uint32_t *__restrict__ at_val,
                                   int64_t *__restrict__ at_rp, uint64_t *__restrict__ codes,
-                                  uint32_t *__restrict__ a_key, uint64_t *__restrict__ a_val, int kbits,
+                                  int kbits,
                                   unsigned long long *__restrict__ job_ncols) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) at_rp[m] = nnz;
@@ -810,8 +736,6 @@ __global__ void emit_fused_kernel(const uint64_t *__restrict__ pre,
         const uint32_t r = (uint32_t)(val[i] >> 32), v = (uint32_t)val[i];
         at_col[o] = (int32_t)r;
         at_val[o] = v;
-        a_key[o] = r;
-        a_val[o] = ((uint64_t)col << 32) | v;
     }
 }
 
@@ -824,7 +748,7 @@ __global__ void emit_fused_kernel(const uint64_t *__restrict__ pre,
 //         segment) << 1 -- and the tile's two totals;
 //   emit: after exclusive scans of the tile totals, each tile recovers every candidate's column
 //         and At slot from its tile's prefixes and a block scan of its flags, and writes At, the
-//         codes and the pairs sorted into A (emit_fused_kernel's outputs).
+//         codes (emit_fused_kernel's outputs).
 // Keys are equal when they lie in the same bucket range and agree in their code bits. "First of
 // its read" tests whether the previous candidate's window lies in the extent [off[r], off[r + 1])
 // of the read r holding this one; the reads are found by searches that run for DS_GROUP
@@ -1032,7 +956,6 @@ __global__ void __launch_bounds__(DS_NT, 4) seg_emit_kernel(SegArgs a, const uin
                                                         const int64_t *__restrict__ pkeep, int64_t m, int64_t nnz,
                                                         int32_t *__restrict__ at_col, uint32_t *__restrict__ at_val,
                                                         int64_t *__restrict__ at_rp, uint64_t *__restrict__ codes,
-                                                        uint32_t *__restrict__ a_key, uint64_t *__restrict__ a_val,
                                                         unsigned long long *__restrict__ job_ncols) {
     constexpr int NW = DS_NT / 32;
     __shared__ uint64_t sk[DS_SMEM];
@@ -1129,46 +1052,12 @@ __global__ void __launch_bounds__(DS_NT, 4) seg_emit_kernel(SegArgs a, const uin
                 const uint32_t v = (uint32_t)(q[u] - a.off[r[u]]) | (uint32_t)((p & 1u) << 31);
                 at_col[o] = (int32_t)rr;
                 at_val[o] = v;
-                a_key[o] = rr;
-                a_val[o] = ((uint64_t)col << 32) | v;
             }
         }
     }
 }
 
-// Row pointers of A from the read ids of its entries, sorted ascending.
-__global__ void rowptr_from_sorted_kernel(const uint32_t *__restrict__ rows, int64_t nnz, int64_t n,
-                                          int64_t *__restrict__ rp) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e > nnz) return;
-    int64_t prev = (e == 0) ? -1 : (int64_t)rows[e - 1];
-    int64_t cur = (e == nnz) ? n : (int64_t)rows[e];
-    // always in bounds, even for rows that a failed sort left unsorted (the call then fails)
-    if (!SG_IN_BOUNDS(prev >= -1 && cur <= n && prev <= cur, 107, cur) || prev < -1 || cur > n) return;
-    for (int64_t r = prev + 1; r <= cur; r++) rp[r] = e;
-}
-
-__global__ void split_pairs_kernel(const uint64_t *__restrict__ pv, int64_t nnz, int32_t *__restrict__ col,
-                                   uint32_t *__restrict__ val) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nnz) return;
-    uint64_t x = pv[e];
-    col[e] = (int32_t)(x >> 32);
-    val[e] = (uint32_t)x;
-}
-
 static inline int64_t blocks_for(int64_t n, int nt) { return (n + nt - 1) / nt; }
-
-// Runs f with k as a compile-time constant for the common k (17 is the paper's), else 0.
-template <class F>
-static sg_status dispatch_k(int k, F &&f) {
-    switch (k) {
-        case 17: return f(std::integral_constant<int, 17>{});
-        case 21: return f(std::integral_constant<int, 21>{});
-        case 31: return f(std::integral_constant<int, 31>{});
-        default: return f(std::integral_constant<int, 0>{});
-    }
-}
 
 // jm.ro == nullptr: one read set with range [lo, hi]. Otherwise a batch: lohi (device) holds
 // each job's range and job_ncols (device, zeroed, njobs entries) receives each job's column count.
@@ -1177,10 +1066,33 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
                      cudaStream_t s, Scratch &sc, JobMap jm, const uint32_t *lohi,
                      unsigned long long *job_ncols, uint32_t hmax) {
     const int NT = 256;
-    uint32_t *err = sc.get<uint32_t>(1);
+    uint32_t *err = sc.get<uint32_t>(4);  // error word | longest read (u64 at [2])
     if (!err) return SG_ERR_OOM;
-    SG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-    SG_LAUNCH("validate_offsets", validate_offsets_kernel, blocks_for(n + 1, NT), NT, 0, s, off, n, total, err);
+    unsigned long long *maxlen = (unsigned long long *)(err + 2);
+    SG_CUDA_TRY(cudaMemsetAsync(err, 0, 4 * sizeof(uint32_t), s));
+    SG_TRY(check_offsets(off, n, total, err, maxlen, s));
+    // A from At: rows by read, and the last word on the call's errors
+    auto transpose = [&](int pbits) -> sg_status {
+        SG_ALLOC(A->row_ptr, int64_t, n + 1, s);
+        SG_ALLOC(A->col, int32_t, At->nnz, s);
+        SG_ALLOC(A->val, uint32_t, At->nnz, s);
+        A->n_rows = n; A->n_cols = At->n_rows; A->nnz = At->nnz;
+        SG_TRY(transpose_impl(At, A, pbits, s, err));
+        uint32_t herr = 0;
+        SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));
+        return herr ? timeout_error("build_kmer_matrix") : SG_OK;
+    };
+    {
+        bool taken = false;
+        int pbits = 31;
+        Scratch sb(s);
+        SG_TRY(build_bucketed(seq, off, n, total, k, lo, hi, At, codes_out, s, sb, jm, lohi, job_ncols, hmax, err,
+                              maxlen, &pbits, &taken));
+        if (taken) {
+            StageScope mat("CreateSpMat", s);
+            return transpose(pbits);
+        }
+    }
 
     const int64_t nblk = blocks_for(total, KM_CHUNK);
     const int use_bloom = lo >= 2 ? 1 : 0;
@@ -1363,6 +1275,8 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
     for (int b = 0; b <= bk.nb; b++)
         SG_CUDA_TRY(cudaMemcpyAsync(&bs.start[b], wpos + (int64_t)b * nwarp, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     uint32_t herr = 0;
+    unsigned long long longest = 0;
+    SG_CUDA_TRY(cudaMemcpyAsync(&longest, maxlen, sizeof(longest), cudaMemcpyDeviceToHost, s));
     SG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     SG_CUDA_TRY(cudaStreamSynchronize(s));
     const int64_t nc = bs.start[bk.nb];
@@ -1543,52 +1457,30 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
     SG_ALLOC(*codes_out, uint64_t, m, s);
     At->n_rows = m; At->n_cols = n; At->nnz = nnz;
 
-    stage.emplace("CreateSpMat", s);  // a5: At, then A by a sort on the read
-    uint32_t *ak0 = sc.get<uint32_t>(nnz);
-    uint64_t *av0 = sc.get<uint64_t>(nnz);
-    if (!ak0 || !av0) return SG_ERR_OOM;
+    stage.emplace("CreateSpMat", s);  // a5: At, then A by grouping its entries by read
     if (direct) {
         const int64_t ntiles = (nc + DS_TILE - 1) / DS_TILE;
         SG_LAUNCH("emit_at", seg_emit_kernel, ntiles, DS_NT, 0, s, dargs, (const uint32_t *)dflags,
                   (const int64_t *)dpre, (const int64_t *)(dpre + ntiles + 1), m, nnz, At->col, At->val,
-                  At->row_ptr, *codes_out, ak0, av0, job_ncols);
+                  At->row_ptr, *codes_out, job_ncols);
     } else if (fused)
         SG_LAUNCH("emit_at", emit_fused_kernel, blocks_for(nc > 0 ? nc : 1, NT), NT, 0, s, (const uint64_t *)pre, key,
-                  (const uint64_t *)val, nc, m, nnz, At->col, At->val, At->row_ptr, *codes_out, ak0, av0, 2 * k,
+                  (const uint64_t *)val, nc, m, nnz, At->col, At->val, At->row_ptr, *codes_out, 2 * k,
                   job_ncols);
     else
         SG_LAUNCH("emit_at", emit_at_kernel, blocks_for(nc > 0 ? nc : 1, NT), NT, 0, s, head, seg_excl, rel,
-                  col_of_seg, keep, out_pos, key, val, nc, m, nnz, At->col, At->val, At->row_ptr, *codes_out, ak0,
-                  av0, 2 * k, job_ncols);
+                  col_of_seg, keep, out_pos, key, val, nc, m, nnz, At->col, At->val, At->row_ptr, *codes_out, 2 * k,
+                  job_ncols);
     for (const void *p : {(const void *)key, (const void *)val, (const void *)pre, (const void *)sorted,
                           (const void *)dflags, (const void *)dpre,
                           (const void *)head, (const void *)seg_excl, (const void *)seg_start, (const void *)rel,
                           (const void *)col_of_seg, (const void *)keep, (const void *)out_pos})
         if (p) sc.release(p);
-    SG_ALLOC(A->row_ptr, int64_t, n + 1, s);
-    SG_ALLOC(A->col, int32_t, nnz, s);
-    SG_ALLOC(A->val, uint32_t, nnz, s);
-    A->n_rows = n; A->n_cols = m; A->nnz = nnz;
-    uint32_t *ak1 = sc.get<uint32_t>(nnz);
-    uint64_t *av1 = sc.get<uint64_t>(nnz);
-    if (!ak1 || !av1) return SG_ERR_OOM;
-    int rbits = 0;
-    while (rbits < 32 && ((int64_t)1 << rbits) < n) rbits++;
     kmer_stats().m = m;
     kmer_stats().nnz = nnz;
-    kmer_stats().a_sort_passes = nnz > 1 ? (rbits + 7) / 8 : 0;
-    bool aalt = false;
-    const bool split = nnz > 1 && rbits > 0;  // the sort's last pass writes A's columns and values
-    if (split)
-        SG_TRY(radix_sort_pairs_split(ak0, av0, ak1, av1, nnz, rbits, &aalt, (uint32_t *)A->col, A->val, s, err));
-    const uint32_t *arow = aalt ? ak1 : ak0;
-    const uint64_t *apv = aalt ? av1 : av0;
-    SG_LAUNCH("rowptr_from_sorted", rowptr_from_sorted_kernel, blocks_for(nnz + 1, NT), NT, 0, s, arow, nnz, n,
-              A->row_ptr);
-    if (!split) SG_LAUNCH("split_pairs", split_pairs_kernel, blocks_for(nnz, NT), NT, 0, s, apv, nnz, A->col, A->val);
-    SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));  // the sort of A waits between tiles
-    if (herr) return timeout_error("build_kmer_matrix");
-    return SG_OK;
+    int pbits = 1;
+    while (((unsigned long long)1 << pbits) < longest) pbits++;
+    return transpose(pbits);
 }
 
 }  // namespace sg

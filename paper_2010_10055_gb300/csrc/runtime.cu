@@ -283,6 +283,8 @@ static Tunable g_tunables[] = {
                                           // (B2: a quarter of it)
     {"bloom_scatter_cfg", 0, 0, 2},       // bin scatter tile: 0 512x16, 1 256x16, 2 256x32 hashes
     {"bloom_scatter_levels", 0, 0, 2},    // passes grouping hashes by bin (0: two beyond 4096 bins)
+    {"kmer_bucketed", 1, 0, 1},           // 1: windows grouped by code and counted in shared memory where
+                                          // that form applies; 0: filters and radix sort (general form)
     {"kmer_sort_buckets", 3, 0, 3},       // at most this many top code bits become candidate buckets
     {"kmer_direct_seg", 1, 0, 1},         // 1: segments and At straight from the sorted packed keys
     {"radix_match", 0, 0, 1},             // radix sort ranking: 1 one match instruction per key, 0 ballots
