@@ -14,10 +14,10 @@ namespace sg {
 // Record a printf-style description of the current error for sg_last_error().
 void set_error(const char *fmt, ...);
 
-// Device allocation through the installed allocator (default cudaMallocAsync on `s`).
-// Returns nullptr and records an error on failure. bytes == 0 allocates 16 bytes so that the
-// result is always a valid, distinct pointer.
-void *dalloc(size_t bytes, cudaStream_t s);
+// Device allocation through the installed allocator (default: the library's stream-ordered pools,
+// one for temporaries of a call and one for outputs). Returns nullptr and records an error on
+// failure. bytes == 0 allocates 16 bytes so that the result is always a valid, distinct pointer.
+void *dalloc(size_t bytes, cudaStream_t s, bool temporary = false);
 void dfree(void *p, cudaStream_t s);
 
 // Launch bookkeeping: counts launches and, while profiling is on, brackets them with events.
@@ -50,7 +50,7 @@ struct Scratch {
     Scratch(const Scratch &) = delete;
     Scratch &operator=(const Scratch &) = delete;
     template <class T> T *get(size_t count) {
-        void *p = dalloc(count * sizeof(T), s);
+        void *p = dalloc(count * sizeof(T), s, true);
         if (p) ptrs.push_back(p);
         return (T *)p;
     }

@@ -40,16 +40,19 @@ static sg_free_fn g_free = nullptr;
 static void *g_alloc_ctx = nullptr;
 static std::atomic<int64_t> g_fail_after{0};
 
-// The library's own stream-ordered pool on each device. Its release threshold is unbounded, so
-// memory freed at the end of one call is reused by the next instead of being unmapped at every
-// synchronisation (the default pool's threshold of 0 returns it to the driver each time). The
-// pool belongs to this process and disappears with it.
+// The library's own stream-ordered pools on each device: one for the temporaries of a call, one for
+// outputs. Their release threshold is unbounded, so memory freed at the end of one call is reused by
+// the next instead of being unmapped at every synchronisation (the default pool's threshold of 0
+// returns it to the driver each time). Outputs live across calls: in one pool with the temporaries
+// they came to lie inside the large blocks that the next call wants back whole, and the driver
+// remapped tens of GB to make one (20-75 ms of a 400 ms step at 100 Mbp 40x). The pools belong to
+// this process and disappear with it.
 int64_t tune(const char *name);
 static std::mutex g_pool_mu;
-static cudaMemPool_t g_pools[256];
+static cudaMemPool_t g_pools[256][2];
 static bool g_pool_tried[256];
 
-static cudaMemPool_t library_pool() {
+static cudaMemPool_t library_pool(int which) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) {
         cudaGetLastError();
@@ -58,24 +61,42 @@ static cudaMemPool_t library_pool() {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     if (!g_pool_tried[dev]) {
         g_pool_tried[dev] = true;
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
-        if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
-            uint64_t thr = ~0ull;
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-            int reuse = tune("pool_cross_stream_reuse") ? 1 : 0;
-            cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowOpportunistic, &reuse);
-            cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &reuse);
-            g_pools[dev] = pool;
-        } else {
-            cudaGetLastError();
+        for (int w = 0; w < 2; w++) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t pool = nullptr;
+            if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+                uint64_t thr = ~0ull;
+                cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+                int reuse = tune("pool_cross_stream_reuse") ? 1 : 0;
+                cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowOpportunistic, &reuse);
+                cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &reuse);
+                g_pools[dev][w] = pool;
+            } else {
+                cudaGetLastError();
+            }
         }
     }
-    return g_pools[dev];
+    return g_pools[dev][which];
+}
+
+// Bytes of both pools under one attribute; false if it cannot be read.
+static bool pool_bytes(cudaMemPoolAttr attr, uint64_t *out) {
+    *out = 0;
+    for (int w = 0; w < 2; w++) {
+        cudaMemPool_t pool = library_pool(w);
+        uint64_t v = 0;
+        if (!pool) continue;
+        if (cudaMemPoolGetAttribute(pool, attr, &v) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        *out += v;
+    }
+    return true;
 }
 
 // Multiprocessors of the current device (152 on a GB300), for grid sizes; read once per device.
@@ -104,18 +125,14 @@ size_t device_bytes_available() {
         cudaGetLastError();
         return 0;
     }
-    cudaMemPool_t pool = g_alloc ? nullptr : library_pool();
-    if (pool) {
-        uint64_t reserved = 0, used = 0;
-        if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
-            cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
-            free_b += (size_t)(reserved - used);
-        cudaGetLastError();
-    }
+    uint64_t reserved = 0, used = 0;
+    if (!g_alloc && pool_bytes(cudaMemPoolAttrReservedMemCurrent, &reserved) &&
+        pool_bytes(cudaMemPoolAttrUsedMemCurrent, &used) && reserved > used)
+        free_b += (size_t)(reserved - used);
     return free_b;
 }
 
-void *dalloc(size_t bytes, cudaStream_t s) {
+void *dalloc(size_t bytes, cudaStream_t s, bool temporary) {
     if (bytes == 0) bytes = 16;
     int64_t f = g_fail_after.load();
     if (f > 0) {
@@ -135,13 +152,15 @@ void *dalloc(size_t bytes, cudaStream_t s) {
         }
         return p;
     }
-    cudaMemPool_t pool = library_pool();
+    cudaMemPool_t pool = library_pool(temporary ? 0 : 1);
     cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, s) : cudaMallocAsync(&p, bytes, s);
     if (e != cudaSuccess && pool) {
-        // the pool keeps freed memory reserved; blocks freed by earlier calls may not fit this
-        // request. Once this stream's frees have completed, give the unused part back and retry.
+        // the pools keep freed memory reserved; blocks freed by earlier calls may not fit this
+        // request. Once this stream's frees have completed, give the unused parts back and retry.
         cudaGetLastError();
-        if (cudaStreamSynchronize(s) == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess)
+        cudaMemPool_t other = library_pool(temporary ? 1 : 0);
+        if (cudaStreamSynchronize(s) == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess &&
+            (!other || cudaMemPoolTrimTo(other, 0) == cudaSuccess))
             e = cudaMallocFromPoolAsync(&p, bytes, pool, s);
     }
     if (e != cudaSuccess) {
@@ -149,10 +168,9 @@ void *dalloc(size_t bytes, cudaStream_t s) {
         size_t free_b = 0, total_b = 0;
         uint64_t reserved = 0, used = 0;
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
-        if (pool && (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
-                     cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess))
-            cudaGetLastError();
-        set_error("cudaMallocAsync(%zu bytes) failed: %s (device: %.1f of %.1f GB free; library pool: %.1f GB "
+        pool_bytes(cudaMemPoolAttrReservedMemCurrent, &reserved);
+        pool_bytes(cudaMemPoolAttrUsedMemCurrent, &used);
+        set_error("cudaMallocAsync(%zu bytes) failed: %s (device: %.1f of %.1f GB free; library pools: %.1f GB "
                   "reserved, %.1f GB in use)",
                   bytes, cudaGetErrorString(e), free_b / 1e9, total_b / 1e9, reserved / 1e9, used / 1e9);
         return nullptr;
@@ -399,12 +417,10 @@ uint64_t sg_launch_count(void) { return sg::g_launches.load(); }
 
 sg_status sg_memory_stats(uint64_t *reserved, uint64_t *in_use, uint64_t *in_use_peak) {
     uint64_t r = 0, u = 0, h = 0;
-    cudaMemPool_t pool = sg::g_alloc ? nullptr : sg::library_pool();
-    if (pool && (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &r) != cudaSuccess ||
-                 cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &u) != cudaSuccess ||
-                 cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &h) != cudaSuccess)) {
-        cudaGetLastError();
-        sg::set_error("memory_stats: the pool cannot be queried");
+    if (!sg::g_alloc && !(sg::pool_bytes(cudaMemPoolAttrReservedMemCurrent, &r) &&
+                          sg::pool_bytes(cudaMemPoolAttrUsedMemCurrent, &u) &&
+                          sg::pool_bytes(cudaMemPoolAttrUsedMemHigh, &h))) {
+        sg::set_error("memory_stats: the pools cannot be queried");
         return SG_ERR_CUDA;
     }
     if (reserved) *reserved = r;
@@ -414,9 +430,11 @@ sg_status sg_memory_stats(uint64_t *reserved, uint64_t *in_use, uint64_t *in_use
 }
 
 void sg_memory_reset_peak(void) {
-    cudaMemPool_t pool = sg::g_alloc ? nullptr : sg::library_pool();
-    uint64_t zero = 0;
-    if (pool && cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero) != cudaSuccess) cudaGetLastError();
+    for (int w = 0; w < 2 && !sg::g_alloc; w++) {
+        cudaMemPool_t pool = sg::library_pool(w);
+        uint64_t zero = 0;
+        if (pool && cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero) != cudaSuccess) cudaGetLastError();
+    }
 }
 
 void sg_last_kmer_stats(sg_kmer_stats *out) {
