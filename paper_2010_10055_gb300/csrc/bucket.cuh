@@ -12,6 +12,7 @@
 // comparison. No pass depends on the order of another block's writes, so nothing waits.
 #pragma once
 
+#include "check.cuh"
 #include "prim.cuh"
 
 namespace sg {
@@ -93,6 +94,7 @@ struct KbPlan {
     unsigned long long *cur2;     // [nsub_max] write cursors of the second pass
     uint32_t *count2;             // [nsub_max + 1]
     int64_t nsub_max;
+    int64_t cap;                  // records a buffer holds
     // the bucket's prefix, its first code (below the prefix) and its code bits
     __device__ __forceinline__ int prefix(int64_t b) const { return two ? (int)sub2p[b] : (int)b; }
 };
@@ -117,7 +119,7 @@ template <class K, bool BINARR, class BinOf>
 __device__ __forceinline__ void scatter_tail(ScatterSmem<K> &sm, uint32_t *cnt, unsigned long long *gb,
                                              uint16_t *sbin, int nb, const typename K::T (&key)[K::ITEMS],
                                              const uint32_t (&br)[K::ITEMS], unsigned long long *__restrict__ cur,
-                                             typename K::T *__restrict__ out, BinOf &&binof) {
+                                             typename K::T *__restrict__ out, int64_t cap, BinOf &&binof) {
     constexpr int PER = KB_MAXBINS / KB_NT;  // bins t, t + KB_NT, ... belong to thread t
     __syncthreads();
     // runs are reserved first: the atomics travel while the tile is scanned and ordered
@@ -144,6 +146,7 @@ __device__ __forceinline__ void scatter_tail(ScatterSmem<K> &sm, uint32_t *cnt, 
     for (int u = 0; u < K::ITEMS; u++)
         if (br[u] != 0xFFFFFFFFu) {
             const uint32_t p = cnt[br[u] >> 16] + (br[u] & 0xFFFFu);
+            if (!SG_IN_BOUNDS(p < (uint32_t)kb_tile<K>(), 704, p)) continue;
             sm.tile[p] = key[u];
             if (BINARR) sbin[p] = (uint16_t)(br[u] >> 16);
         }
@@ -156,7 +159,7 @@ __device__ __forceinline__ void scatter_tail(ScatterSmem<K> &sm, uint32_t *cnt, 
     for (uint32_t i = threadIdx.x; i < ntot; i += KB_NT) {
         const typename K::T k = sm.tile[i];
         const uint32_t b = BINARR ? sbin[i] : binof(k);
-        out[gb[b] + i] = k;
+        if (SG_IN_BOUNDS(b < (uint32_t)nb && (int64_t)(gb[b] + i) < cap, 705, gb[b] + i)) out[gb[b] + i] = k;
     }
 }
 
@@ -210,7 +213,8 @@ __global__ void __launch_bounds__(KB_NT) kb_hist2_kernel(KbPlan pl, const typena
         for (int u = 0; u < U; u++) k[u] = i + u * KB_NT < a1 ? K::load(in + i + u * KB_NT) : K::none();
 #pragma unroll
         for (int u = 0; u < U; u++)
-            if (i + u * KB_NT < a1) atomicAdd(cnt + (uint32_t)(K::code(k[u], lowbits) >> sh), 1u);
+            if (i + u * KB_NT < a1 && SG_IN_BOUNDS((K::code(k[u], lowbits) >> sh) < (uint64_t)(1 << b), 706, i))
+                atomicAdd(cnt + (uint32_t)(K::code(k[u], lowbits) >> sh), 1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < (1 << b); i += KB_NT)
@@ -254,10 +258,10 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter2_kernel(KbPlan pl, const 
         br[u] = 0xFFFFFFFFu;
         if (i < a1) {
             const uint32_t s = K::slot(key[u], 0ull, lowbits, sh);
-            br[u] = (s << 16) | atomicAdd(cnt + s, 1u);
+            if (SG_IN_BOUNDS(s < (uint32_t)nb, 707, s)) br[u] = (s << 16) | atomicAdd(cnt + s, 1u);
         }
     }
-    scatter_tail<K, false>(*sm, cnt, gb, nullptr, nb, key, br, pl.cur2 + pl.sb[p], out,
+    scatter_tail<K, false>(*sm, cnt, gb, nullptr, nb, key, br, pl.cur2 + pl.sb[p], out, pl.cap,
                            [&](const typename K::T &k) { return K::slot(k, 0ull, lowbits, sh); });
 }
 

@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter1_kernel(WindowSrc w, KbPl
                          lowbits);
         br[u] = (b << 16) | atomicAdd(cnt + b, 1u);
     }
-    scatter_tail<K, true>(*sm, cnt, gb, sbin, nb, key, br, pl.cur1, out,
+    scatter_tail<K, true>(*sm, cnt, gb, sbin, nb, key, br, pl.cur1, out, pl.cap,
                           [](const typename K::T &) { return 0u; });
 }
 
@@ -423,7 +423,8 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
         uint32_t r = 0;
         if (u * KB_NT + tid < n) {
             const uint32_t s = slot_of(key[u]), h = (s & 1u) * 16u;
-            r = (atomicAdd(sm.slots + slot_pad((int)(s >> 1)), 1u << h) >> h) & 0xffffu;
+            if (SG_IN_BOUNDS(s < (1u << ls), 708, s))
+                r = (atomicAdd(sm.slots + slot_pad((int)(s >> 1)), 1u << h) >> h) & 0xffffu;
         }
         if (u & 1) rk[u / 2] |= r << 16; else rk[u / 2] = r;
     }
@@ -463,6 +464,7 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
             int d = o;
             for (int j = o; j < e; j++) d += K::less(sm.sk[j], k) ? 1 : 0;
             const uint64_t low = K::low(k, lowbits);
+            if (!SG_IN_BOUNDS(base + d < a.pl.cap, 709, base + d)) continue;
             a.col[base + d] = (int32_t)(K::code(k, lowbits) & cmask);
             a.val[base + d] = (uint32_t)((low >> 1) & pmask) | (uint32_t)((low & 1u) << 31);
         }
@@ -547,7 +549,7 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
             const uint32_t d = (dst[u / 2] >> (16 * (u & 1))) & 0xffffu;
             if (d == 0xffffu) continue;
             const uint32_t o = sm.wpre[d >> 5] + __popc(sm.bits[d >> 5] & ((1u << (d & 31u)) - 1u));
-            out[base + o] = sm.sk[u * KB_NT + tid];
+            if (SG_IN_BOUNDS(base + o < a.pl.cap, 710, base + o)) out[base + o] = sm.sk[u * KB_NT + tid];
         }
         __syncthreads();
         return kept;
@@ -690,6 +692,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const
     for (int64_t b = blockIdx.x; b < nsub; b += gridDim.x) {
         const int64_t s0 = start[b], n = start[b + 1] - s0;
         const int p = pl.prefix(b);
+        if (!SG_IN_BOUNDS(n >= 0 && s0 + n <= pl.cap && p < pl.nb1, 711, b)) continue;
         const int bits = pl.rem - (pl.two ? pl.b2[p] : 0);  // code bits below the bucket's
         const uint64_t c0 = pl.two && bits < 64 ? (uint64_t)(b - pl.sb[p]) << bits : 0ull;
         uint32_t kept = 0, segs = 0;
@@ -874,7 +877,7 @@ __global__ void __launch_bounds__(KB_NT, 2) at_scatter_kernel(const int64_t *__r
         key[u] = K::make(((uint64_t)((uint32_t)rd[u] & rmask) << cbits) | col, low, lowbits);
         br[u] = (b << 16) | atomicAdd(cnt + b, 1u);
     }
-    scatter_tail<K, true>(*sm, cnt, gb, sbin, nb, key, br, pl.cur1, out,
+    scatter_tail<K, true>(*sm, cnt, gb, sbin, nb, key, br, pl.cur1, out, pl.cap,
                           [](const typename K::T &) { return 0u; });
 }
 
@@ -891,6 +894,7 @@ static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t record
     pl.nb1 = 1 << pb1;
     pl.rem = cb - pb1;
     pl.two = two ? 1 : 0;
+    pl.cap = records;
     // a prefix of c records splits into fewer than 2 c / target + 1 buckets (2^b2min at least)
     pl.nsub_max = two ? ((int64_t)pl.nb1 << b2min) + 2 * (records / target + 1) : pl.nb1;
     const size_t nb = (size_t)pl.nb1, ns = two ? (size_t)pl.nsub_max : 0;
