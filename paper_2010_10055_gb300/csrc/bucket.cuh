@@ -266,10 +266,10 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter2_kernel(KbPlan pl, const 
 }
 
 // ----------------------------------------------------------------------------- finishing
-// Slot counters of 16 bits, two per word; one pad word after every 16 so that a thread scanning 16
-// consecutive words does not meet its neighbours' banks.
-__device__ __forceinline__ int slot_pad(int w) { return w + (w >> 4); }
-constexpr int KB_SLOT_WORDS = (1 << (KB_NS - 1)) + (1 << (KB_NS - 5)) + 8;
+// Slot counters of 16 bits, two per word; four pad words after every 16, so that threads scanning
+// 16 consecutive words with 16-byte loads hit distinct banks.
+__device__ __forceinline__ int slot_pad(int w) { return w + (w >> 4) * 4; }
+constexpr int KB_SLOT_WORDS = (1 << (KB_NS - 1)) + (1 << (KB_NS - 3)) + 8;
 
 constexpr int KB_STACK = 8;    // nested refinements of an oversized bucket (13 code bits each)
 constexpr int KB_GROUPS = 64;  // slot ranges taken from one count of an oversized bucket
@@ -279,6 +279,8 @@ struct FinishSmem {
     typename K::T sk[KB_NT * K::ITEMS];   // records by slot
     uint32_t slots[KB_SLOT_WORDS];
     uint32_t bits[KB_NT * K::ITEMS / 32], wpre[KB_NT * K::ITEMS / 32 + 1];
+    uint32_t heads[KB_NT * K::ITEMS / 32 + 2];   // bit i + 32: record i of sk starts a slot
+    uint32_t codes[KB_NT * K::ITEMS / 32 + 2];   // ... (in order) a code
     uint32_t tmp[KB_NT / 32 + 1];
     uint32_t nseg, nst;
     uint64_t f_base[KB_STACK];  // refinement frames: codes with code >> f_bits == f_base, from slot f_a

@@ -399,7 +399,7 @@ struct FinishArgs {
 // block, where its records do.
 template <class K, bool COUNT>
 __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const FinishArgs &a, int p,
-                                                 const typename K::T (&key)[K::ITEMS], int n, uint64_t c0,
+                                                 typename K::T (&key)[K::ITEMS], int n, uint64_t c0,
                                                  uint64_t cend, int sh, int ls, int64_t base,
                                                  typename K::T *__restrict__ out) {
     using T = typename K::T;
@@ -408,12 +408,16 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
     const uint64_t sbase = K::slot_base(c0, lowbits);
     auto slot_of = [&](const T &k) { return K::slot(k, sbase, lowbits, sh); };
     // records of a slot that are kept for the ranking: not a lone one (a singleton, where lo >= 2);
-    // where a slot is one code, none of a code outside every range
+    // where a slot is one code, none of a code outside every range. Both counts of a word at once:
+    // bit 15 of c + (0x8000 - least) says c >= least, of c + (0x7fff - most) that c > most
     const bool exact = COUNT && sh == 0;
-    const uint32_t least = exact ? a.lo : (a.lo >= 2 ? 2u : 0u), span = exact ? a.hmax - least : 0xffffffffu - least;
-    auto eff = [&](uint32_t c) { return COUNT && c - least > span ? 0u : c; };
+    const uint32_t least = exact ? (a.lo < 0x7fffu ? a.lo : 0x7fffu) : (a.lo >= 2 ? 2u : 0u);
+    const uint32_t most = exact && a.hmax < 0x7fffu ? a.hmax : 0x7fffu;
+    const uint32_t ge = (0x8000u - least) * 0x10001u, gt = (0x7fffu - most) * 0x10001u;
+    auto mask = [&](uint32_t v) { return ((((v + ge) & ~(v + gt)) & 0x80008000u) >> 15) * 0xffffu; };
+    auto eff = [&](uint32_t v) { return COUNT ? v & mask(v) : v; };
     for (int w = tid; w <= slot_pad(W) / 4; w += KB_NT) reinterpret_cast<uint4 *>(sm.slots)[w] = make_uint4(0, 0, 0, 0);
-    if (COUNT && tid < K::ITEMS * KB_NT / 32) sm.bits[tid] = 0;
+    if (tid < K::ITEMS * KB_NT / 32 + 2) sm.heads[tid] = 0;
     if (tid == 0) sm.nseg = 0;
     __syncthreads();
     uint32_t rk[(K::ITEMS + 1) / 2];
@@ -429,19 +433,41 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
         if (u & 1) rk[u / 2] |= r << 16; else rk[u / 2] = r;
     }
     __syncthreads();
-    const int pw = (W + KB_NT - 1) / KB_NT, w0 = tid * pw, w1 = w0 + pw < W ? w0 + pw : W;
-    uint32_t sum = 0;
-    for (int w = w0; w < w1; w++) {
-        const uint32_t v = sm.slots[slot_pad(w)];
-        sum += eff(v & 0xffffu) + eff(v >> 16);
-    }
+    // slot counts -> first record of each slot, 1 to 16 words per thread
+    const int pw = (W + KB_NT - 1) / KB_NT;
     uint32_t tot;
-    uint32_t ex = block_exclusive_scan<KB_NT>(sum, sm.tmp, &tot);
-    for (int w = w0; w < w1; w++) {
-        const uint32_t v = sm.slots[slot_pad(w)];
-        const uint32_t o1 = ex + eff(v & 0xffffu);
-        sm.slots[slot_pad(w)] = ex | (o1 << 16);
-        ex = o1 + eff(v >> 16);
+    auto step = [&](uint32_t c, uint32_t &ex) {  // a dropped (or empty) slot starts at 0xffff
+        const uint32_t m = COUNT ? mask(c) : 0xffffffffu, v = c & m, o0 = ex, o1 = ex + (v & 0xffffu);
+        ex = o1 + (v >> 16);
+        return (o0 | (o1 << 16)) | ~m;
+    };
+    if (pw < 4) {
+        const int w0 = tid * pw, w1 = w0 + pw < W ? w0 + pw : W;
+        uint32_t sum = 0;
+        for (int w = w0; w < w1; w++) sum = __dp2a_lo(eff(sm.slots[slot_pad(w)]), 0x0101u, sum);
+        uint32_t ex = block_exclusive_scan<KB_NT>(sum, sm.tmp, &tot);
+        for (int w = w0; w < w1; w++) {
+            sm.slots[slot_pad(w)] = step(sm.slots[slot_pad(w)], ex);
+        }
+    } else {  // W = pw * KB_NT, pw a power of two: whole groups of 4 words
+        uint4 *mine = reinterpret_cast<uint4 *>(sm.slots + slot_pad(tid * pw));
+        uint32_t sum = 0;
+        for (int x = 0; x < pw / 4; x++) {
+            const uint4 v = mine[x];
+            sum = __dp2a_lo(eff(v.x), 0x0101u, sum);
+            sum = __dp2a_lo(eff(v.y), 0x0101u, sum);
+            sum = __dp2a_lo(eff(v.z), 0x0101u, sum);
+            sum = __dp2a_lo(eff(v.w), 0x0101u, sum);
+        }
+        uint32_t ex = block_exclusive_scan<KB_NT>(sum, sm.tmp, &tot);
+        for (int x = 0; x < pw / 4; x++) {
+            uint4 v = mine[x];
+            v.x = step(v.x, ex);
+            v.y = step(v.y, ex);
+            v.z = step(v.z, ex);
+            v.w = step(v.w, ex);
+            mine[x] = v;
+        }
     }
     if (tid == 0) sm.slots[slot_pad(W)] = tot;
     __syncthreads();
@@ -450,23 +476,49 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
     for (int u = 0; u < K::ITEMS; u++) {
         if (u * KB_NT >= n) break;
         if (u * KB_NT + tid >= n) continue;
-        const uint32_t s = slot_of(key[u]), o = off(s);
-        if (!COUNT || off(s + 1) != o) sm.sk[o + ((rk[u / 2] >> (16 * (u & 1))) & 0xffffu)] = key[u];
+        const uint32_t o = off(slot_of(key[u])), r = (rk[u / 2] >> (16 * (u & 1))) & 0xffffu;
+        if (COUNT && o == 0xffffu) continue;
+        if (SG_IN_BOUNDS(o + r < (uint32_t)kb_tile<K>(), 712, o + r)) sm.sk[o + r] = key[u];
+        if (r == 0) atomicOr(sm.heads + 1 + (o >> 5), 1u << (o & 31u));
     }
-    __syncthreads();
     const int ne = (int)tot;
+    if (tid == 0) atomicOr(sm.heads + 1 + (ne >> 5), 1u << (ne & 31));
+    __syncthreads();
+    // record i lies in a run of records [o, e): from the run starts of its word (the same for the
+    // whole warp) and, where the run reaches past it, of its neighbours
+    auto run_of = [&](const uint32_t *starts, int i, int &o, int &e) {
+        const int w = i >> 5, l = i & 31;
+        const uint32_t m = starts[1 + w];
+        uint32_t below = m & ((2u << l) - 1u), above = l == 31 ? 0u : m & ~((2u << l) - 1u);
+        int wb = w, wa = w;
+        while (below == 0) below = starts[1 + --wb];  // record 0 starts a run
+        while (above == 0) above = starts[1 + ++wa];  // and so, in effect, does record ne
+        o = 32 * wb + 31 - __clz(below);
+        e = 32 * wa + __ffs(above) - 1;
+    };
+    // a record's place is its slot's start plus the smaller records of the slot
+    auto place = [&](int i, const T &k) {
+        int o, e;
+        run_of(sm.heads, i, o, e);
+        uint32_t d = (uint32_t)o;
+        for (int j = o; j < e; j += 4) {  // independent loads, the first repeated past e
+            T x[4];
+#pragma unroll
+            for (int v = 0; v < 4; v++) x[v] = sm.sk[j + v < e ? j + v : j];
+#pragma unroll
+            for (int v = 0; v < 4; v++) d += j + v < e && K::less(x[v], k) ? 1u : 0u;
+        }
+        return d;
+    };
     if constexpr (!COUNT) {
         const uint64_t cmask = (1ull << a.cbits) - 1, pmask = (1ull << a.kb.pbits) - 1;
         for (int i = tid; i < ne; i += KB_NT) {
             const T k = sm.sk[i];
-            const uint32_t s = slot_of(k);
-            const int o = (int)off(s), e = (int)off(s + 1);
-            int d = o;
-            for (int j = o; j < e; j++) d += K::less(sm.sk[j], k) ? 1 : 0;
+            const int64_t d = base + place(i, k);
             const uint64_t low = K::low(k, lowbits);
-            if (!SG_IN_BOUNDS(base + d < a.pl.cap, 709, base + d)) continue;
-            a.col[base + d] = (int32_t)(K::code(k, lowbits) & cmask);
-            a.val[base + d] = (uint32_t)((low >> 1) & pmask) | (uint32_t)((low & 1u) << 31);
+            if (!SG_IN_BOUNDS(d < a.pl.cap, 709, d)) continue;
+            a.col[d] = (int32_t)(K::code(k, lowbits) & cmask);
+            a.val[d] = (uint32_t)((low >> 1) & pmask) | (uint32_t)((low & 1u) << 31);
         }
         // rows that start in [c0, cend): sh <= cbits and c0 is a multiple of 2^sh, so a
         // row starts where a slot does
@@ -479,77 +531,87 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
         __syncthreads();
         return (uint32_t)ne;
     } else {
-        const uint64_t code_mask = K::code_mask(lowbits), read_mask = K::read_mask(a.kb.pbits);
-        uint32_t dst[(K::ITEMS + 1) / 2];
-        uint32_t heads = 0;
+        uint32_t(&dst)[(K::ITEMS + 1) / 2] = rk;
 #pragma unroll
         for (int u = 0; u < K::ITEMS; u++) {
-            const int i = u * KB_NT + tid;
-            uint32_t mine = 0xffffu;
             if (u * KB_NT >= ne) break;
+            const int i = u * KB_NT + tid;
+            uint32_t d = 0;
             if (i < ne) {
-                const T k = sm.sk[i];
-                const uint32_t s = slot_of(k);
-                const int o = (int)off(s), e = (int)off(s + 1);
-                int less = 0;
-                uint32_t f = 0;
-                bool first = true, dup = false;  // no smaller record of this code; one of this read
-                if (exact) {  // one code: its frequency is the slot's count
-                    f = (uint32_t)(e - o);
-                    for (int j = o; j < e; j++) {
-                        const T x = sm.sk[j];
-                        if (K::less(x, k)) {
-                            less++;
-                            dup |= K::same(x, k, read_mask);
-                        }
-                    }
-                    first = less == 0;
-                } else {
-                    for (int j = o; j < e; j++) {
-                        const T x = sm.sk[j];
-                        const bool lt = K::less(x, k);
-                        less += lt ? 1 : 0;
-                        if (K::same(x, k, code_mask)) {
-                            if (++f > a.hmax) break;  // above every range
-                            if (lt) {
-                                first = false;
-                                dup |= K::same(x, k, read_mask);
-                            }
-                        }
-                    }
-                }
+                key[u] = sm.sk[i];
+                d = place(i, key[u]);
+            }
+            if (u & 1) dst[u / 2] |= d << 16; else dst[u / 2] = d;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < K::ITEMS; u++) {
+            if (u * KB_NT >= ne) break;
+            if (u * KB_NT + tid < ne) sm.sk[(dst[u / 2] >> (16 * (u & 1))) & 0xffffu] = key[u];
+        }
+        __syncthreads();
+        // codes are runs now; of a read's records of a code, the first is its lowest position
+        const uint64_t code_mask = K::code_mask(lowbits), read_mask = K::read_mask(a.kb.pbits);
+        uint32_t again = 0, starts = 0;  // bit u: this thread's record repeats its predecessor's read; starts a code
+#pragma unroll
+        for (int u = 0; u < K::ITEMS; u++) {
+            if (u * KB_NT >= ne) break;
+            const int i = u * KB_NT + tid;
+            bool st = i == ne;  // the end counts as a start
+            if (i < ne) {
+                const T k = sm.sk[i], x = sm.sk[i > 0 ? i - 1 : 0];
+                st = i == 0 || !K::same(x, k, code_mask);
+                if (!st && K::same(x, k, read_mask)) again |= 1u << u;
+                if (st) starts |= 1u << u;
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, st);
+            if ((tid & 31) == 0 && (i <= ne)) sm.codes[1 + (i >> 5)] = m;
+        }
+        if (tid == 0 && ne % KB_NT == 0) sm.codes[1 + (ne >> 5)] = 1u;
+        __syncthreads();
+        uint32_t nst = 0;
+        uint32_t keep = 0;
+#pragma unroll
+        for (int u = 0; u < K::ITEMS; u++) {
+            if (u * KB_NT >= ne) break;
+            const int i = u * KB_NT + tid;
+            bool kp = false;
+            if (i < ne) {
+                int o, e;
+                run_of(sm.codes, i, o, e);
                 uint32_t lo = a.lo, hi = a.hi;
                 if (a.lohi) {
-                    const uint64_t job = (((uint64_t)p << a.pl.rem) | K::code(k, lowbits)) >> a.kbits;
+                    const uint64_t job = (((uint64_t)p << a.pl.rem) | K::code(sm.sk[i], lowbits)) >> a.kbits;
                     lo = a.lohi[2 * job];
                     hi = a.lohi[2 * job + 1];
                 }
+                const uint32_t f = (uint32_t)(e - o);
                 const bool rel = f >= lo && f <= hi;
-                heads += rel && first ? 1u : 0u;
-                if (rel && !dup) {
-                    mine = (uint32_t)(o + less);
-                    atomicOr(sm.bits + (mine >> 5), 1u << (mine & 31u));
-                }
+                nst += rel && ((starts >> u) & 1u) ? 1u : 0u;
+                kp = rel && !((again >> u) & 1u);
+                keep |= kp ? 1u << u : 0u;
             }
-            if (u & 1) dst[u / 2] |= mine << 16; else dst[u / 2] = mine;
+            const uint32_t m = __ballot_sync(0xffffffffu, kp);
+            if ((tid & 31) == 0 && i < ne) sm.bits[i >> 5] = m;
         }
-        heads = __reduce_add_sync(0xffffffffu, heads);
-        if ((tid & 31) == 0 && heads) atomicAdd(&sm.nseg, heads);
+        nst = __reduce_add_sync(0xffffffffu, nst);
+        if ((tid & 31) == 0 && nst) atomicAdd(&sm.nseg, nst);
         __syncthreads();
         uint32_t kept;
         {
-            const uint32_t c = tid < K::ITEMS * KB_NT / 32 ? __popc(sm.bits[tid]) : 0u;
+            const int nw = (ne + 31) / 32;  // at most one word per thread
+            const uint32_t c = tid < nw ? __popc(sm.bits[tid]) : 0u;
             const uint32_t x = block_exclusive_scan<KB_NT>(c, sm.tmp, &kept);
-            if (tid < K::ITEMS * KB_NT / 32) sm.wpre[tid] = x;
+            if (tid < nw) sm.wpre[tid] = x;
         }
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < K::ITEMS; u++) {
             if (u * KB_NT >= ne) break;
-            const uint32_t d = (dst[u / 2] >> (16 * (u & 1))) & 0xffffu;
-            if (d == 0xffffu) continue;
-            const uint32_t o = sm.wpre[d >> 5] + __popc(sm.bits[d >> 5] & ((1u << (d & 31u)) - 1u));
-            if (SG_IN_BOUNDS(base + o < a.pl.cap, 710, base + o)) out[base + o] = sm.sk[u * KB_NT + tid];
+            if (!((keep >> u) & 1u)) continue;
+            const int i = u * KB_NT + tid;
+            const uint32_t o = sm.wpre[i >> 5] + __popc(sm.bits[i >> 5] & ((1u << (i & 31)) - 1u));
+            if (SG_IN_BOUNDS(base + o < a.pl.cap, 710, base + o)) out[base + o] = sm.sk[i];
         }
         __syncthreads();
         return kept;
