@@ -1,7 +1,7 @@
 // tr.cu -- transitive reduction of the bidirected overlap graph R (Algorithm 1, Sec. IV-E) with
 // the MinPlus semiring of Algorithm 3, on the GPU.
 //
-// One round, for every row i in one thread block:
+// One round, for every row i:
 //   N_ik = min over j of R_ij + R_jk, over walks i->j->k that are valid (the two heads at j
 //          point opposite ways: in(d_ij) == out(d_jk), Sec. II) -- only for k with R_ik present,
 //          since Algorithm 1 compares M and N only where both exist;
@@ -14,16 +14,17 @@
 //
 // Direction encoding: d = 2 * o_first + o_second (o = 1: the read is traversed reverse-
 // complemented). in(d) = d & 1, out(d) = d >> 1; the walk's composite dir is
-// 2 * out(d_ij) + in(d_jk). N is kept as (sum << 2 | composite) in one 64-bit word so that
-// DIRMATCH (composite must equal d_ik before the min) and LITERAL (lexicographic min of
-// (sum, composite), checked after) share one atomicMin.
+// 2 * out(d_ij) + in(d_jk). Where N is needed it is kept as (sum << 2 | composite) in one 64-bit
+// word, so that DIRMATCH (composite must equal d_ik before the min) and LITERAL (lexicographic min
+// of (sum, composite), checked after) share one atomicMin; a DIRMATCH reduction needs only to know
+// whether some walk is short enough.
+#include <algorithm>
+
 #include "check.cuh"
 #include "ops.cuh"
 
 namespace sg {
 
-constexpr int TR_NT = 128;
-constexpr int TR_SMEM_ROW = 1024;  // rows up to this degree stage their entries in shared memory
 constexpr unsigned long long TR_NONE = ~0ull;
 
 struct TrGraph {
@@ -34,7 +35,65 @@ struct TrGraph {
     int64_t n;
 };
 
-__global__ void validate_graph_kernel(TrGraph g, int64_t nnz, uint32_t *__restrict__ err) {
+// An entry as one 64-bit word: column << 32 | suffix << 2 | dir (suffix < 2^30, dir <= 3), so that a
+// product costs one load.
+__device__ __forceinline__ uint64_t tr_pack(int32_t col, uint32_t suf, uint32_t dir) {
+    return ((uint64_t)(uint32_t)col << 32) | (suf << 2) | dir;
+}
+
+// The graph the rounds work on: packed entries in row order (e; nullptr: the caller's arrays, in
+// `in`), and each row's entries with those of out(d) = 0 first (p): a walk i -> j -> k continues only
+// with the entries of j whose out(d) is in(d_ij), so a neighbour's other half is never read.
+// row[i] = {first entry, low word; its high word; entries with out 0; entries with out 1}.
+struct TrPacked {
+    const uint64_t *e, *p;
+    const uint4 *row;
+    int64_t n;
+    TrGraph in;
+};
+struct TrBuf {
+    uint64_t *e = nullptr, *p = nullptr;
+    uint4 *row = nullptr;
+};
+
+__device__ __forceinline__ uint64_t tr_entry(const TrPacked &g, int64_t x) {
+    return g.e ? g.e[x] : tr_pack(g.in.col[x], g.in.suf[x], g.in.dir[x]);
+}
+
+__device__ __forceinline__ int64_t tr_first(const uint4 &r) { return (int64_t)(((uint64_t)r.y << 32) | r.x); }
+
+// One warp writes a row of the packed graph: its entries from `first` on, given in order through
+// next(t) (t < deg, every lane), kept where keep(t).
+template <class Next, class Keep>
+__device__ __forceinline__ void tr_write_row(const TrBuf &o, int64_t row, int64_t first, int64_t deg, Next &&next,
+                                             Keep &&keep) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    uint32_t n0 = 0, n1 = 0;
+    for (int64_t b = 0; b < deg; b += 32) {
+        const bool have = b + lane < deg && keep(b + lane);
+        const uint64_t x = have ? next(b + lane) : 0ull;
+        n0 += __popc(__ballot_sync(0xffffffffu, have && !(x & 2u)));
+        n1 += __popc(__ballot_sync(0xffffffffu, have && (x & 2u)));
+    }
+    int64_t w = first, w0 = first, w1 = first + n0;
+    for (int64_t b = 0; b < deg; b += 32) {
+        const bool have = b + lane < deg && keep(b + lane);
+        const uint64_t x = have ? next(b + lane) : 0ull;
+        const uint32_t m0 = __ballot_sync(0xffffffffu, have && !(x & 2u)), m1 = __ballot_sync(0xffffffffu, have && (x & 2u));
+        if (have) {
+            if (o.e) o.e[w + __popc((m0 | m1) & lt)] = x;
+            o.p[(x & 2u) ? w1 + __popc(m1 & lt) : w0 + __popc(m0 & lt)] = x;
+        }
+        w += __popc(m0 | m1);
+        w0 += __popc(m0);
+        w1 += __popc(m1);
+    }
+    if (lane == 0) o.row[row] = make_uint4((uint32_t)first, (uint32_t)((uint64_t)first >> 32), n0, n1);
+}
+
+// Checks the CSR contract and packs the graph: one warp per row.
+__global__ void validate_graph_kernel(TrGraph g, int64_t nnz, TrBuf o, uint32_t *__restrict__ err) {
     int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (row > g.n) return;
@@ -49,268 +108,417 @@ __global__ void validate_graph_kernel(TrGraph g, int64_t nnz, uint32_t *__restri
     }
     bool bad = false;
     for (int64_t e = r0 + lane; e < r1; e += 32) {
-        int32_t c = g.col[e];
+        const int32_t c = g.col[e];
         if (c < 0 || c >= g.n || c == row) bad = true;
         if (e > r0 && g.col[e - 1] >= c) bad = true;
         if (g.suf[e] >= (1u << 30) || g.dir[e] > 3) bad = true;
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(err, (uint32_t)DEV_INVALID);
+    tr_write_row(o, row, r0, r1 - r0, [&](int64_t t) { return tr_pack(g.col[r0 + t], g.suf[r0 + t], g.dir[r0 + t] & 3u); },
+                 [](int64_t) { return true; });
 }
 
-// index of k in the sorted cols[0..deg), or -1
-__device__ __forceinline__ int64_t find_col(const int32_t *cols, int64_t deg, int32_t k) {
-    int64_t lo = 0, hi = deg;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (cols[mid] < k) lo = mid + 1; else hi = mid;
+// ------------------------------------------------------------------------------- one round
+// Row i's columns go into a hash table in shared memory; every entry (j, k) of the fitting half of
+// every neighbour j's row is then one 8-byte load, a length check and a probe of the table.
+//   MIN == false (reduction, DIRMATCH): entry (i, k) is transitive iff some valid walk i -> j -> k
+//     with d_ik's end orientations has length <= the bound of its end: a flag, no minimum.
+//   MIN == true (LITERAL, or N itself is wanted): the minimum of (length << 2 | orientations).
+// Rows of up to TR_WROW entries take one warp each (its table is its own: no block barrier); four
+// neighbours are walked at once, 8 lanes each, since half a row is a few tens of entries. Longer
+// rows are listed and take a block; above TR_BROW entries the row is searched in place instead of
+// hashed.
+// The table is buckets of two columns, four to eight buckets per entry, so that one 8-byte load
+// settles all but a few percent of the probes: at two slots per entry the longest of a warp's 32
+// probe chains took 9 of 13 ms on 22 M edges.
+constexpr int TR_NT = 128;
+constexpr int TR_WROW = 128;   // entries of a warp's row
+constexpr int TR_BNT = 256;
+constexpr int TR_BROW = 2048;  // entries of a block's hashed row
+constexpr uint32_t TR_FREE = 0xFFFFFFFFu;
+
+struct TrArgs {
+    TrPacked g;
+    const uint32_t *err;
+    int mode;
+    uint32_t fuzz;
+    unsigned long long *gbest;     // per-entry minima of rows above TR_BROW (MIN)
+    uint8_t *keep;
+    int64_t *kept;
+    uint32_t *outN;
+    uint8_t *outD;
+    int32_t *big;                  // rows for blocks, and their number (nullptr: blocks look for them)
+    unsigned long long *n_big;
+    int warp_rows;                 // 0: every row takes a block
+};
+
+// The bounds of a row's entries by read end (out(d)): the row maximum, whole or per end, plus fuzz.
+__device__ __forceinline__ void tr_bounds(const TrArgs &a, uint32_t m0, uint32_t m1, uint32_t &v0, uint32_t &v1) {
+    const uint32_t m = m0 > m1 ? m0 : m1;
+    const bool per_end = (a.mode & SG_TR_PER_END) != 0;
+    v0 = (per_end ? m0 : m) + a.fuzz;  // both below 2^30
+    v1 = (per_end ? m1 : m) + a.fuzz;
+}
+
+// Columns -> entries of one row: buckets of two keys (2^lb of them); val = entry << 2 | dir.
+struct TrTable {
+    uint32_t *key;
+    uint16_t *val;
+    int lb;
+    __device__ __forceinline__ uint32_t bucket(uint32_t k) const { return (k * 2654435761u) >> (32 - lb); }
+    __device__ __forceinline__ void insert(uint32_t k, uint32_t v) const {
+        uint32_t h = 2u * bucket(k);
+        const uint32_t msk = (2u << lb) - 1u;
+        while (atomicCAS(key + h, TR_FREE, k) != TR_FREE) h = (h + 1) & msk;  // far from full
+        val[h] = (uint16_t)v;
     }
-    return (lo < deg && cols[lo] == k) ? lo : -1;
+    __device__ __forceinline__ uint2 load(uint32_t h) const { return *reinterpret_cast<const uint2 *>(key + 2 * h); }
+    // slot of k from its bucket's keys, or -1
+    __device__ __forceinline__ int find(uint32_t k, uint32_t h, uint2 x) const {
+        for (;;) {
+            if (x.x == k) return (int)(2 * h);
+            if (x.y == k) return (int)(2 * h + 1);
+            if (x.y == TR_FREE) return -1;  // filled in order
+            h = (h + 1) & ((1u << lb) - 1u);
+            x = load(h);
+        }
+    }
+};
+
+// Entries of four consecutive steps of a neighbour's half row, taken together so that their loads
+// and their probes travel together. len(x) sums, ok(x) whether a walk of that length matters,
+// hit(slot, walk orientations, length).
+template <class Ok, class Hit>
+__device__ __forceinline__ void tr_four(const TrTable &tb, uint32_t lij, const uint64_t *__restrict__ row, uint32_t b,
+                                        uint32_t cnt, Ok &&ok, Hit &&hit) {
+    uint64_t x[4];
+    uint2 kk[4];
+    uint32_t len[4];
+    bool go[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) x[u] = b + 8 * u < cnt ? row[b + 8 * u] : 0ull;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        len[u] = (lij >> 2) + ((uint32_t)x[u] >> 2);
+        go[u] = b + 8 * u < cnt && ok((lij & 2u) | ((uint32_t)x[u] & 1u), len[u]);
+        if (go[u]) kk[u] = tb.load(tb.bucket((uint32_t)(x[u] >> 32)));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        if (!go[u]) continue;
+        const uint32_t k = (uint32_t)(x[u] >> 32);
+        const int sl = tb.find(k, tb.bucket(k), kk[u]);
+        if (sl >= 0) hit(sl, (lij & 2u) | ((uint32_t)x[u] & 1u), len[u]);
+    }
 }
 
-// One block per row. GMEM: the row is read in place from global memory and the per-entry
-// minima live in `gbest` (indexed by entry); otherwise the row is staged in shared memory.
-template <bool GMEM>
-__global__ void __launch_bounds__(TR_NT) minplus_mark_kernel(TrGraph g, const int32_t *__restrict__ rows,
-                                                            const unsigned long long *__restrict__ nrows_p,
-                                                            const uint32_t *__restrict__ err, int mode, uint32_t fuzz,
-                                                            unsigned long long *__restrict__ gbest,
-                                                            int64_t *__restrict__ gpre,
-                                                            uint8_t *__restrict__ keep, int64_t *__restrict__ kept,
-                                                            uint32_t *__restrict__ outN, uint8_t *__restrict__ outD,
-                                                            int warp_rows) {
-    __shared__ int32_t s_col[GMEM ? 1 : TR_SMEM_ROW];
-    __shared__ uint32_t s_suf[GMEM ? 1 : TR_SMEM_ROW];
-    __shared__ uint8_t s_dir[GMEM ? 1 : TR_SMEM_ROW];
-    __shared__ unsigned long long s_best[GMEM ? 1 : TR_SMEM_ROW];
-    __shared__ int64_t s_pre[GMEM ? 1 : TR_SMEM_ROW + 1];
-    __shared__ int64_t s_tmp[TR_NT / 32 + 1];
-    __shared__ uint32_t s_red[2 * (TR_NT / 32)];
-    __shared__ int64_t s_kept[TR_NT / 32];
-    if (*err) return;  // the graph failed validation: touch nothing
-    const int64_t nrows = (int64_t)*nrows_p;
+// A warp's 32 neighbours (one per lane: entry, first entry and length of the fitting half row; 0
+// entries past the row's end), four at a time.
+template <class Ok, class Hit>
+__device__ __forceinline__ void tr_walk(const TrTable &tb, const uint64_t *__restrict__ P, uint64_t ent, int64_t jb,
+                                        uint32_t jn, int count, Ok &&ok, Hit &&hit) {
+    const int lane = threadIdx.x & 31, sub = lane >> 3, l8 = lane & 7;
+    for (int s4 = 0; s4 < count; s4 += 4) {
+        const int src = s4 + sub;  // the lane that holds this group's neighbour
+        const uint32_t lij = __shfl_sync(0xffffffffu, (uint32_t)ent, src);
+        const int64_t b0 = __shfl_sync(0xffffffffu, jb, src);
+        const uint32_t cnt = __shfl_sync(0xffffffffu, jn, src);
+        for (uint32_t b = l8; b < cnt; b += 32) tr_four(tb, lij, P + b0, b, cnt, ok, hit);
+        __syncwarp();
+    }
+}
+
+// The fitting half of the neighbour behind entry x.
+__device__ __forceinline__ void tr_half(const TrPacked &g, uint64_t x, int64_t &jb, uint32_t &jn) {
+    const uint4 r = __ldg(g.row + (x >> 32));
+    const bool in = x & 1u;
+    jb = tr_first(r) + (in ? r.z : 0u);
+    jn = in ? r.w : r.z;
+}
+
+// The outcome of entry t (packed ent): writes keep / N / Ndir; returns whether it is kept.
+template <bool MIN>
+__device__ __forceinline__ bool tr_outcome(const TrArgs &a, int64_t at, uint64_t ent, bool flag, unsigned long long best,
+                                           uint32_t v0, uint32_t v1) {
+    const uint32_t d = (uint32_t)ent & 3u;
+    bool transitive = flag;
+    if (MIN) {
+        const bool has = best != TR_NONE;
+        const uint64_t N = best >> 2;
+        transitive = has && (uint32_t)(best & 3u) == d && ((d >> 1) ? v1 : v0) >= N;
+        if (a.outN) a.outN[at] = has ? (uint32_t)N : 0xFFFFFFFFu;
+        if (a.outD) a.outD[at] = has ? (uint8_t)(best & 3u) : (uint8_t)d;
+    }
+    if (a.keep) a.keep[at] = transitive ? 0 : 1;
+    return !transitive;
+}
+
+__device__ __forceinline__ void tr_min(unsigned long long *best, uint32_t comp, uint32_t len) {
+    const unsigned long long w = ((unsigned long long)len << 2) | comp;
+    if (w < *(volatile unsigned long long *)best) atomicMin(best, w);
+}
+
+template <bool MIN>
+struct __align__(16) TrWarpSmem {
+    uint32_t key[8 * TR_WROW];  // cleared 16 bytes at a time
+    unsigned long long best[MIN ? TR_WROW : 1];
+    uint16_t val[8 * TR_WROW];
+    uint8_t flag[MIN ? 4 : TR_WROW];
+};
+static_assert(sizeof(TrWarpSmem<true>) % 16 == 0 && sizeof(TrWarpSmem<false>) % 16 == 0, "16-byte rows of key");
+
+template <bool MIN>
+__global__ void __launch_bounds__(TR_NT) tr_mark_kernel(TrArgs a) {
+    __shared__ TrWarpSmem<MIN> s_all[TR_NT / 32];
+    if (*a.err) {  // the graph failed validation: touch nothing of it (the caller's scan reads kept)
+        if (a.kept)
+            for (int64_t i = (int64_t)blockIdx.x * TR_NT + threadIdx.x; i < a.g.n; i += (int64_t)gridDim.x * TR_NT)
+                a.kept[i] = 0;
+        return;
+    }
+    constexpr int Q = TR_WROW / 32;
+    TrWarpSmem<MIN> &s = s_all[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * TR_NT) >> 5;
+    for (int64_t i = ((int64_t)blockIdx.x * TR_NT + threadIdx.x) >> 5; i < a.g.n; i += nw) {
+        const uint4 r = a.g.row[i];
+        const int64_t r0 = tr_first(r), degl = (int64_t)r.z + r.w;
+        if (degl == 0) {
+            if (lane == 0 && a.kept) a.kept[i] = 0;
+            continue;
+        }
+        if (degl > TR_WROW || (a.big && !a.warp_rows)) {
+            if (lane == 0 && a.big) {
+                const unsigned long long q = atomicAdd(a.n_big, 1ull);
+                if (SG_IN_BOUNDS((int64_t)q < a.g.n, 403, q)) a.big[q] = (int32_t)i;
+            }
+            continue;
+        }
+        const int deg = (int)degl;
+        TrTable tb{s.key, s.val, 4};
+        while ((1 << tb.lb) < 4 * deg && tb.lb < 9) tb.lb++;
+        for (int x = lane; x < (2 << tb.lb) / 4; x += 32)
+            reinterpret_cast<uint4 *>(s.key)[x] = make_uint4(TR_FREE, TR_FREE, TR_FREE, TR_FREE);
+        // the row, its neighbours' fitting halves, its maxima; the table
+        uint64_t ent[Q];
+        int64_t jb[Q];
+        uint32_t jn[Q], m0 = 0, m1 = 0;
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const int t = 32 * q + lane;
+            ent[q] = 0;
+            jb[q] = 0;
+            jn[q] = 0;
+            if (t < deg) {
+                ent[q] = tr_entry(a.g, r0 + t);
+                tr_half(a.g, ent[q], jb[q], jn[q]);
+                const uint32_t sv = (uint32_t)ent[q] >> 2;
+                if (ent[q] & 2u) m1 = sv > m1 ? sv : m1; else m0 = sv > m0 ? sv : m0;
+                if (MIN) s.best[MIN ? t : 0] = TR_NONE; else s.flag[MIN ? 0 : t] = 0;
+            }
+        }
+        m0 = __reduce_max_sync(0xffffffffu, m0);
+        m1 = __reduce_max_sync(0xffffffffu, m1);
+        uint32_t v0, v1;
+        tr_bounds(a, m0, m1, v0, v1);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const int t = 32 * q + lane;
+            if (t < deg) tb.insert((uint32_t)(ent[q] >> 32), (uint32_t)(t << 2) | ((uint32_t)ent[q] & 3u));
+        }
+        __syncwarp();
+        auto ok = [&](uint32_t comp, uint32_t len) { return MIN || len <= ((comp & 2u) ? v1 : v0); };
+        auto hit = [&](int sl, uint32_t comp, uint32_t len) {
+            const uint32_t v = s.val[sl];
+            if (MIN) {
+                if ((a.mode & 1) == SG_TR_DIRMATCH && comp != (v & 3u)) return;
+                tr_min(s.best + (MIN ? v >> 2 : 0u), comp, len);
+            } else if (comp == (v & 3u)) {
+                s.flag[MIN ? 0u : v >> 2] = 1;
+            }
+        };
+#pragma unroll
+        for (int q = 0; q < Q; q++)
+            if (32 * q < deg) tr_walk(tb, a.g.p, ent[q], jb[q], jn[q], deg - 32 * q < 32 ? deg - 32 * q : 32, ok, hit);
+        __syncwarp();
+        int mykept = 0;
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const int t = 32 * q + lane;
+            if (t < deg) mykept += tr_outcome<MIN>(a, r0 + t, ent[q], !MIN && s.flag[MIN ? 0 : t],
+                                                   MIN ? s.best[MIN ? t : 0] : TR_NONE, v0, v1) ? 1 : 0;
+        }
+        mykept = __reduce_add_sync(0xffffffffu, mykept);
+        if (lane == 0 && a.kept) a.kept[i] = mykept;
+        __syncwarp();  // the table is cleared next
+    }
+}
+
+// Listed rows, one block each: the row's neighbours in groups of 32, a warp per group.
+template <bool MIN>
+constexpr size_t tr_big_smem() {
+    return (size_t)TR_BROW * (MIN ? 8 : 0) + (size_t)4 * TR_BROW * 6 + (MIN ? 0 : TR_BROW);
+}
+template <bool MIN>
+__global__ void __launch_bounds__(TR_BNT) tr_mark_big_kernel(TrArgs a) {
+    extern __shared__ __align__(16) unsigned char tr_raw[];
+    unsigned long long *sbest = reinterpret_cast<unsigned long long *>(tr_raw);                     // (MIN)
+    uint32_t *key = reinterpret_cast<uint32_t *>(tr_raw + (size_t)TR_BROW * (MIN ? 8 : 0));         // [4 TR_BROW]
+    uint16_t *val = reinterpret_cast<uint16_t *>(key + 4 * TR_BROW);                                // entry
+    uint8_t *flag = reinterpret_cast<uint8_t *>(val + 4 * TR_BROW);                                 // (!MIN)
+    __shared__ uint32_t s_m[2];
+    __shared__ int s_kept;
+    if (*a.err) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto E = [&](int64_t t) { return tr_entry(a.g, t); };
+    const int64_t nrows = a.big ? (int64_t)*a.n_big : a.g.n;
     for (int64_t rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int32_t i = rows[rb];
-        if (!SG_IN_BOUNDS(i >= 0 && i < g.n, 404, i)) continue;
-        const int64_t r0 = g.rp[i], r1 = g.rp[i + 1], deg = r1 - r0;
-        const int32_t *col = GMEM ? g.col + r0 : s_col;
-        const uint32_t *suf = GMEM ? g.suf + r0 : s_suf;
-        const uint8_t *dir = GMEM ? g.dir + r0 : s_dir;
-        unsigned long long *best = GMEM ? gbest + r0 : s_best;
-        int64_t *pre = GMEM ? gpre + r0 + i : s_pre;  // deg + 1 slots per row
-        // stage row i and the exclusive prefix of its neighbours' degrees; the row max per read
-        // end of i (out(d)), folded into one for the whole-row form
-        uint32_t vmax0 = 0, vmax1 = 0;
-        int64_t run = 0;
-        for (int64_t base = 0; base < deg; base += TR_NT) {
-            int64_t a = base + threadIdx.x;
-            int64_t dj = 0;
-            if (a < deg) {
-                int32_t j = g.col[r0 + a];
-                uint32_t sv = g.suf[r0 + a];
-                const uint8_t da = g.dir[r0 + a];
-                if (!GMEM) {
-                    s_col[a] = j;
-                    s_suf[a] = sv;
-                    s_dir[a] = da;
-                }
-                best[a] = TR_NONE;
-                if (da >> 1) vmax1 = sv > vmax1 ? sv : vmax1;
-                else vmax0 = sv > vmax0 ? sv : vmax0;
-                dj = g.rp[j + 1] - g.rp[j];
+        const int32_t i = a.big ? a.big[rb] : (int32_t)rb;
+        if (!SG_IN_BOUNDS(i >= 0 && i < a.g.n, 404, i)) continue;
+        const uint4 r = a.g.row[i];
+        const int64_t r0 = tr_first(r), deg = (int64_t)r.z + r.w;
+        if (!a.big && deg <= TR_WROW) continue;  // a warp's
+        const bool hashed = deg <= TR_BROW;
+        unsigned long long *best = hashed ? sbest : a.gbest + r0;
+        TrTable tb{key, val, 4};
+        while (hashed && (1 << tb.lb) < 2 * deg) tb.lb++;
+        if (threadIdx.x < 2) s_m[threadIdx.x] = 0;
+        if (threadIdx.x == 0) s_kept = 0;
+        if (hashed)
+            for (int x = threadIdx.x; x < (2 << tb.lb); x += TR_BNT) key[x] = TR_FREE;
+        __syncthreads();
+        uint32_t m0 = 0, m1 = 0;
+        for (int64_t t = threadIdx.x; t < deg; t += TR_BNT) {
+            const uint64_t ent = E(r0 + t);
+            const uint32_t sv = (uint32_t)ent >> 2;
+            if (ent & 2u) m1 = sv > m1 ? sv : m1; else m0 = sv > m0 ? sv : m0;
+            if (MIN) best[t] = TR_NONE;
+            else if (hashed) flag[t] = 0;
+            else a.keep[r0 + t] = 1;
+            if (hashed) tb.insert((uint32_t)(ent >> 32), (uint32_t)((t << 2) | (ent & 3u)));
+        }
+        atomicMax(s_m, m0);
+        atomicMax(s_m + 1, m1);
+        __syncthreads();
+        uint32_t v0, v1;
+        tr_bounds(a, s_m[0], s_m[1], v0, v1);
+        auto ok = [&](uint32_t comp, uint32_t len) { return MIN || len <= ((comp & 2u) ? v1 : v0); };
+        auto hit_at = [&](int64_t t, uint32_t d, uint32_t comp, uint32_t len) {
+            if (MIN) {
+                if ((a.mode & 1) == SG_TR_DIRMATCH && comp != d) return;
+                tr_min(best + t, comp, len);
+            } else if (comp == d) {
+                if (hashed) flag[t] = 1; else a.keep[r0 + t] = 0;
             }
-            int64_t tot;
-            int64_t ex = block_exclusive_scan<TR_NT>(dj, s_tmp, &tot);
-            if (a < deg) pre[a] = run + ex;
-            run += tot;
-        }
-        if (threadIdx.x == 0) pre[deg] = run;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            uint32_t y = __shfl_xor_sync(0xffffffffu, vmax0, o);
-            vmax0 = y > vmax0 ? y : vmax0;
-            y = __shfl_xor_sync(0xffffffffu, vmax1, o);
-            vmax1 = y > vmax1 ? y : vmax1;
-        }
-        if ((threadIdx.x & 31) == 0) {
-            s_red[2 * (threadIdx.x >> 5)] = vmax0;
-            s_red[2 * (threadIdx.x >> 5) + 1] = vmax1;
+        };
+        auto hit = [&](int sl, uint32_t comp, uint32_t len) { hit_at(val[sl] >> 2, val[sl] & 3u, comp, len); };
+        for (int64_t c = (int64_t)warp * 32; c < deg; c += TR_BNT) {
+            const int64_t t = c + lane;
+            uint64_t ent = 0;
+            int64_t jb = 0;
+            uint32_t jn = 0;
+            if (t < deg) {
+                ent = E(r0 + t);
+                tr_half(a.g, ent, jb, jn);
+            }
+            const int count = deg - c < 32 ? (int)(deg - c) : 32;
+            if (hashed) {
+                tr_walk(tb, a.g.p, ent, jb, jn, count, ok, hit);
+                continue;
+            }
+            for (int q = 0; q < count; q++) {
+                const uint32_t lij = __shfl_sync(0xffffffffu, (uint32_t)ent, q);
+                const int64_t b0 = __shfl_sync(0xffffffffu, jb, q);
+                const uint32_t cnt = __shfl_sync(0xffffffffu, jn, q);
+                for (uint32_t b = lane; b < cnt; b += 32) {
+                    const uint64_t x = a.g.p[b0 + b];
+                    const uint32_t comp = (lij & 2u) | ((uint32_t)x & 1u), len = (lij >> 2) + ((uint32_t)x >> 2);
+                    if (!ok(comp, len)) continue;
+                    int64_t lo = 0, hi = deg;  // first entry with column >= k
+                    while (lo < hi) {
+                        const int64_t mid = (lo + hi) >> 1;
+                        if ((E(r0 + mid) >> 32) < (x >> 32)) lo = mid + 1; else hi = mid;
+                    }
+                    if (lo < deg && (E(r0 + lo) >> 32) == (x >> 32)) hit_at(lo, (uint32_t)E(r0 + lo) & 3u, comp, len);
+                }
+            }
         }
         __syncthreads();
-        const int64_t P = pre[deg];
-        // N = R^2 on the pattern of row i: a warp per neighbour j walking j's row (staged rows,
-        // warp_rows), or every thread on the flattened products, each finding its neighbour by a
-        // search of the degree prefix
-        if (!GMEM && warp_rows) {
-            const int lane = threadIdx.x & 31;
-            for (int64_t a = threadIdx.x >> 5; a < deg; a += TR_NT / 32) {
-                const int32_t j = col[a];
-                const int64_t jb = g.rp[j], je = g.rp[j + 1];
-                const uint32_t dij = dir[a], sa = suf[a];
-                for (int64_t b = jb + lane; b < je; b += 32) {
-                    const int32_t k = g.col[b];
-                    if (k == i) continue;
-                    const int64_t t = find_col(col, deg, k);
-                    if (t < 0) continue;
-                    const uint32_t djk = g.dir[b];
-                    if ((dij & 1u) != (djk >> 1)) continue;  // heads at j must point opposite ways
-                    const uint32_t comp = (dij & 2u) | (djk & 1u);
-                    if ((mode & 1) == SG_TR_DIRMATCH && comp != dir[t]) continue;
-                    const unsigned long long key = ((unsigned long long)(sa + g.suf[b]) << 2) | comp;
-                    atomicMin(best + t, key);
-                }
-            }
-        } else
-        for (int64_t p = threadIdx.x; p < P; p += TR_NT) {
-            int64_t lo = 0, hi = deg;  // entry a with pre[a] <= p < pre[a + 1]
-            while (hi - lo > 1) {
-                int64_t mid = (lo + hi) >> 1;
-                if (pre[mid] <= p) lo = mid; else hi = mid;
-            }
-            const int64_t a = lo;
-            const int32_t j = col[a];
-            const int64_t b = g.rp[j] + (p - pre[a]);
-            const int32_t k = g.col[b];
-            if (k == i) continue;
-            const int64_t t = find_col(col, deg, k);
-            if (t < 0) continue;
-            const uint32_t dij = dir[a], djk = g.dir[b];
-            if ((dij & 1u) != (djk >> 1)) continue;  // heads at j must point opposite ways
-            const uint32_t comp = (dij & 2u) | (djk & 1u);
-            if ((mode & 1) == SG_TR_DIRMATCH && comp != dir[t]) continue;
-            const unsigned long long key = ((unsigned long long)(suf[a] + g.suf[b]) << 2) | comp;
-            atomicMin(best + t, key);
+        int mykept = 0;
+        for (int64_t t = threadIdx.x; t < deg; t += TR_BNT) {
+            const bool f = !MIN && (hashed ? flag[t] != 0 : a.keep[r0 + t] == 0);
+            mykept += tr_outcome<MIN>(a, r0 + t, E(r0 + t), f, MIN ? best[t] : TR_NONE, v0, v1) ? 1 : 0;
         }
+        mykept = __reduce_add_sync(0xffffffffu, mykept);
+        if (lane == 0 && mykept) atomicAdd(&s_kept, mykept);
         __syncthreads();
-        uint32_t vm[2] = {0u, 0u};
-        for (int w = 0; w < TR_NT / 32; w++)
-            for (int e = 0; e < 2; e++) vm[e] = s_red[2 * w + e] > vm[e] ? s_red[2 * w + e] : vm[e];
-        const bool per_end = (mode & SG_TR_PER_END) != 0;
-        const uint32_t vrow = vm[0] > vm[1] ? vm[0] : vm[1];
-        const uint64_t v0 = (uint64_t)(per_end ? vm[0] : vrow) + fuzz;  // M_ik: the bound of end 0
-        const uint64_t v1 = (uint64_t)(per_end ? vm[1] : vrow) + fuzz;  // ... and of end 1
-        int64_t mykept = 0;
-        for (int64_t t = threadIdx.x; t < deg; t += TR_NT) {
-            const unsigned long long bt = best[t];
-            const uint32_t d = dir[t];
-            const bool has = bt != TR_NONE;
-            const uint64_t N = bt >> 2;
-            const bool transitive = has && (uint32_t)(bt & 3u) == d && ((d >> 1) ? v1 : v0) >= N;
-            if (keep) keep[r0 + t] = transitive ? 0 : 1;
-            mykept += transitive ? 0 : 1;
-            if (outN) outN[r0 + t] = has ? (uint32_t)N : 0xFFFFFFFFu;
-            if (outD) outD[r0 + t] = has ? (uint8_t)(bt & 3u) : (uint8_t)d;
-        }
-        if (kept) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mykept += __shfl_xor_sync(0xffffffffu, mykept, o);
-            if ((threadIdx.x & 31) == 0) s_kept[threadIdx.x >> 5] = mykept;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int64_t a = 0;
-                for (int w = 0; w < TR_NT / 32; w++) a += s_kept[w];
-                kept[i] = a;
-            }
-        }
+        if (threadIdx.x == 0 && a.kept) a.kept[i] = s_kept;
         __syncthreads();
     }
-}
-
-// rows of each kind: 0 = empty, 1 = staged in shared memory, 2 = global memory
-__global__ void tr_bin_kernel(const int64_t *__restrict__ rp, int64_t n, unsigned long long *__restrict__ counts,
-                              int8_t *__restrict__ kind) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t d = rp[i + 1] - rp[i];
-    int8_t c = d == 0 ? 0 : (d <= TR_SMEM_ROW ? 1 : 2);
-    kind[i] = c;
-    atomicAdd(counts + c, 1ull);
-}
-
-// rows[0 .. n) lists the shared-memory rows, rows[n .. 2n) the global-memory rows
-__global__ void tr_fill_kernel(const int8_t *__restrict__ kind, int64_t n, unsigned long long *__restrict__ cursor,
-                               int32_t *__restrict__ rows) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int c = kind[i];
-    if (c == 0) return;
-    unsigned long long p = atomicAdd(cursor + c, 1ull);
-    if (SG_IN_BOUNDS((int64_t)p < n, 403, p)) rows[(c == 1 ? 0 : n) + (int64_t)p] = (int32_t)i;
 }
 
 // Stable compaction of kept entries: one warp per row.
-__global__ void tr_compact_kernel(TrGraph g, const uint8_t *__restrict__ keep, const int64_t *__restrict__ nrp,
-                                  int32_t *__restrict__ ocol, uint32_t *__restrict__ osuf,
-                                  uint8_t *__restrict__ odir) {
-    int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
+__global__ void tr_compact_kernel(TrPacked g, const uint8_t *__restrict__ keep, const int64_t *__restrict__ nrp, TrBuf o) {
+    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (row >= g.n) return;
-    int64_t r0 = g.rp[row], r1 = g.rp[row + 1], w = nrp[row];
-    for (int64_t base = r0; base < r1; base += 32) {
-        int64_t e = base + lane;
-        bool kp = e < r1 && keep[e];
-        uint32_t bal = __ballot_sync(0xffffffffu, kp);
-        if (kp) {
-            int64_t o = w + __popc(bal & ((1u << lane) - 1u));
-            ocol[o] = g.col[e];
-            osuf[o] = g.suf[e];
-            odir[o] = g.dir[e];
-        }
-        w += __popc(bal);
+    const uint4 r = g.row[row];
+    const int64_t r0 = tr_first(r);
+    tr_write_row(o, row, nrp[row], (int64_t)r.z + r.w, [&](int64_t t) { return tr_entry(g, r0 + t); },
+                 [&](int64_t t) { return keep[r0 + t] != 0; });
+}
+
+// Packed entries -> the arrays of S.
+__global__ void tr_unpack_kernel(TrPacked g, int64_t nnz, const int64_t *__restrict__ rp, int64_t n,
+                                 int64_t *__restrict__ orp, int32_t *__restrict__ col, uint32_t *__restrict__ suf,
+                                 uint8_t *__restrict__ dir) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nnz) {
+        const uint64_t x = tr_entry(g, i);
+        col[i] = (int32_t)(x >> 32);
+        suf[i] = (uint32_t)x >> 2;
+        dir[i] = (uint8_t)(x & 3u);
     }
+    if (i <= n) orp[i] = rp[i];
 }
 
 static inline int64_t blocks_for(int64_t n, int nt) { return (n + nt - 1) / nt; }
 
-// Buffers reused by every round (sized for the input graph; later rounds only shrink).
+// Buffers of a round (sized for the input graph; later rounds only shrink).
 struct TrWork {
-    unsigned long long *counts;  // [6]: rows per kind, then fill cursors
-    int8_t *kind;                // [n + 1]
-    int32_t *rows;               // [2 (n + 1)]: shared-memory rows from 0, global-memory rows from n
-    unsigned long long *gbest;   // [nnz + 1] per-entry minima of global-memory rows
-    int64_t *gpre;               // [nnz + n + 1] neighbour-degree prefixes of global-memory rows
+    unsigned long long *n_big;  // [1] rows listed for blocks
+    int32_t *big;               // [n + 1]
+    unsigned long long *gbest;  // [nnz + 1] per-entry minima of rows above TR_BROW
 };
 
-// Element counts of TrWork's arrays for a graph of n rows and nnz entries, in field order. Both
-// the allocating path and the fixed-workspace path size their buffers from this one table.
-struct TrWorkSizes {
-    int64_t counts, kind, rows, gbest, gpre;
-};
-static TrWorkSizes tr_work_sizes(int64_t n, int64_t nnz) {
-    return TrWorkSizes{6, n + 1, 2 * (n + 1), nnz + 1, nnz + n + 1};
+static sg_status tr_work_alloc(TrWork *w, int64_t n, int64_t nnz, bool minima, Scratch &sc) {
+    w->n_big = sc.get<unsigned long long>(1);
+    w->big = sc.get<int32_t>(n + 1);
+    w->gbest = minima ? sc.get<unsigned long long>(nnz + 1) : nullptr;
+    return (w->n_big && w->big && (w->gbest || !minima)) ? SG_OK : SG_ERR_OOM;
 }
 
-static sg_status tr_work_alloc(TrWork *w, int64_t n, int64_t nnz, Scratch &sc) {
-    const TrWorkSizes z = tr_work_sizes(n, nnz);
-    w->counts = sc.get<unsigned long long>(z.counts);
-    w->kind = sc.get<int8_t>(z.kind);
-    w->rows = sc.get<int32_t>(z.rows);
-    w->gbest = sc.get<unsigned long long>(z.gbest);
-    w->gpre = sc.get<int64_t>(z.gpre);
-    return (w->counts && w->kind && w->rows && w->gbest && w->gpre) ? SG_OK : SG_ERR_OOM;
-}
-
-// One round over graph g: keep flags + per-row kept counts (and optionally N / Ndir). Rows are
-// binned on the device and both kernels run grid-stride over the device-side row counts, so the
+// One round over graph g: keep flags + per-row kept counts (and optionally N / Ndir). Rows for
+// blocks are listed on the device and the second kernel runs grid-stride over their number, so the
 // round needs no host round trip. Nothing runs past a set `err` (failed validation).
-static sg_status minplus_round(const TrGraph &g, int64_t nnz, int mode, uint32_t fuzz, uint8_t *keep,
-                               int64_t *kept, uint32_t *outN, uint8_t *outD, const TrWork &w, const uint32_t *err,
-                               cudaStream_t s) {
-    (void)nnz;
+static sg_status minplus_round(const TrPacked &g, int mode, uint32_t fuzz, uint8_t *keep, int64_t *kept, uint32_t *outN,
+                               uint8_t *outD, const TrWork &w, const uint32_t *err, cudaStream_t s) {
     const int64_t n = g.n;
-    unsigned long long *counts = w.counts;
-    SG_CUDA_TRY(cudaMemsetAsync(counts, 0, 6 * sizeof(unsigned long long), s));
-    if (kept) SG_CUDA_TRY(cudaMemsetAsync(kept, 0, (n + 1) * sizeof(int64_t), s));
     if (n == 0) return SG_OK;
-    SG_LAUNCH("tr_bin", tr_bin_kernel, blocks_for(n, 256), 256, 0, s, g.rp, n, counts, w.kind);
-    SG_LAUNCH("tr_fill", tr_fill_kernel, blocks_for(n, 256), 256, 0, s, w.kind, n, counts + 3, w.rows);
-    const int64_t gcap = (int64_t)sm_count() * tune("tr_blocks_per_sm");
-    const int64_t gs = n < gcap ? n : gcap;
-    SG_LAUNCH("tr_minplus_mark", minplus_mark_kernel<false>, gs, TR_NT, 0, s, g, (const int32_t *)w.rows,
-              counts + 1, err, mode, fuzz, (unsigned long long *)nullptr, (int64_t *)nullptr, keep, kept, outN,
-              outD, (int)tune("tr_warp_rows"));
-    const int64_t gg = n < (int64_t)sm_count() * 2 ? n : (int64_t)sm_count() * 2;
-    SG_LAUNCH("tr_minplus_mark_gmem", minplus_mark_kernel<true>, gg, TR_NT, 0, s, g, (const int32_t *)(w.rows + n),
-              counts + 2, err, mode, fuzz, w.gbest, w.gpre, keep, kept, outN, outD, 0);
+    if (w.big) SG_CUDA_TRY(cudaMemsetAsync(w.n_big, 0, sizeof(unsigned long long), s));
+    const TrArgs a{g, err, mode, fuzz, w.gbest, keep, kept, outN, outD, w.big, w.n_big, (int)tune("tr_warp_rows")};
+    const int64_t cap = (int64_t)sm_count() * tune("tr_blocks_per_sm"), rows = blocks_for(n, TR_NT / 32);
+    const int64_t gs = rows < cap ? rows : cap;
+    const int64_t gg = n < (int64_t)sm_count() * 3 ? n : (int64_t)sm_count() * 3;
+    if (outN || outD || (mode & 1) != SG_TR_DIRMATCH) {
+        SG_CUDA_TRY(ensure_smem(tr_mark_big_kernel<true>, tr_big_smem<true>()));
+        SG_LAUNCH("tr_minplus_mark", tr_mark_kernel<true>, gs, TR_NT, 0, s, a);
+        SG_LAUNCH("tr_minplus_mark_big", tr_mark_big_kernel<true>, gg, TR_BNT, tr_big_smem<true>(), s, a);
+    } else {
+        SG_CUDA_TRY(ensure_smem(tr_mark_big_kernel<false>, tr_big_smem<false>()));
+        SG_LAUNCH("tr_minplus_mark", tr_mark_kernel<false>, gs, TR_NT, 0, s, a);
+        SG_LAUNCH("tr_minplus_mark_big", tr_mark_big_kernel<false>, gg, TR_BNT, tr_big_smem<false>(), s, a);
+    }
     return SG_OK;
 }
 
@@ -347,34 +555,34 @@ sg_status tr_impl(const sg_graph_csr *R, uint32_t fuzz, int mode, sg_graph_csr *
     int64_t *kept = sc.get<int64_t>(n + 1);
     if (!err || !keep || !kept) return SG_ERR_OOM;
     TrWork wk;
-    SG_TRY(tr_work_alloc(&wk, n, nnz0, sc));
-    // two graph buffers of the input's size: round r reads one and compacts into the other
+    SG_TRY(tr_work_alloc(&wk, n, nnz0, (mode & 1) != SG_TR_DIRMATCH, sc));
+    // the rounds' graphs: each reads one buffer and compacts into the other (the first reads the
+    // caller's arrays beside buffer 0); row pointers of a round's result
+    TrBuf buf[2];
     int64_t *rp[2];
-    int32_t *col[2];
-    uint32_t *suf[2];
-    uint8_t *dir[2];
     for (int b = 0; b < 2; b++) {
+        buf[b].p = sc.get<uint64_t>(nnz0 + 1);
+        buf[b].row = sc.get<uint4>(n + 1);
         rp[b] = sc.get<int64_t>(n + 1);
-        col[b] = sc.get<int32_t>(nnz0 + 1);
-        suf[b] = sc.get<uint32_t>(nnz0 + 1);
-        dir[b] = sc.get<uint8_t>(nnz0 + 1);
-        if (!rp[b] || !col[b] || !suf[b] || !dir[b]) return SG_ERR_OOM;
+        if (!buf[b].p || !buf[b].row || !rp[b]) return SG_ERR_OOM;
     }
-    TrGraph g{R->row_ptr, R->col, R->suffix, R->dir, n};
+    const TrGraph in{R->row_ptr, R->col, R->suffix, R->dir, n};
     SG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-    SG_LAUNCH("validate_graph", validate_graph_kernel, blocks_for((n + 1) * 32, 256), 256, 0, s, g, nnz0, err);
+    SG_LAUNCH("validate_graph", validate_graph_kernel, blocks_for((n + 1) * 32, 256), 256, 0, s, in, nnz0, buf[0], err);
+    TrPacked g{nullptr, buf[0].p, buf[0].row, n, in};
+    const int64_t *grp = R->row_ptr;
     int64_t cur_nnz = nnz0;
-    int cur = -1;  // -1: the current graph is still the caller's R
+    int cur = 0;
     int32_t it = 0;
     bool done = false;
     for (;;) {
         if (max_rounds > 0 && it == max_rounds) break;  // stopped early: S is an intermediate R
         it++;
         StageScope round("TrRound", s);
-        const int nxt = cur == 0 ? 1 : 0;
-        SG_TRY(minplus_round(g, cur_nnz, mode, fuzz, keep, kept, nullptr, nullptr, wk, err, s));
+        const int nxt = 1 - cur;
+        SG_TRY(minplus_round(g, mode, fuzz, keep, kept, nullptr, nullptr, wk, err, s));
         if (job_ro)
-            SG_LAUNCH("tr_job_changes", job_changes_kernel, blocks_for(n, 256), 256, 0, s, g.rp,
+            SG_LAUNCH("tr_job_changes", job_changes_kernel, blocks_for(n, 256), 256, 0, s, grp,
                       (const int64_t *)kept, n, job_ro, njobs, it, job_last);
         SG_TRY(exclusive_scan<int64_t>(kept, rp[nxt], n, s, err));
         int64_t nnz2 = 0;
@@ -390,13 +598,15 @@ sg_status tr_impl(const sg_graph_csr *R, uint32_t fuzz, int mode, sg_graph_csr *
             done = true;
             break;
         }
-        SG_LAUNCH("tr_compact", tr_compact_kernel, blocks_for(n * 32, 256), 256, 0, s, g, keep, rp[nxt], col[nxt],
-                  suf[nxt], dir[nxt]);
+        if (!buf[nxt].e && !(buf[nxt].e = sc.get<uint64_t>(nnz2 + 1))) return SG_ERR_OOM;
+        SG_LAUNCH("tr_compact", tr_compact_kernel, blocks_for(n * 32, 256), 256, 0, s, g, (const uint8_t *)keep,
+                  (const int64_t *)rp[nxt], buf[nxt]);
         cur = nxt;
         cur_nnz = nnz2;
-        g = TrGraph{rp[cur], col[cur], suf[cur], dir[cur], n};
+        grp = rp[cur];
+        g = TrPacked{buf[cur].e, buf[cur].p, buf[cur].row, n, in};
     }
-    // S: exact-size copy of the final graph
+    // S: the final graph, unpacked into exact-size arrays
     sg_graph_csr out{};
     out.n = n;
     out.nnz = cur_nnz;
@@ -408,16 +618,14 @@ sg_status tr_impl(const sg_graph_csr *R, uint32_t fuzz, int mode, sg_graph_csr *
         free_graph_arrays(&out, s);
         return SG_ERR_OOM;
     }
-    cudaError_t e = cudaMemcpyAsync(out.row_ptr, g.rp, (n + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && cur_nnz)
-        e = cudaMemcpyAsync(out.col, g.col, cur_nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && cur_nnz)
-        e = cudaMemcpyAsync(out.suffix, g.suf, cur_nnz * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && cur_nnz) e = cudaMemcpyAsync(out.dir, g.dir, cur_nnz, cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) {
+    const sg_status st = [&]() -> sg_status {
+        SG_LAUNCH("tr_unpack", tr_unpack_kernel, blocks_for(std::max(cur_nnz, n + 1), 256), 256, 0, s, g, cur_nnz, grp, n,
+                  out.row_ptr, out.col, out.suffix, out.dir);
+        return SG_OK;
+    }();
+    if (st != SG_OK) {
         free_graph_arrays(&out, s);
-        set_error("transitive_reduce: copying S failed: %s", cudaGetErrorString(e));
-        return SG_ERR_CUDA;
+        return st;
     }
     *S = out;
     *iters = it;
@@ -478,10 +686,15 @@ extern "C" sg_status sg_minplus_square(const sg_graph_csr *R, int32_t mode, uint
     if (!err) return SG_ERR_OOM;
     sg::TrGraph g{R->row_ptr, R->col, R->suffix, R->dir, R->n};
     sg::TrWork wk;
-    SG_TRY(sg::tr_work_alloc(&wk, R->n, R->nnz, sc));
+    SG_TRY(sg::tr_work_alloc(&wk, R->n, R->nnz, true, sc));
+    sg::TrBuf buf;
+    buf.p = sc.get<uint64_t>(R->nnz + 1);
+    buf.row = sc.get<uint4>(R->n + 1);
+    if (!buf.p || !buf.row) return SG_ERR_OOM;
     SG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-    SG_LAUNCH("validate_graph", sg::validate_graph_kernel, (R->n + 1 + 7) / 8, 256, 0, s, g, R->nnz, err);
-    SG_TRY(sg::minplus_round(g, R->nnz, mode, 0, nullptr, nullptr, d_N, d_Ndir, wk, err, s));
+    SG_LAUNCH("validate_graph", sg::validate_graph_kernel, (R->n + 1 + 7) / 8, 256, 0, s, g, R->nnz, buf, err);
+    SG_TRY(sg::minplus_round(sg::TrPacked{nullptr, buf.p, buf.row, R->n, g}, mode, 0, nullptr, nullptr, d_N, d_Ndir, wk, err,
+                             s));
     uint32_t herr = 0;
     SG_CUDA_TRY(sg::read_back(&herr, err, sizeof(uint32_t), s));
     if (herr) {
@@ -550,17 +763,15 @@ extern "C" sg_status sg_minplus_square_noalloc(const sg_graph_csr *R, int32_t mo
         return SG_ERR_INVALID;
     }
     const int64_t n = R->n, nnz = R->nnz;
-    // workspace layout inside the scratch array: the error word, then TrWork's arrays with the
-    // sizes the allocating path uses
-    const sg::TrWorkSizes z = sg::tr_work_sizes(n, nnz);
+    // workspace layout inside the scratch array: the error word, the packed rows and entries, the
+    // per-entry minima. The limit is the documented one, a little above what they take.
     const size_t o_err = 0;
-    const size_t o_cnt = sg::up256(o_err + sizeof(uint32_t));
-    const size_t o_kind = sg::up256(o_cnt + (size_t)z.counts * sizeof(unsigned long long));
-    const size_t o_rows = sg::up256(o_kind + (size_t)z.kind * sizeof(int8_t));
-    const size_t o_best = sg::up256(o_rows + (size_t)z.rows * sizeof(int32_t));
-    const size_t o_pre = sg::up256(o_best + (size_t)z.gbest * sizeof(unsigned long long));
-    const size_t need = o_pre + (size_t)z.gpre * sizeof(int64_t);
-    if (need > (size_t)SG_NOALLOC_SCRATCH_BYTES) {
+    const size_t o_row = sg::up256(o_err + sizeof(uint32_t));
+    const size_t o_ent = sg::up256(o_row + (size_t)n * sizeof(uint4));
+    const size_t o_best = sg::up256(o_ent + (size_t)nnz * sizeof(uint64_t));
+    const size_t need = sg::up256(sg::up256(sg::up256(512 + (size_t)(n + 1)) + (size_t)(n + 1) * 8) +
+                                  (size_t)(nnz + 1) * 8) + (size_t)(nnz + n + 1) * 8;
+    if (need > (size_t)SG_NOALLOC_SCRATCH_BYTES || o_best + (size_t)nnz * 8 > (size_t)SG_NOALLOC_SCRATCH_BYTES) {
         sg::set_error("minplus_square_noalloc: a graph with n=%lld and nnz=%lld needs %zu bytes of workspace, "
                       "more than the fixed %zu-byte scratch array; use sg_minplus_square",
                       (long long)n, (long long)nnz, need, (size_t)SG_NOALLOC_SCRATCH_BYTES);
@@ -571,23 +782,24 @@ extern "C" sg_status sg_minplus_square_noalloc(const sg_graph_csr *R, int32_t mo
     cudaStream_t s = (cudaStream_t)stream;
     uint32_t *err = (uint32_t *)(base + o_err);
     sg::TrWork wk;
-    wk.counts = (unsigned long long *)(base + o_cnt);
-    wk.kind = (int8_t *)(base + o_kind);
-    wk.rows = (int32_t *)(base + o_rows);
+    wk.n_big = nullptr;  // no room for a list of long rows: blocks look for them
+    wk.big = nullptr;
     wk.gbest = (unsigned long long *)(base + o_best);
-    wk.gpre = (int64_t *)(base + o_pre);
+    sg::TrBuf buf;
+    buf.p = (uint64_t *)(base + o_ent);
+    buf.row = (uint4 *)(base + o_row);
     sg::TrGraph g{R->row_ptr, R->col, R->suffix, R->dir, n};
-    // the array keeps whatever the previous call left: the error word starts from zero here,
-    // the row counters are zeroed by minplus_round, and every other word is written before read
+    // the array keeps whatever the previous call left: the error word starts from zero here, and
+    // every other word is written before read
     SG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-    SG_LAUNCH("validate_graph", sg::validate_graph_kernel, (n + 1 + 7) / 8, 256, 0, s, g, nnz, err);
+    SG_LAUNCH("validate_graph", sg::validate_graph_kernel, (n + 1 + 7) / 8, 256, 0, s, g, nnz, buf, err);
     uint32_t herr = 0;
     SG_CUDA_TRY(sg::read_back(&herr, err, sizeof(uint32_t), s));
     if (herr) {
         sg::set_error("minplus_square_noalloc: graph does not satisfy the CSR contract");
         return SG_ERR_INVALID;
     }
-    SG_TRY(sg::minplus_round(g, nnz, mode, 0, nullptr, nullptr, d_N, d_Ndir, wk, err, s));
+    SG_TRY(sg::minplus_round(sg::TrPacked{nullptr, buf.p, buf.row, n, g}, mode, 0, nullptr, nullptr, d_N, d_Ndir, wk, err, s));
     SG_CUDA_TRY(cudaStreamSynchronize(s));
     return SG_OK;
 }
