@@ -313,7 +313,7 @@ static Tunable g_tunables[] = {
                                           // mirrors them (C is symmetric); 0: whole rows
     {"spgemm_at_records", 1, 0, 1},       // 1: the fused pass reads At rows as 32-byte records
     {"spgemm_smem_carveout", -1, -1, 100},// fused-pass shared-memory carveout, % (-1: the driver's)
-    {"spgemm_escalate", 1, 0, 8},         // a guessed table that overflows is tried once more
+    {"spgemm_escalate", 2, 0, 8},         // a guessed table that overflows is tried once more
                                           // 2^this times larger in shared memory (0: global memory)
     {"spgemm_mirror_rec", 1, 0, 1},       // 1: (mirror sort) U's entries copied into 32-byte records that
                                           // the mirror reads, instead of C's arrays (max_seeds <= 3)
@@ -322,9 +322,9 @@ static Tunable g_tunables[] = {
     {"spgemm_lower_smem", 4096, 1, 4096}, // (0 above) parts up to this long are sorted in shared memory
     {"spgemm_tab_warps", 64, 0, 64},      // fused-pass blocks: threads for about this many warps per SM
                                           // across the blocks that fit (0: fixed threads per table size)
-    {"spgemm_tab_warps_big", 32, 1, 64},  // ... the same for tables of 4 K slots and more
+    {"spgemm_tab_warps_big", 64, 1, 64},  // ... the same for tables of 4 K slots and more
     {"spgemm_sample_rows", 256, 0, 1 << 20},  // rows sampled for the fused tables' guesses (0: none)
-    {"spgemm_guess_pct", 200, 1, 10000},  // guess = pct / 100 x sampled partners per A entry x entries
+    {"spgemm_guess_pct", 180, 1, 10000},  // guess = pct / 100 x sampled partners per A entry x entries
     {"spgemm_tmp_pct", 125, 1, 10000},    // fused temporary region = pct / 100 x sampled kept entries
                                           // (+ 4 per row); rows that find it full are redone
     {"spgemm_fused_max_mb", 65536, 0, 1 << 30},  // temporary C region above which the two passes run
@@ -335,7 +335,7 @@ static Tunable g_tunables[] = {
                                           // may first mark partners seen twice (0: never)
     {"spgemm_filter_log2", 17, 10, 19},   // at most 2^this bits per seen-once / seen-twice filter
     {"sym_guess_shift", 2, 0, 8},         // symbolic table guess = products >> shift
-    {"spgemm_blocks_per_sm", 16, 1, 64},  // grid of each SpGEMM class launch
+    {"spgemm_blocks_per_sm", 64, 1, 64},  // grid of each SpGEMM class launch
     {"spgemm_big_threads", 1024, 512, 1024},  // threads of numeric blocks with 4 K table slots or more
     {"tr_blocks_per_sm", 32, 1, 64},      // grid of the min-plus launch
     {"tr_warp_rows", 1, 0, 1},            // 1: rows of up to 128 entries reduced by a warp each; 0: by blocks

@@ -621,8 +621,8 @@ __device__ __forceinline__ void at_extent(const SpArgs &g, int64_t a, int32_t gi
     len = (uint32_t)(e - lo);
 }
 
-// Products of row i (read id gi) with their partner counts: f(k, idx) for every product, k = the
-// partner, idx = index of the A entry within the row; k == gi is skipped. Warp-cooperative: a warp
+// Products of row i (read id gi): f(k, idx, ok) by every lane of the warp, for every product (ok): k =
+// the partner, idx = index of the A entry within the row; k == gi is no product. Warp-cooperative: a warp
 // takes 32 consecutive entries of A's row, finds their extents, scans their lengths (32-bit) and
 // walks the flattened products TU_U x 32 at a time, each lane finding its entry by a 5-step
 // shuffle search; the gathers of the next step are issued before the current step's table
@@ -699,8 +699,7 @@ __device__ __forceinline__ void enum_fused(const SpArgs &g, int32_t gi, int64_t 
             }
             if (base + 32 * TU_U < total) gather(base + 32 * TU_U);
 #pragma unroll
-            for (int u = 0; u < TU_U; u++)
-                if (k_cur[u] != gi) f(k_cur[u], i_cur[u]);
+            for (int u = 0; u < TU_U; u++) f(k_cur[u], i_cur[u], k_cur[u] != gi);
         }
     }
 }
@@ -716,6 +715,51 @@ __device__ __forceinline__ uint32_t at_value_cv(const int32_t *__restrict__ t_co
         if (t_col[mid] <= k) lo = mid; else hi = mid;
     }
     return t_val[lo];
+}
+
+// The seed positions of pair (i, k) met through A entries a0 (and a1, N == 2): i's own, and k's with
+// the strands' xor.
+template <int N>
+__device__ __forceinline__ void seeds_of(const SpArgs &g, int64_t a0, int64_t a1, int32_t k, uint32_t *si, uint32_t *sk) {
+    uint32_t vi[N], vk[N];
+    int32_t j[N];
+    int64_t b[N], at[N];
+    uint32_t len[N];
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+        vi[q] = g.a_val[q ? a1 : a0];
+        j[q] = g.a_col[q ? a1 : a0];
+    }
+    if (g.t_rec) {
+        AtRec rr[N];
+#pragma unroll
+        for (int q = 0; q < N; q++) rr[q] = load_rec(g.t_rec + j[q]);
+#pragma unroll
+        for (int q = 0; q < N; q++) {
+            b[q] = at[q] = rr[q].b;
+            len[q] = rr[q].len;
+            if (len[q] <= AT_INL) {
+#pragma unroll
+                for (int t = 1; t < AT_INL; t++)
+                    if (t < (int)rr[q].len && rr[q].r[t] <= k) at[q] = b[q] + t;
+                len[q] = 0;  // found
+            }
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; q++) {
+            b[q] = g.t_rp[j[q]];
+            len[q] = (uint32_t)(g.t_rp[j[q] + 1] - b[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < N; q++) vk[q] = len[q] == 0 ? g.t_val[at[q]] : 0u;
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+        if (len[q]) vk[q] = at_value_cv(g.t_col, g.t_val, b[q], len[q], k);
+        si[q] = vi[q] & 0x7FFFFFFFu;
+        sk[q] = (vk[q] & 0x7FFFFFFFu) | ((vi[q] ^ vk[q]) & 0x80000000u);
+    }
 }
 
 // Bytes of one table of T slots with S seeds: slots u64[T] | seeds | sort buffer u64[T / 2].
@@ -809,7 +853,8 @@ __global__ void SG_TAB_BOUNDS tab_numeric_kernel(SpArgs g, const int32_t *__rest
             return fid ? (uint32_t)k & ((1u << log2F) - 1u) : ((uint32_t)k * 2654435761u) >> (32 - log2F);
         };
         if (FILT) {  // seen once -> F1, seen again -> F2 (bits are only ever set)
-            enum_fused<UPPER>(g, gi, r0, r1, nullptr, wb, [&](int32_t k, uint32_t) {
+            enum_fused<UPPER>(g, gi, r0, r1, nullptr, wb, [&](int32_t k, uint32_t, bool ok) {
+                if (!ok) return;
                 const uint32_t b = fbit(k), m = 1u << (b & 31u);
                 if (((volatile uint32_t *)F2)[b >> 5] & m) return;
                 if (atomicOr(F1 + (b >> 5), m) & m) atomicOr(F2 + (b >> 5), m);
@@ -817,8 +862,8 @@ __global__ void SG_TAB_BOUNDS tab_numeric_kernel(SpArgs g, const int32_t *__rest
             __syncthreads();
         }
         const int cap = (T >> 1) + (T >> 2);
-        enum_fused<UPPER>(g, gi, r0, r1, GSLICE ? nullptr : &s_ovf, wb, [&](int32_t k, uint32_t idx) {
-            if (!GSLICE && *(volatile int *)&s_ovf) return;
+        enum_fused<UPPER>(g, gi, r0, r1, GSLICE ? nullptr : &s_ovf, wb, [&](int32_t k, uint32_t idx, bool ok) {
+            if (!ok || (!GSLICE && *(volatile int *)&s_ovf)) return;
             if (FILT) {
                 const uint32_t b = fbit(k);
                 if (!((F2[b >> 5] >> (b & 31u)) & 1u)) return;
@@ -945,30 +990,257 @@ __global__ void SG_TAB_BOUNDS tab_numeric_kernel(SpArgs g, const int32_t *__rest
                 else sdx = seed1[(int64_t)x * S + s];
                 uint32_t si = SEED_NONE, sk = SEED_NONE;
                 if (sdx != SEED_NONE) {
-                    const int64_t a = r0 + sdx;
-                    const uint32_t vi = g.a_val[a];
-                    const int32_t j = g.a_col[a];
-                    uint32_t vk;
-                    if (g.t_rec) {
-                        const AtRec rr = load_rec(g.t_rec + j);
-                        if (rr.len <= AT_INL) {
-                            int q = 0;
-#pragma unroll
-                            for (int t = 1; t < AT_INL; t++)
-                                if (t < (int)rr.len && rr.r[t] <= k) q = t;
-                            vk = g.t_val[rr.b + q];
-                        } else {
-                            vk = at_value_cv(g.t_col, g.t_val, rr.b, rr.len, k);
-                        }
-                    } else {
-                        const int64_t tb0 = g.t_rp[j];
-                        vk = at_value_cv(g.t_col, g.t_val, tb0, g.t_rp[j + 1] - tb0, k);
-                    }
-                    si = vi & 0x7FFFFFFFu;
-                    sk = (vk & 0x7FFFFFFFu) | ((vi ^ vk) & 0x80000000u);
+                    seeds_of<1>(g, r0 + sdx, 0, k, &si, &sk);
                 }
                 o.si[(int64_t)s * o.cap + e] = si;
                 o.sk[(int64_t)s * o.cap + e] = sk;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The shared-memory pass for max_seeds <= 2 and rows of fewer than 2^16 A entries: the table of
+// tab_numeric_kernel in 10 bytes per slot instead of 20 -- key u32, the two smallest A-entry indices
+// of a partner in one u32, its count in 16 bits -- so that a 16 K-slot table fits a block, an 8 K-slot
+// one fits twice on an SM, and every update is a 32-bit shared-memory atomic. New partners are
+// counted once per warp step. Kept partners are ordered by counting into as many bins as there are
+// partners between the smallest and the largest (bitonic only where a bin gets crowded). The pass
+// stays bound by the gathers (random At records, about 40 G sectors per second) and their latency.
+// With the fitted table sizes, one call: 5 Mbp at 30x 2.26 -> 1.79 ms, 25 Mbp at 40x 14.4 -> 12.3 ms.
+constexpr int CT_ROW = 65535;   // A entries of a row
+constexpr int CT_CROWD = 48;    // partners of one bin ranked against each other
+constexpr uint32_t CT_FREE = 0xFFFFFFFFu;
+
+// slots | seeds | counts | bins u32 and two lists u16 of T >> oblog entries
+__host__ __device__ inline size_t ctab_bytes(int64_t T, int S, int oblog) {
+    return (size_t)T * (S > 0 ? 10 : 6) + (size_t)(T >> oblog) * 8;
+}
+
+// 32 registers: 64 warps per SM, which the gathers' latency wants (25 Mbp at 40x: 12.3 ms a call; 40
+// registers and 48 warps: 13.2 ms).
+template <int SK, bool UPPER>
+__global__ void __maxnreg__(32) ctab_numeric_kernel(SpArgs g, const int32_t *__restrict__ rows,
+                                                  const unsigned long long *__restrict__ nrows_p, int lT, int oblog,
+                                                  TmpOut o, int32_t *__restrict__ ovf_list,
+                                                  unsigned long long *__restrict__ ovf_count, int64_t wb_off,
+                                                  int8_t *__restrict__ ovf_lt) {
+    extern __shared__ __align__(16) unsigned char tab_raw[];
+    __shared__ int s_ctr, s_ins, s_ovf, s_full, s_fail, s_crowd;
+    __shared__ uint32_t s_lo, s_hi, s_w[33];
+    __shared__ unsigned long long s_e0;
+    const int T = 1 << lT, OB = T >> oblog, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t *key = reinterpret_cast<uint32_t *>(tab_raw);
+    uint32_t *sd = key + T;
+    uint32_t *cnt2 = sd + (SK > 0 ? T : 0);
+    uint32_t *bins = cnt2 + T / 2;
+    uint16_t *la = reinterpret_cast<uint16_t *>(bins + OB), *lb = la + OB;
+    int32_t *wb = g.t_rec ? (int32_t *)(tab_raw + wb_off) : nullptr;  // record reads, per warp
+    const uint32_t msk = (uint32_t)T - 1u;
+    const int cap = (T >> 1) + (T >> 2);
+    const int64_t nrows = (int64_t)*nrows_p;
+    auto count_of = [&](uint32_t x) { return (cnt2[x >> 1] >> (16 * (x & 1u))) & 0xffffu; };
+    for (int64_t rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
+        const int32_t i = rows[rb];
+        if (!SG_IN_BOUNDS(i >= 0 && i < g.n, 308, i)) continue;
+        const int32_t gi = (int32_t)(g.row0 + i);
+        const uint4 ones = make_uint4(CT_FREE, CT_FREE, CT_FREE, CT_FREE);
+        for (int x = tid; x < (SK > 0 ? T / 2 : T / 4); x += nt) reinterpret_cast<uint4 *>(key)[x] = ones;
+        for (int x = tid; x < T / 8; x += nt) reinterpret_cast<uint4 *>(cnt2)[x] = make_uint4(0, 0, 0, 0);
+        if (tid == 0) {
+            s_ctr = s_ins = s_ovf = s_full = s_crowd = 0;
+            s_lo = 0xFFFFFFFFu;
+            s_hi = 0;
+        }
+        __syncthreads();
+        const int64_t r0 = g.a_rp[i], r1 = g.a_rp[i + 1];
+        enum_fused<UPPER>(g, gi, r0, r1, &s_ovf, wb, [&](int32_t kk, uint32_t idx, bool ok) {
+            bool fresh = false;
+            if (ok && !*(volatile int *)&s_ovf) {
+                const uint32_t k = (uint32_t)kk;
+                uint32_t h = hash_slot(kk, lT);
+                int probe = 0;
+                for (;;) {
+                    uint32_t v = ((volatile uint32_t *)key)[h];
+                    if (v == CT_FREE) {
+                        v = atomicCAS(key + h, CT_FREE, k);
+                        fresh = v == CT_FREE;
+                        if (fresh) break;
+                    }
+                    if (v == k) break;
+                    h = (h + 1) & msk;
+                    if (++probe == T) {  // went round the whole table
+                        s_ovf = 1;
+                        break;
+                    }
+                }
+                if (probe < T) {
+                    atomicAdd(cnt2 + (h >> 1), 1u << (16 * (h & 1u)));
+                    if (SK == 1) {
+                        if (idx < *(volatile uint32_t *)(sd + h)) atomicMin(sd + h, idx);
+                    } else if (SK == 2) {
+                        uint32_t w = ((volatile uint32_t *)sd)[h];
+                        for (;;) {  // smallest << 16 | second smallest; indices of a partner are distinct
+                            const uint32_t m1 = w >> 16, m2 = w & 0xffffu;
+                            if (idx >= m2) break;
+                            const uint32_t old = atomicCAS(sd + h, w, idx < m1 ? (idx << 16) | m1 : (m1 << 16) | idx);
+                            if (old == w) break;
+                            w = old;
+                        }
+                    }
+                }
+            }
+            const uint32_t fm = __ballot_sync(0xffffffffu, fresh);
+            if (fm && lane == 0 && atomicAdd(&s_ins, __popc(fm)) + __popc(fm) > cap) s_ovf = 1;
+        });
+        __syncthreads();
+        if (!s_ovf) {  // kept partners -> la
+            for (int x0 = 0; x0 < T; x0 += nt) {
+                const int x = x0 + tid;
+                const bool kept = x < T && count_of(x) >= g.min_shared;
+                const uint32_t m = __ballot_sync(0xffffffffu, kept);
+                if (m == 0) continue;
+                int p = 0;
+                if (lane == 0) p = atomicAdd(&s_ctr, __popc(m));
+                p = __shfl_sync(0xffffffffu, p, 0) + __popc(m & ((1u << lane) - 1u));
+                if (kept) {
+                    if (p < OB) la[p] = (uint16_t)x; else s_full = 1;
+                }
+                const uint32_t k = kept ? key[x] : 0u;
+                const uint32_t lo = __reduce_min_sync(0xffffffffu, kept ? k : 0xFFFFFFFFu);
+                const uint32_t hi = __reduce_max_sync(0xffffffffu, k);
+                if (lane == 0) {
+                    atomicMin(&s_lo, lo);
+                    atomicMax(&s_hi, hi);
+                }
+            }
+        }
+        __syncthreads();
+        if (s_ovf || s_full) {  // redone in a larger table
+            if (tid == 0) {
+                const unsigned long long q = atomicAdd(ovf_count, 1ull);
+                if (SG_IN_BOUNDS((int64_t)q < g.n, 311, q)) {
+                    ovf_list[q] = i;
+                    if (ovf_lt) ovf_lt[q] = (int8_t)lT;  // the table that was too small
+                }
+            }
+            __syncthreads();
+            continue;
+        }
+        const int nv = s_ctr;
+        if (tid == 0) {  // reserve the row's entries in the temporary region
+            const unsigned long long e0 = atomicAdd(o.cursor, (unsigned long long)nv);
+            s_e0 = e0;
+            s_fail = e0 + (unsigned long long)nv > (unsigned long long)o.cap;
+            if (s_fail) {
+                const unsigned long long q = atomicAdd(o.n_retry, 1ull);
+                if (SG_IN_BOUNDS((int64_t)q < g.n, 316, q)) o.retry[q] = i;
+            } else {
+                o.off[i] = (int64_t)e0;
+                o.len[i] = nv;
+            }
+        }
+        int nb = 32;
+        while (nb < nv && nb < OB) nb <<= 1;
+        if (nb > OB) nb = OB;
+        for (int x = tid; x < nb; x += nt) bins[x] = 0;
+        __syncthreads();
+        if (s_fail) continue;  // the region is full: the row is redone in a grown one
+        const uint32_t klo = s_lo;
+        const float scale = (float)nb / ((float)(s_hi - klo) + 1.0f);
+        auto bin_of = [&](uint32_t k) {  // ascending with k
+            const uint32_t b = (uint32_t)((float)(k - klo) * scale);
+            return b < (uint32_t)nb ? b : (uint32_t)nb - 1u;
+        };
+        for (int q = tid; q < nv; q += nt)
+            if (atomicAdd(bins + bin_of(key[la[q]]), 1u) == CT_CROWD) s_crowd = 1;
+        __syncthreads();
+        {  // bins -> their starts
+            const int per = (nb + nt - 1) / nt, b0 = tid * per;
+            uint32_t sum = 0;
+            for (int b = b0; b < b0 + per && b < nb; b++) sum += bins[b];
+            uint32_t inc = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= d) inc += y;
+            }
+            if (lane == 31) s_w[warp] = inc;
+            __syncthreads();
+            if (warp == 0) {
+                uint32_t t = lane < nt / 32 ? s_w[lane] : 0u;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, t, d);
+                    if (lane >= d) t += y;
+                }
+                s_w[lane + 1] = t;
+                if (lane == 0) s_w[0] = 0;
+            }
+            __syncthreads();
+            uint32_t ex = s_w[warp] + inc - sum;
+            for (int b = b0; b < b0 + per && b < nb; b++) {
+                const uint32_t c = bins[b];
+                bins[b] = ex;
+                ex += c;
+            }
+        }
+        __syncthreads();
+        if (!s_crowd) {
+            for (int q = tid; q < nv; q += nt) {
+                const uint16_t x = la[q];
+                lb[atomicAdd(bins + bin_of(key[x]), 1u)] = x;
+            }
+            __syncthreads();
+            for (int q = tid; q < nv; q += nt) {  // bins[b] is now the end of bin b
+                const uint16_t x = lb[q];
+                const uint32_t k = key[x], b = bin_of(k);
+                uint32_t d = b ? bins[b - 1] : 0u;
+                for (uint32_t j = d, e = bins[b]; j < e; j++) d += key[lb[j]] < k ? 1u : 0u;
+                la[d] = x;
+            }
+            __syncthreads();
+        } else {
+            int P2 = 1;
+            while (P2 < nv) P2 <<= 1;  // <= OB
+            for (int x = nv + tid; x < P2; x += nt) la[x] = 0xffffu;
+            __syncthreads();
+            auto key_at = [&](uint16_t x) { return x == 0xffffu ? 0xFFFFFFFFu : key[x]; };
+            for (int kk = 2; kk <= P2; kk <<= 1)
+                for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+                    for (int x = tid; x < P2; x += nt) {
+                        const int y = x ^ jj;
+                        if (y < x) continue;
+                        const uint16_t a = la[x], b = la[y];
+                        if ((key_at(a) > key_at(b)) == ((x & kk) == 0)) {
+                            la[x] = b;
+                            la[y] = a;
+                        }
+                    }
+                    __syncthreads();
+                }
+        }
+        const int64_t e0 = (int64_t)s_e0;
+        for (int q = tid; q < nv; q += nt) {
+            const uint32_t x = la[q];
+            const int32_t k = (int32_t)key[x];
+            const int64_t e = e0 + q;
+            o.col[e] = k;
+            o.cnt[e] = count_of(x);
+            if (o.colcnt) atomicAdd(o.colcnt + k, 1u);
+            if (SK == 0) continue;
+            const uint32_t w = sd[x];
+            // every partner has a first seed; both chains of loads travel together
+            const int64_t a0 = r0 + (SK == 2 ? w >> 16 : w);
+            const bool second = SK == 2 && (w & 0xffffu) != 0xffffu;
+            const int64_t a1 = second ? r0 + (w & 0xffffu) : a0;
+            uint32_t si[2], sk[2];
+            seeds_of<SK == 2 ? 2 : 1>(g, a0, a1, k, si, sk);
+            o.si[e] = si[0];
+            o.sk[e] = sk[0];
+            if (SK == 2) {
+                o.si[o.cap + e] = second ? si[1] : SEED_NONE;
+                o.sk[o.cap + e] = second ? sk[1] : SEED_NONE;
             }
         }
         __syncthreads();
@@ -1007,10 +1279,10 @@ __global__ void rows_work_kernel(SpArgs g, const int32_t *__restrict__ rows, con
 
 // Sampled rows (every stride-th row, one block each): the row's A entries, and the bits set in the
 // seen-once and seen-twice filters after its products -- about its distinct partners and its
-// partners seen at least twice. sums = {sum of A entries, sum F1 bits, sum F2 bits}.
+// partners seen at least twice. rec[3 b] = {A entries, F1 bits, F2 bits} of sampled row b.
 template <bool UPPER>
 __global__ void __launch_bounds__(512) sample_fx_kernel(SpArgs g, int64_t stride, int log2F,
-                                                       unsigned long long *__restrict__ sums) {
+                                                       unsigned long long *__restrict__ rec) {
     extern __shared__ __align__(16) uint32_t smp_f[];
     __shared__ unsigned long long s_c[2];
     const int64_t i = (int64_t)blockIdx.x * stride;
@@ -1022,7 +1294,8 @@ __global__ void __launch_bounds__(512) sample_fx_kernel(SpArgs g, int64_t stride
     __syncthreads();
     const bool fid = g.np <= ((int64_t)1 << log2F);
     int32_t *wb = g.t_rec ? (int32_t *)(smp_f + 2 * nw) : nullptr;
-    enum_fused<UPPER>(g, (int32_t)(g.row0 + i), g.a_rp[i], g.a_rp[i + 1], nullptr, wb, [&](int32_t k, uint32_t) {
+    enum_fused<UPPER>(g, (int32_t)(g.row0 + i), g.a_rp[i], g.a_rp[i + 1], nullptr, wb, [&](int32_t k, uint32_t, bool ok) {
+        if (!ok) return;
         const uint32_t b = fid ? (uint32_t)k & ((1u << log2F) - 1u) : ((uint32_t)k * 2654435761u) >> (32 - log2F);
         const uint32_t m = 1u << (b & 31u);
         if (((volatile uint32_t *)F2)[b >> 5] & m) return;
@@ -1038,33 +1311,78 @@ __global__ void __launch_bounds__(512) sample_fx_kernel(SpArgs g, int64_t stride
     atomicAdd(&s_c[1], c2);
     __syncthreads();
     if (threadIdx.x == 0) {
-        atomicAdd(sums, (unsigned long long)(g.a_rp[i + 1] - g.a_rp[i]));
-        atomicAdd(sums + 1, s_c[0]);
-        atomicAdd(sums + 2, s_c[1]);
+        rec[3 * (int64_t)blockIdx.x] = (unsigned long long)(g.a_rp[i + 1] - g.a_rp[i]);
+        rec[3 * (int64_t)blockIdx.x + 1] = s_c[0];
+        rec[3 * (int64_t)blockIdx.x + 2] = s_c[1];
     }
 }
 
-// Table requests of the fused pass, from each row's number of A entries L: a guess of
-// (L * fu) >> 16 partners (fu = sampled partners per A entry, fixed point), at least 64 slots.
+// Partners of row i, with L entries of A, as L (base + slope (1 - i / n)) (fixed point, 16 bits):
+// in the upper-triangle form a row meets only later reads. Whether their number falls with i
+// depends on the order of the reads (random: base = 0; along the genome: slope = 0), so both are
+// fitted to the sample.
+struct PartnerFit {
+    uint64_t base, slope;
+};
+__device__ __forceinline__ int64_t fit_at(const PartnerFit &f, int64_t L, int64_t i, int64_t n) {
+    const double x = (double)f.base + (double)f.slope * ((double)(n - i) / (double)n);
+    return (int64_t)((double)L * x * (1.0 / 65536.0));
+}
+
+// Table requests of the fused pass, from each row's number of A entries L: a guess of fu's partners,
+// at least 64 slots; *kept += fk's (the kept partners).
 // Rows with L >= fwork (fwork > 0) take the filtered pass: their guess ((L * ff) >> 16, at most
 // fcap = the largest filtered shared-memory table) goes to need_f and need is 0, else need_f is 0.
-__global__ void fx_need_kernel(const int64_t *__restrict__ a_rp, int64_t n, uint64_t fu, int64_t fwork, uint64_t ff,
-                               int64_t fcap, int64_t tcap, int64_t *__restrict__ need, int64_t *__restrict__ need_f) {
+// Unfiltered rows of more than lmax entries take the global-memory class.
+__global__ void fx_need_kernel(const int64_t *__restrict__ a_rp, int64_t n, PartnerFit fu, PartnerFit fk, int64_t fwork,
+                               uint64_t ff, int64_t fcap, int64_t tcap, int64_t lmax, int64_t *__restrict__ need,
+                               int64_t *__restrict__ need_f, unsigned long long *__restrict__ kept) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t L = a_rp[i + 1] - a_rp[i];
-    need_f[i] = 0;
-    if (L <= 0) {
+    unsigned long long mine = 0;
+    if (i < n) {
+        const int64_t L = a_rp[i + 1] - a_rp[i];
+        need_f[i] = 0;
         need[i] = 0;
-        return;
+        if (L > 0) {
+            const bool filt = fwork > 0 && L >= fwork;
+            const int64_t g0 = filt ? (int64_t)(((unsigned __int128)L * ff) >> 16) : fit_at(fu, L, i, n);
+            int64_t guess = pow2_at_least(g0 > 64 ? g0 : 64);
+            if (guess > tcap) guess = tcap;  // no row has more partners than the table bound for all reads
+            if (filt && guess > fcap) guess = fcap;
+            if (!filt && L > lmax) guess = (int64_t)1 << 40;
+            (filt ? need_f : need)[i] = guess;
+            mine = (unsigned long long)fit_at(fk, L, i, n);
+        }
     }
-    const bool filt = fwork > 0 && L >= fwork;
-    const int64_t g0 = (int64_t)(((unsigned __int128)L * (filt ? ff : fu)) >> 16);
-    int64_t guess = pow2_at_least(g0 > 64 ? g0 : 64);
-    if (guess > tcap) guess = tcap;  // no row has more partners than the table bound for all reads
-    if (filt && guess > fcap) guess = fcap;
-    (filt ? need_f : need)[i] = guess;
-    if (filt) need[i] = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(kept, mine);
+}
+
+// Least-squares fit of y = L (base + slope x) to the sampled rows (x = 1 - i / n), neither negative.
+struct FitD {
+    double base, slope;
+};
+static FitD fit_partners(const std::vector<unsigned long long> &rec, int col, int64_t stride, int64_t n, bool upper) {
+    double ll = 0, lx = 0, xx = 0, ly = 0, xy = 0;
+    const int64_t nb = (int64_t)rec.size() / 3;
+    for (int64_t b = 0; b < nb; b++) {
+        const double L = (double)rec[3 * b], y = (double)rec[3 * b + col];
+        const double x = upper ? 1.0 - (double)(b * stride) / (double)n : 0.0;
+        ll += L * L;
+        lx += L * L * x;
+        xx += L * L * x * x;
+        ly += L * y;
+        xy += L * x * y;
+    }
+    const double det = ll * xx - lx * lx;
+    FitD f{ll > 0 ? ly / ll : 0.0, 0.0};
+    if (upper && det > 1e-9 * ll * ll) {
+        const double base = (ly * xx - xy * lx) / det, slope = (xy * ll - ly * lx) / det;
+        if (base < 0 && xx > 0) f = FitD{0.0, xy / xx};
+        else if (slope >= 0) f = FitD{base, slope};
+    }
+    return f;
 }
 
 // C from the upper triangle U (rows at tmp_off, lengths nnz_row, seeds slot-major with stride
@@ -1372,7 +1690,9 @@ static int pick_numeric_threads(int log2T, bool filtered) {
 // slots and more, spgemm_tab_warps_big
 // tsm = the table's (and filters') shared memory, warp_bytes = each warp's record buffer; code =
 // log2T, negated for unfiltered tables (for the fixed choice when spgemm_tab_warps is 0)
-static int pick_tab_threads(size_t tsm, size_t warp_bytes, int code) {
+// least: at least this many threads: rows of small tables may have many entries, and a launch of few
+// such rows lasts as long as one of them (64 threads at least: 5 Mbp at 30x 2.15 ms a call, 256: 1.75)
+static int pick_tab_threads(size_t tsm, size_t warp_bytes, int code, int64_t least) {
     const int log2T = code < 0 ? -code : code;
     int64_t want = tune("spgemm_tab_warps");
     if (want <= 0) return pick_numeric_threads(log2T, code > 0);
@@ -1381,7 +1701,7 @@ static int pick_tab_threads(size_t tsm, size_t warp_bytes, int code) {
     for (;;) {
         const size_t bytes = tsm + warp_bytes * (size_t)(threads / 32);
         const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(32, (int64_t)((227u << 10) / bytes)));
-        if (threads >= 1024 || blocks * (threads / 32) >= want) break;
+        if (threads >= 1024 || (threads >= least && blocks * (threads / 32) >= want)) break;
         threads <<= 1;
     }
     return (int)threads;
@@ -1450,14 +1770,18 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
         num.ncls++;
     }
     // the fused pass's guessed tables (up to 220 KB with the record buffers of 1024 threads: one
-    // block per SM)
+    // block per SM): compact for max_seeds <= 2
     const size_t tab_limit = (220u << 10) - wbb(1024);
-    Classes fz{};
-    fz.ncls = 0;
-    while (fz.ncls < SP_NCLS && tab_bytes((int64_t)1 << (SP_MINLOG + fz.ncls), S) <= tab_limit) {
-        fz.log2T[fz.ncls] = SP_MINLOG + fz.ncls;
-        fz.ncls++;
-    }
+    const bool compact = S <= 2;
+    int oblog = 1;  // compact: T >> oblog partners of a table can be kept
+    auto class_ob = [&](int log2T) {  // fewer where the table would not fit otherwise
+        int ob = oblog;
+        while (ob < 3 && ctab_bytes((int64_t)1 << log2T, S, ob) > tab_limit) ob++;
+        return ob;
+    };
+    auto fz_bytes = [&](int log2T) {
+        return compact ? ctab_bytes((int64_t)1 << log2T, S, class_ob(log2T)) : tab_bytes((int64_t)1 << log2T, S);
+    };
     // filtered rows (fused path): two filters of 2^log2F bits, one bit per read while np fits
     int log2F = 10;
     while (log2F < (int)tune("spgemm_filter_log2") && ((int64_t)1 << log2F) < np) log2F++;
@@ -1487,53 +1811,76 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
         unsigned long long *n_retry = counts + 4 * NCNT + 2;  // rows that found the region full
         unsigned long long *gw = counts + 4 * NCNT + 3;       // {largest w, room} of listed rows (2)
         unsigned long long *big_count = counts + 4 * NCNT + 5;  // long mirrored parts
-        unsigned long long *sums = counts + 4 * NCNT + 6;     // sample sums (3)
+        unsigned long long *sums = counts + 4 * NCNT + 6;     // kept partners, by the fit
         // sampled rows: distinct partners (r1) and partners seen at least twice (r2) per A entry
         const int64_t fmode = tune("spgemm_filter_mode");
         int64_t fwork = min_shared >= 2 && ff.ncls > 0 && fmode > 0 ? tune("spgemm_filter_work") : 0;
         double r1 = 0.0, r2 = 0.0;
+        FitD f1{1.0, 0.0}, f2{1.0, 0.0};  // no sample: a partner per A entry
         const int64_t nsamp = tune("spgemm_sample_rows");
         if (nsamp > 0 && n > 0 && A->nnz > 0) {
             const int64_t stride = n > nsamp ? n / nsamp : 1;
             const int64_t nb = (n + stride - 1) / stride;
             const size_t ssm = fbytes + wbb(256);
+            unsigned long long *rec = sc.get<unsigned long long>(3 * (size_t)nb);
+            if (!rec) return SG_ERR_OOM;
             if (upper) {
                 SG_CUDA_TRY(ensure_smem(sample_fx_kernel<true>, ssm));
-                SG_LAUNCH("spgemm_sample", sample_fx_kernel<true>, nb, 256, ssm, s, g, stride, log2F, sums);
+                SG_LAUNCH("spgemm_sample", sample_fx_kernel<true>, nb, 256, ssm, s, g, stride, log2F, rec);
             } else {
                 SG_CUDA_TRY(ensure_smem(sample_fx_kernel<false>, ssm));
-                SG_LAUNCH("spgemm_sample", sample_fx_kernel<false>, nb, 256, ssm, s, g, stride, log2F, sums);
+                SG_LAUNCH("spgemm_sample", sample_fx_kernel<false>, nb, 256, ssm, s, g, stride, log2F, rec);
             }
-            unsigned long long h[3] = {0, 0, 0};
-            SG_CUDA_TRY(read_back(h, sums, sizeof(h), s));
-            if (h[0] > 0) {
-                r1 = (double)h[1] / (double)h[0];
-                r2 = (double)h[2] / (double)h[0];
+            std::vector<unsigned long long> h(3 * (size_t)nb);
+            SG_CUDA_TRY(read_back(h.data(), rec, h.size() * 8, s));
+            double h0 = 0, h1 = 0, h2 = 0;
+            for (int64_t b = 0; b < nb; b++) {
+                h0 += (double)h[3 * b];
+                h1 += (double)h[3 * b + 1];
+                h2 += (double)h[3 * b + 2];
+            }
+            if (h0 > 0 && h1 > 0) {
+                r1 = h1 / h0;
+                r2 = h2 / h0;
+                f1 = fit_partners(h, 1, stride, n, upper);
+                f2 = fit_partners(h, 2, stride, n, upper);
             }
         }
         if (r1 == 0.0) r1 = r2 = 1.0;  // no sample: a partner per A entry
+        // kept partners of a full table (3/4 T), and a tenth
+        const double kept_share = 0.75 * 1.1 * (min_shared >= 2 ? r2 / r1 : 1.0);
+        oblog = kept_share <= 0.125 ? 3 : (kept_share <= 0.25 ? 2 : 1);
+        Classes fz{};
+        while (fz.ncls < SP_NCLS && fz_bytes(SP_MINLOG + fz.ncls) <= tab_limit) {
+            fz.log2T[fz.ncls] = SP_MINLOG + fz.ncls;
+            fz.ncls++;
+        }
         const bool recur = r1 < 2.0 * r2;  // most partners recur: the filter would keep nearly all
         if (fmode == 1 && recur) fwork = 0;
         const double pct = (double)tune("spgemm_guess_pct") / 100.0;
-        const uint64_t fu = (uint64_t)(pct * r1 * 65536.0) + 1, ffq = (uint64_t)(pct * r2 * 65536.0) + 1;
-        SG_LAUNCH("fused_need", fx_need_kernel, blocks_for(n, NT), NT, 0, s, A->row_ptr, n, fu, fwork, ffq,
-                  ff.ncls > 0 ? (int64_t)1 << ff.log2T[ff.ncls - 1] : (int64_t)64, Tmax, need, need_f);
+        auto fixed = [](const FitD &f, double by) {
+            return PartnerFit{(uint64_t)(by * f.base * 65536.0) + 1, (uint64_t)(by * f.slope * 65536.0)};
+        };
+        const uint64_t ffq = (uint64_t)(pct * r2 * 65536.0) + 1;
+        SG_LAUNCH("fused_need", fx_need_kernel, blocks_for(n, NT), NT, 0, s, A->row_ptr, n, fixed(f1, pct),
+                  fixed(min_shared >= 2 ? f2 : f1, 1.0), fwork, ffq,
+                  ff.ncls > 0 ? (int64_t)1 << ff.log2T[ff.ncls - 1] : (int64_t)64, Tmax,
+                  compact ? (int64_t)CT_ROW : (int64_t)1 << 40, need, need_f, sums);
         SG_LAUNCH("classify", classify_kernel, blocks_for(n, NT), NT, 0, s, need, n, fz, fz_counts, lists);
         if (fwork)
             SG_LAUNCH("classify", classify_kernel, blocks_for(n, NT), NT, 0, s, need_f, n, ff, ff_counts, lists_f);
-        unsigned long long h_fz[NCNT], h_ff[NCNT];
+        unsigned long long h_fz[NCNT], h_ff[NCNT], h_kept = 0;
         uint32_t herr = 0;
         SG_CUDA_TRY(cudaMemcpyAsync(h_ff, ff_counts, sizeof(h_ff), cudaMemcpyDeviceToHost, s));
         SG_CUDA_TRY(cudaMemcpyAsync(h_fz, fz_counts, sizeof(h_fz), cudaMemcpyDeviceToHost, s));
+        SG_CUDA_TRY(cudaMemcpyAsync(&h_kept, sums, sizeof(h_kept), cudaMemcpyDeviceToHost, s));
         SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));
         if (herr & DEV_TIMEOUT) return timeout_error("overlap_spgemm");
-        // the temporary region: the sampled kept partners per A entry (r2 for min_shared >= 2, r1
-        // for 1) times nnz(A), with room to spare; rows that find it full are redone in a grown one
+        // the temporary region: the kept partners fitted to the sample (at least twice for
+        // min_shared >= 2), with room to spare; rows that find it full are redone in a grown one
         int64_t cap = opt.tmp_cap;
-        if (cap <= 0) {
-            const double kept = (min_shared >= 2 ? r2 : r1) * (double)A->nnz + 4.0 * (double)n;
-            cap = (int64_t)((double)tune("spgemm_tmp_pct") / 100.0 * kept) + 64;
-        }
+        if (cap <= 0)
+            cap = (int64_t)((double)tune("spgemm_tmp_pct") / 100.0 * ((double)h_kept + 4.0 * (double)n)) + 64;
         const double tmp_bytes = (double)cap * (8.0 + 8.0 * S);
         // at most half of what the device can still give (a row range was sized for its budget)
         const double avail = (double)device_bytes_available();
@@ -1552,12 +1899,14 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             o.retry = retry;
             o.n_retry = n_retry;
             o.colcnt = colcnt;
+            int64_t least = 64;  // about four entries of a mean row per thread
+            while (least < 256 && 4 * least < A->nnz / (n > 0 ? n : 1)) least <<= 1;
             // one launch per table class; the seed form (SK), the filter and the form pick the kernel
             const int carve = (int)tune("spgemm_smem_carveout");
             auto launch_tab = [&](bool filt, int log2T, const int32_t *rl, const unsigned long long *cnt,
                                   const char *name, int32_t *ol, unsigned long long *oc, int8_t *olt) -> sg_status {
-                const size_t tsm = tab_bytes((int64_t)1 << log2T, S) + (filt ? fbytes : 0);
-                const int nt = pick_tab_threads(tsm, wbb(32), filt ? log2T : -log2T);
+                const size_t tsm = filt ? tab_bytes((int64_t)1 << log2T, S) + fbytes : fz_bytes(log2T);
+                const int nt = pick_tab_threads(tsm, wbb(32), filt ? log2T : -log2T, least);
                 const size_t sm = tsm + wbb(nt);
                 const int64_t wb_off = (int64_t)tsm;
 #define SG_TAB_LAUNCH(SKV, FV, UV)                                                                          \
@@ -1578,8 +1927,23 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
     } while (0)
                 if (filt && upper) SG_TAB_SK(true, true);
                 else if (filt) SG_TAB_SK(true, false);
-                else if (upper) SG_TAB_SK(false, true);
-                else SG_TAB_SK(false, false);
+                else if (!compact && upper) SG_TAB_LAUNCH(3, false, true);
+                else if (!compact) SG_TAB_LAUNCH(3, false, false);
+                else {
+                    auto run = [&](auto kern) -> sg_status {
+                        SG_CUDA_TRY(ensure_smem(kern, sm));
+                        if (carve >= 0)
+                            SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
+                        SG_LAUNCH(name, kern, grid, nt, sm, s, g, rl, cnt, log2T, class_ob(log2T), o, ol, oc, wb_off, olt);
+                        return SG_OK;
+                    };
+                    if (upper)
+                        SG_TRY(SK == 0 ? run(ctab_numeric_kernel<0, true>)
+                                       : (SK == 1 ? run(ctab_numeric_kernel<1, true>) : run(ctab_numeric_kernel<2, true>)));
+                    else
+                        SG_TRY(SK == 0 ? run(ctab_numeric_kernel<0, false>)
+                                       : (SK == 1 ? run(ctab_numeric_kernel<1, false>) : run(ctab_numeric_kernel<2, false>)));
+                }
 #undef SG_TAB_SK
 #undef SG_TAB_LAUNCH
                 return SG_OK;
