@@ -90,6 +90,7 @@ struct KbPlan {
     uint32_t *sb;                 // [nb1 + 1] first bucket of each prefix; sb[nb1] = buckets
     uint32_t *chunk2;             // [nb1 + 1] first level-2 chunk of each prefix
     uint16_t *sub2p;              // [buckets] prefix of each bucket
+    uint16_t *chunk2p;            // [chunks] prefix of each chunk
     int64_t *start2;              // [nsub_max + 1] first record of each bucket (two == 0: start1)
     unsigned long long *cur2;     // [nsub_max] write cursors of the second pass
     uint32_t *count2;             // [nsub_max + 1]
@@ -114,12 +115,16 @@ inline size_t scatter_smem_bytes(int nb) {
 // The second half of a grouping pass, on records held in registers: br[u] = bin << 16 | rank in
 // the bin within the tile, or 0xFFFFFFFF for no record; cnt[] holds the tile's counts. Orders the
 // tile by bin in shared memory and writes every bin's run at a place reserved on cur[bin]
-// (positions are absolute). binof(key) recovers a record's bin unless BINARR keeps it.
-template <class K, bool BINARR, class BinOf>
+// (positions are absolute). binof(key) recovers a record's bin unless BINARR keeps it; then() runs
+// once the records are in shared memory.
+struct NoOp {
+    __device__ void operator()() const {}
+};
+template <class K, bool BINARR, class BinOf, class Then = NoOp>
 __device__ __forceinline__ void scatter_tail(ScatterSmem<K> &sm, uint32_t *cnt, unsigned long long *gb,
-                                             uint16_t *sbin, int nb, const typename K::T (&key)[K::ITEMS],
+                                             uint16_t *sbin, int nb, typename K::T (&key)[K::ITEMS],
                                              const uint32_t (&br)[K::ITEMS], unsigned long long *__restrict__ cur,
-                                             typename K::T *__restrict__ out, int64_t cap, BinOf &&binof) {
+                                             typename K::T *__restrict__ out, int64_t cap, BinOf &&binof, Then &&then = NoOp{}) {
     constexpr int PER = KB_MAXBINS / KB_NT;  // bins t, t + KB_NT, ... belong to thread t
     __syncthreads();
     // runs are reserved first: the atomics travel while the tile is scanned and ordered
@@ -155,6 +160,7 @@ __device__ __forceinline__ void scatter_tail(ScatterSmem<K> &sm, uint32_t *cnt, 
         const int b = x * KB_NT + threadIdx.x;
         if (b < nb) gb[b] = g[x] - cnt[b];
     }
+    then();  // the registers are free
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < ntot; i += KB_NT) {
         const typename K::T k = sm.tile[i];
@@ -174,16 +180,6 @@ __device__ __forceinline__ void scatter_layout(unsigned char *raw, int nb, Scatt
     sbin = reinterpret_cast<uint16_t *>(p + (size_t)nb * 12);
 }
 
-// Last index i in [0, n) with a[i] <= x (a ascending, a[0] <= x).
-__device__ __forceinline__ int last_le(const uint32_t *__restrict__ a, int n, uint32_t x) {
-    int lo = 0, hi = n;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (a[mid] <= x) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 // One block per plan: prefix counts -> record ranges, level-2 split, buckets and chunks.
 // b2max bounds the split (0: one level). minb2: at least this many bits (rows per bucket bound).
 __global__ void __launch_bounds__(1024) kb_plan_kernel(const unsigned long long *__restrict__ hist, KbPlan pl,
@@ -194,13 +190,10 @@ template <class K>
 __global__ void __launch_bounds__(KB_NT) kb_hist2_kernel(KbPlan pl, const typename K::T *__restrict__ in,
                                                         int lowbits) {
     __shared__ uint32_t cnt[KB_MAXBINS];
-    __shared__ int s_p;
-    if (threadIdx.x == 0)
-        s_p = blockIdx.x < pl.chunk2[pl.nb1] ? last_le(pl.chunk2, pl.nb1, blockIdx.x) : -1;
+    if (blockIdx.x >= pl.chunk2[pl.nb1]) return;
+    const int p = pl.chunk2p[blockIdx.x];
     for (int i = threadIdx.x; i < KB_MAXBINS; i += KB_NT) cnt[i] = 0;
     __syncthreads();
-    const int p = s_p;
-    if (p < 0) return;
     const int b = pl.b2[p], sh = pl.rem - b;
     const int64_t c0 = pl.start1[p], c1 = pl.start1[p + 1];
     constexpr int64_t CH = (int64_t)KB_CHUNK_TILES * kb_tile<K>();
@@ -221,48 +214,53 @@ __global__ void __launch_bounds__(KB_NT) kb_hist2_kernel(KbPlan pl, const typena
         if (cnt[i]) atomicAdd(pl.count2 + pl.sb[p] + i, cnt[i]);
 }
 
-// Level-2 grouping: a tile of one prefix's records per block.
+// Level-2 grouping: a chunk of one prefix's records per block, tile by tile; the next tile's loads
+// travel while this one is written. 4.1e9 records of 8 bytes (100 Mbp, 40x): 18.6 ms, 3.5 TB/s;
+// one tile per block, its prefix searched for by one thread first, 21.7 ms.
 template <class K>
 __global__ void __launch_bounds__(KB_NT, 2) kb_scatter2_kernel(KbPlan pl, const typename K::T *__restrict__ in,
                                                               typename K::T *__restrict__ out, int lowbits) {
     extern __shared__ __align__(16) unsigned char kb_raw[];
-    __shared__ int s_p;
-    const uint32_t chunk = blockIdx.x / KB_CHUNK_TILES;
-    if (threadIdx.x == 0) s_p = chunk < pl.chunk2[pl.nb1] ? last_le(pl.chunk2, pl.nb1, chunk) : -1;
-    __syncthreads();
-    const int p = s_p;
-    if (p < 0) return;
+    const uint32_t chunk = blockIdx.x;
+    if (chunk >= pl.chunk2[pl.nb1]) return;
+    const int p = pl.chunk2p[chunk];
     constexpr int TILE = kb_tile<K>();
-    const int64_t a0 = pl.start1[p] +
-                       ((int64_t)(chunk - pl.chunk2[p]) * KB_CHUNK_TILES + blockIdx.x % KB_CHUNK_TILES) * TILE;
-    const int64_t a1 = pl.start1[p + 1];
-    if (a0 >= a1) return;
+    const int64_t a0 = pl.start1[p] + (int64_t)(chunk - pl.chunk2[p]) * KB_CHUNK_TILES * TILE;
+    const int64_t end = pl.start1[p + 1];
+    const int64_t a1 = a0 + KB_CHUNK_TILES * TILE < end ? a0 + KB_CHUNK_TILES * TILE : end;
     const int b = pl.b2[p], sh = pl.rem - b, nb = 1 << b;
     ScatterSmem<K> *sm;
     uint32_t *cnt;
     unsigned long long *gb;
     uint16_t *sbin;
     scatter_layout<K>(kb_raw, nb, sm, cnt, gb, sbin);
-    for (int i = threadIdx.x; i < nb; i += KB_NT) cnt[i] = 0;
     typename K::T key[K::ITEMS];
-    uint32_t br[K::ITEMS];
+    auto load = [&](int64_t t0) {
 #pragma unroll
-    for (int u = 0; u < K::ITEMS; u++) {
-        const int64_t i = a0 + u * KB_NT + threadIdx.x;
-        key[u] = i < a1 ? K::load(in + i) : K::none();
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < K::ITEMS; u++) {
-        const int64_t i = a0 + u * KB_NT + threadIdx.x;
-        br[u] = 0xFFFFFFFFu;
-        if (i < a1) {
-            const uint32_t s = K::slot(key[u], 0ull, lowbits, sh);
-            if (SG_IN_BOUNDS(s < (uint32_t)nb, 707, s)) br[u] = (s << 16) | atomicAdd(cnt + s, 1u);
+        for (int u = 0; u < K::ITEMS; u++) {
+            const int64_t i = t0 + u * KB_NT + threadIdx.x;
+            key[u] = i < a1 ? K::load(in + i) : K::none();
         }
+    };
+    load(a0);
+    for (int64_t t0 = a0; t0 < a1; t0 += TILE) {
+        for (int i = threadIdx.x; i < nb; i += KB_NT) cnt[i] = 0;
+        __syncthreads();
+        uint32_t br[K::ITEMS];
+#pragma unroll
+        for (int u = 0; u < K::ITEMS; u++) {
+            const int64_t i = t0 + u * KB_NT + threadIdx.x;
+            br[u] = 0xFFFFFFFFu;
+            if (i < a1) {
+                const uint32_t s = K::slot(key[u], 0ull, lowbits, sh);
+                if (SG_IN_BOUNDS(s < (uint32_t)nb, 707, s)) br[u] = (s << 16) | atomicAdd(cnt + s, 1u);
+            }
+        }
+        scatter_tail<K, false>(*sm, cnt, gb, nullptr, nb, key, br, pl.cur2 + pl.sb[p], out, pl.cap,
+                               [&](const typename K::T &k) { return K::slot(k, 0ull, lowbits, sh); },
+                               [&] { if (t0 + TILE < a1) load(t0 + TILE); });
+        __syncthreads();
     }
-    scatter_tail<K, false>(*sm, cnt, gb, nullptr, nb, key, br, pl.cur2 + pl.sb[p], out, pl.cap,
-                           [&](const typename K::T &k) { return K::slot(k, 0ull, lowbits, sh); });
 }
 
 // ----------------------------------------------------------------------------- finishing

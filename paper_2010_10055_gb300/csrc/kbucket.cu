@@ -75,12 +75,13 @@ __global__ void __launch_bounds__(1024) kb_plan_kernel(const unsigned long long 
     }
 }
 
-// sub2p[b] = the prefix of bucket b: one warp per prefix.
+// The prefixes of the buckets and of the chunks: one warp per prefix.
 __global__ void kb_sub2p_kernel(KbPlan pl) {
     const int p = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (p >= pl.nb1) return;
     for (uint32_t x = pl.sb[p] + (threadIdx.x & 31); x < pl.sb[p + 1]; x += 32)
         if (SG_IN_BOUNDS((int64_t)x < pl.nsub_max, 701, x)) pl.sub2p[x] = (uint16_t)p;
+    for (uint32_t x = pl.chunk2[p] + (threadIdx.x & 31); x < pl.chunk2[p + 1]; x += 32) pl.chunk2p[x] = (uint16_t)p;
 }
 
 // ----------------------------------------------------------------------------------- pack
@@ -952,7 +953,8 @@ static int bits_for(int64_t n) {  // bits of the ids 0 .. n - 1
 
 // A plan for `records` records with code bits `cb` above the prefix's end: prefix bits, whether a
 // second level is needed, and the device arrays (one allocation).
-static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t records, int target, int b2min, Scratch &sc) {
+static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t records, int tile, int target, int b2min,
+                           Scratch &sc) {
     pl.nb1 = 1 << pb1;
     pl.rem = cb - pb1;
     pl.two = two ? 1 : 0;
@@ -960,8 +962,9 @@ static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t record
     // a prefix of c records splits into fewer than 2 c / target + 1 buckets (2^b2min at least)
     pl.nsub_max = two ? ((int64_t)pl.nb1 << b2min) + 2 * (records / target + 1) : pl.nb1;
     const size_t nb = (size_t)pl.nb1, ns = two ? (size_t)pl.nsub_max : 0;
+    const size_t nc = two ? (size_t)(records / (KB_CHUNK_TILES * (int64_t)tile) + pl.nb1) : 0;  // a partial chunk per prefix
     const size_t words = (nb + 1) + nb + (ns + 1) + ns;  // 8-byte arrays
-    uint64_t *w = sc.get<uint64_t>(words + ((nb + 1) * 2 * 4 + (ns + 1) * 4 + ns * 2 + nb + 64) / 8);
+    uint64_t *w = sc.get<uint64_t>(words + ((nb + 1) * 2 * 4 + (ns + 1) * 4 + (ns + nc) * 2 + nb + 64) / 8);
     if (!w) return SG_ERR_OOM;
     pl.start1 = (int64_t *)w;
     pl.cur1 = (unsigned long long *)(w + nb + 1);
@@ -971,7 +974,8 @@ static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t record
     pl.chunk2 = pl.sb + nb + 1;
     pl.count2 = pl.chunk2 + nb + 1;
     pl.sub2p = (uint16_t *)(pl.count2 + ns + 1);
-    pl.b2 = (uint8_t *)(pl.sub2p + ns);
+    pl.chunk2p = pl.sub2p + ns;
+    pl.b2 = (uint8_t *)(pl.chunk2p + nc);
     return SG_OK;
 }
 
@@ -988,7 +992,7 @@ static sg_status second_level(KbPlan &pl, const typename K::T *in, typename K::T
     SG_CUDA_TRY(cudaMemcpyAsync(pl.cur2, pl.start2, (size_t)pl.nsub_max * 8, cudaMemcpyDeviceToDevice, s));
     const size_t sm = scatter_smem_bytes<K, false>(KB_MAXBINS);
     SG_CUDA_TRY(ensure_smem(kb_scatter2_kernel<K>, sm));
-    SG_LAUNCH(sname, kb_scatter2_kernel<K>, nch * KB_CHUNK_TILES, KB_NT, sm, s, pl, in, out, lowbits);
+    SG_LAUNCH(sname, kb_scatter2_kernel<K>, nch, KB_NT, sm, s, pl, in, out, lowbits);
     return SG_OK;
 }
 
@@ -1016,7 +1020,7 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     // rows of one bucket: at most 2^12, a slot each
     const int rest = rbits - pb1, b2min = two && rest > 12 ? rest - 12 : 0;
     KbPlan pl;
-    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, kb_target<K>(), b2min, sc));
+    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, kb_target<K>(), b2min, sc));
     const int64_t ntiles = blocks_for(nnz, TILE);
     int32_t *tcol = sc.get<int32_t>(ntiles);
     typename K::T *r0 = sc.get<typename K::T>(nnz), *r1 = two ? sc.get<typename K::T>(nnz) : nullptr;
@@ -1089,7 +1093,7 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
     using T = typename K::T;
     constexpr int TILE = kb_tile<K>();
     KbPlan pl;
-    SG_TRY(make_plan(pl, q.pb1, q.cb, q.two, q.total, kb_target<K>(), 0, sc));
+    SG_TRY(make_plan(pl, q.pb1, q.cb, q.two, q.total, TILE, kb_target<K>(), 0, sc));
     SG_LAUNCH("kmer_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, kb_target<K>(),
               q.two ? std::min(KB_MAXB2, pl.rem) : 0, 0, KB_CHUNK_TILES * TILE);
     T *r0 = sc.get<T>(q.total), *r1 = sc.get<T>(q.total);
