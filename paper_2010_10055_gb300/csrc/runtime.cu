@@ -335,7 +335,7 @@ static Tunable g_tunables[] = {
                                           // may first mark partners seen twice (0: never)
     {"spgemm_filter_log2", 17, 10, 19},   // at most 2^this bits per seen-once / seen-twice filter
     {"sym_guess_shift", 2, 0, 8},         // symbolic table guess = products >> shift
-    {"spgemm_blocks_per_sm", 64, 1, 64},  // grid of each SpGEMM class launch
+    {"spgemm_blocks_per_sm", 256, 1, 1024},  // grid of each SpGEMM class launch
     {"spgemm_big_threads", 1024, 512, 1024},  // threads of numeric blocks with 4 K table slots or more
     {"tr_blocks_per_sm", 32, 1, 64},      // grid of the min-plus launch
     {"tr_warp_rows", 1, 0, 1},            // 1: rows of up to 128 entries reduced by a warp each; 0: by blocks

@@ -1007,7 +1007,8 @@ __global__ void SG_TAB_BOUNDS tab_numeric_kernel(SpArgs g, const int32_t *__rest
 // counted once per warp step. Kept partners are ordered by counting into as many bins as there are
 // partners between the smallest and the largest (bitonic only where a bin gets crowded). The pass
 // stays bound by the gathers (random At records, about 40 G sectors per second) and their latency.
-// With the fitted table sizes, one call: 5 Mbp at 30x 2.26 -> 1.79 ms, 25 Mbp at 40x 14.4 -> 12.3 ms.
+// With the fitted table sizes, one call: 5 Mbp at 30x 2.26 -> 1.79 ms, 25 Mbp at 40x 14.4 -> 12.3 ms
+// (a launch per class).
 constexpr int CT_ROW = 65535;   // A entries of a row
 constexpr int CT_CROWD = 48;    // partners of one bin ranked against each other
 constexpr uint32_t CT_FREE = 0xFFFFFFFFu;
@@ -1017,11 +1018,18 @@ __host__ __device__ inline size_t ctab_bytes(int64_t T, int S, int oblog) {
     return (size_t)T * (S > 0 ? 10 : 6) + (size_t)(T >> oblog) * 8;
 }
 
+// The table classes of one launch, largest first: their row lists, one after the other.
+struct TabGroup {
+    int nc, shift;  // shift: log2 of the growth of a table that was too small (0: no second try here)
+    int lT[SP_NCLS], ob[SP_NCLS];
+    uint32_t cnt[SP_NCLS];
+    const int32_t *rows[SP_NCLS];
+};
+
 // 32 registers: 64 warps per SM, which the gathers' latency wants (25 Mbp at 40x: 12.3 ms a call; 40
 // registers and 48 warps: 13.2 ms).
 template <int SK, bool UPPER>
-__global__ void __maxnreg__(32) ctab_numeric_kernel(SpArgs g, const int32_t *__restrict__ rows,
-                                                  const unsigned long long *__restrict__ nrows_p, int lT, int oblog,
+__global__ void __maxnreg__(32) ctab_numeric_kernel(SpArgs g, const __grid_constant__ TabGroup tg, uint32_t nrows,
                                                   TmpOut o, int32_t *__restrict__ ovf_list,
                                                   unsigned long long *__restrict__ ovf_count, int64_t wb_off,
                                                   int8_t *__restrict__ ovf_lt) {
@@ -1029,21 +1037,31 @@ __global__ void __maxnreg__(32) ctab_numeric_kernel(SpArgs g, const int32_t *__r
     __shared__ int s_ctr, s_ins, s_ovf, s_full, s_fail, s_crowd;
     __shared__ uint32_t s_lo, s_hi, s_w[33];
     __shared__ unsigned long long s_e0;
-    const int T = 1 << lT, OB = T >> oblog, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     uint32_t *key = reinterpret_cast<uint32_t *>(tab_raw);
-    uint32_t *sd = key + T;
-    uint32_t *cnt2 = sd + (SK > 0 ? T : 0);
-    uint32_t *bins = cnt2 + T / 2;
-    uint16_t *la = reinterpret_cast<uint16_t *>(bins + OB), *lb = la + OB;
     int32_t *wb = g.t_rec ? (int32_t *)(tab_raw + wb_off) : nullptr;  // record reads, per warp
-    const uint32_t msk = (uint32_t)T - 1u;
-    const int cap = (T >> 1) + (T >> 2);
-    const int64_t nrows = (int64_t)*nrows_p;
-    auto count_of = [&](uint32_t x) { return (cnt2[x >> 1] >> (16 * (x & 1u))) & 0xffffu; };
-    for (int64_t rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int32_t i = rows[rb];
+    int c = 0;
+    uint32_t again = 0;  // 1: the row once more, in the larger table of class c
+    for (uint32_t rb = blockIdx.x; rb < nrows; rb += again ? 0u : gridDim.x) {
+        uint32_t cq = rb;
+        {
+            int x = 0;
+            while (x + 1 < tg.nc && cq >= tg.cnt[x]) cq -= tg.cnt[x++];
+            if (!again) c = x;
+            cq = (uint32_t)tg.rows[x][cq];
+        }
+        again = 0;
+        const int32_t i = (int32_t)cq;
         if (!SG_IN_BOUNDS(i >= 0 && i < g.n, 308, i)) continue;
         const int32_t gi = (int32_t)(g.row0 + i);
+        const int lT = tg.lT[c], T = 1 << lT, OB = T >> tg.ob[c];
+        uint32_t *sd = key + T;
+        uint32_t *cnt2 = sd + (SK > 0 ? T : 0);
+        uint32_t *bins = cnt2 + T / 2;
+        uint16_t *la = reinterpret_cast<uint16_t *>(bins + OB), *lb = la + OB;
+        const uint32_t msk = (uint32_t)T - 1u;
+        const int cap = (T >> 1) + (T >> 2);
+        auto count_of = [&](uint32_t x) { return (cnt2[x >> 1] >> (16 * (x & 1u))) & 0xffffu; };
         const uint4 ones = make_uint4(CT_FREE, CT_FREE, CT_FREE, CT_FREE);
         for (int x = tid; x < (SK > 0 ? T / 2 : T / 4); x += nt) reinterpret_cast<uint4 *>(key)[x] = ones;
         for (int x = tid; x < T / 8; x += nt) reinterpret_cast<uint4 *>(cnt2)[x] = make_uint4(0, 0, 0, 0);
@@ -1116,8 +1134,12 @@ __global__ void __maxnreg__(32) ctab_numeric_kernel(SpArgs g, const int32_t *__r
             }
         }
         __syncthreads();
-        if (s_ovf || s_full) {  // redone in a larger table
-            if (tid == 0) {
+        if (s_ovf || s_full) {  // redone in a larger table: here, where this launch has one
+            again = tg.shift > 0 && c > 0;
+            if (again) {
+                const int want = lT + tg.shift;
+                while (c > 0 && tg.lT[c] < want) c--;
+            } else if (tid == 0) {
                 const unsigned long long q = atomicAdd(ovf_count, 1ull);
                 if (SG_IN_BOUNDS((int64_t)q < g.n, 311, q)) {
                     ovf_list[q] = i;
@@ -1903,6 +1925,73 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             while (least < 256 && 4 * least < A->nnz / (n > 0 ? n : 1)) least <<= 1;
             // one launch per table class; the seed form (SK), the filter and the form pick the kernel
             const int carve = (int)tune("spgemm_smem_carveout");
+            // Classes that run with the same threads share a launch, largest tables first, so that one
+            // tail is waited for instead of one per class and a table that turns out too small is
+            // redone in place. They share the largest one's shared memory, so a class joins only
+            // where that keeps its blocks per SM and leaves L1 (8 K tables in the 16 K launch at 100
+            // Mbp: 58 -> 78 ms), or where all rows are within one wave. A launch per class and a
+            // second one for its overflows: 5 Mbp at 30x 1.78 ms a call, 25 Mbp at 40x 12.3; now
+            // 1.33 and 11.8.
+            auto launch_group = [&](const int32_t *ls, const unsigned long long *h_cnt, int32_t *ol,
+                                    unsigned long long *oc, int8_t *olt) -> sg_status {
+                struct Shape {
+                    int threads;
+                    int64_t blocks;  // on an SM
+                    bool small;      // their shared memory leaves the L1 cache some
+                };
+                auto shape = [&](int cl) {
+                    const size_t bytes = fz_bytes(fz.log2T[cl]);
+                    const int nt = pick_tab_threads(bytes, wbb(32), -fz.log2T[cl], least);
+                    const size_t one = bytes + wbb(nt) + 1024;
+                    const int64_t blocks =
+                        std::max<int64_t>(1, std::min<int64_t>(64 / (nt / 32), (int64_t)((228u << 10) / one)));
+                    return Shape{nt, blocks, (size_t)blocks * one <= (176u << 10)};
+                };
+                for (int c1 = fz.ncls - 1; c1 >= 0;) {
+                    const Shape lead = shape(c1);
+                    if (!h_cnt[c1] && !lead.small) {
+                        c1--;
+                        continue;
+                    }
+                    const int nt = lead.threads;
+                    TabGroup tg{};
+                    tg.shift = (int)tune("spgemm_escalate");
+                    size_t tsm = 0;
+                    uint64_t nrows = 0;
+                    for (; c1 >= 0; c1--) {
+                        const Shape sh = shape(c1);
+                        if (sh.threads != nt) break;
+                        if (tg.nc > 0 && !(lead.small && sh.blocks == lead.blocks) &&
+                            (int64_t)(nrows + h_cnt[c1]) > lead.blocks * nsm)
+                            break;
+                        const int q = tg.nc++;
+                        tg.lT[q] = fz.log2T[c1];
+                        tg.ob[q] = class_ob(fz.log2T[c1]);
+                        tg.cnt[q] = (uint32_t)h_cnt[c1];
+                        tg.rows[q] = ls + (int64_t)c1 * n;
+                        tsm = std::max(tsm, fz_bytes(fz.log2T[c1]));
+                        nrows += h_cnt[c1];
+                    }
+                    if (nrows == 0) continue;
+                    auto run = [&](auto kern) -> sg_status {
+                        const size_t sm = tsm + wbb(nt);
+                        SG_CUDA_TRY(ensure_smem(kern, sm));
+                        if (carve >= 0)
+                            SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
+                        const int64_t blocks = std::min<int64_t>((int64_t)nrows, grid);
+                        SG_LAUNCH(NUM_NAMES[tg.lT[0] - SP_MINLOG], kern, blocks, nt, sm, s, g, tg, (uint32_t)nrows, o, ol, oc,
+                                  (int64_t)tsm, olt);
+                        return SG_OK;
+                    };
+                    if (upper)
+                        SG_TRY(SK == 0 ? run(ctab_numeric_kernel<0, true>)
+                                       : (SK == 1 ? run(ctab_numeric_kernel<1, true>) : run(ctab_numeric_kernel<2, true>)));
+                    else
+                        SG_TRY(SK == 0 ? run(ctab_numeric_kernel<0, false>)
+                                       : (SK == 1 ? run(ctab_numeric_kernel<1, false>) : run(ctab_numeric_kernel<2, false>)));
+                }
+                return SG_OK;
+            };
             auto launch_tab = [&](bool filt, int log2T, const int32_t *rl, const unsigned long long *cnt,
                                   const char *name, int32_t *ol, unsigned long long *oc, int8_t *olt) -> sg_status {
                 const size_t tsm = filt ? tab_bytes((int64_t)1 << log2T, S) + fbytes : fz_bytes(log2T);
@@ -1927,23 +2016,8 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
     } while (0)
                 if (filt && upper) SG_TAB_SK(true, true);
                 else if (filt) SG_TAB_SK(true, false);
-                else if (!compact && upper) SG_TAB_LAUNCH(3, false, true);
-                else if (!compact) SG_TAB_LAUNCH(3, false, false);
-                else {
-                    auto run = [&](auto kern) -> sg_status {
-                        SG_CUDA_TRY(ensure_smem(kern, sm));
-                        if (carve >= 0)
-                            SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
-                        SG_LAUNCH(name, kern, grid, nt, sm, s, g, rl, cnt, log2T, class_ob(log2T), o, ol, oc, wb_off, olt);
-                        return SG_OK;
-                    };
-                    if (upper)
-                        SG_TRY(SK == 0 ? run(ctab_numeric_kernel<0, true>)
-                                       : (SK == 1 ? run(ctab_numeric_kernel<1, true>) : run(ctab_numeric_kernel<2, true>)));
-                    else
-                        SG_TRY(SK == 0 ? run(ctab_numeric_kernel<0, false>)
-                                       : (SK == 1 ? run(ctab_numeric_kernel<1, false>) : run(ctab_numeric_kernel<2, false>)));
-                }
+                else if (upper) SG_TAB_LAUNCH(3, false, true);
+                else SG_TAB_LAUNCH(3, false, false);
 #undef SG_TAB_SK
 #undef SG_TAB_LAUNCH
                 return SG_OK;
@@ -1997,7 +2071,8 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             int32_t *esc_ovf = esc_shift > 0 ? sc.get<int32_t>(n + 1) : nullptr;
             if (esc_shift > 0 && (!ovf_lt || !esc_counts || !esc_lists || !esc_ovf)) return SG_ERR_OOM;
             if (esc_shift > 0) SG_CUDA_TRY(cudaMemsetAsync(esc_counts, 0, (NCNT + 1) * sizeof(unsigned long long), s));
-            for (int c = 0; c < fz.ncls; c++) {
+            if (compact) SG_TRY(launch_group(lists, h_fz, ovf, fz_ovf, ovf_lt));
+            for (int c = 0; !compact && c < fz.ncls; c++) {
                 if (!h_fz[c]) continue;
                 SG_TRY(launch_tab(false, fz.log2T[c], lists + (int64_t)c * n, fz_counts + c,
                                   NUM_NAMES[fz.log2T[c] - SP_MINLOG], ovf, fz_ovf, ovf_lt));
@@ -2016,7 +2091,8 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                           (const int8_t *)ovf_lt, (const unsigned long long *)fz_ovf, esc_shift, fz, n, esc_counts,
                           esc_lists);
                 SG_CUDA_TRY(read_back(h_esc, esc_counts, sizeof(h_esc), s));
-                for (int c = 0; c < fz.ncls; c++) {
+                if (compact) SG_TRY(launch_group(esc_lists, h_esc, esc_ovf, esc_counts + NCNT, nullptr));
+                for (int c = 0; !compact && c < fz.ncls; c++) {
                     if (!h_esc[c]) continue;
                     SG_TRY(launch_tab(false, fz.log2T[c], esc_lists + (int64_t)c * n, esc_counts + c,
                                       NUM_NAMES[fz.log2T[c] - SP_MINLOG], esc_ovf, esc_counts + NCNT, nullptr));
