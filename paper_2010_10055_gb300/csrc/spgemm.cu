@@ -1351,34 +1351,44 @@ __device__ __forceinline__ int64_t fit_at(const PartnerFit &f, int64_t L, int64_
     return (int64_t)((double)L * x * (1.0 / 65536.0));
 }
 
-// Table requests of the fused pass, from each row's number of A entries L: a guess of fu's partners,
-// at least 64 slots; *kept += fk's (the kept partners).
-// Rows with L >= fwork (fwork > 0) take the filtered pass: their guess ((L * ff) >> 16, at most
-// fcap = the largest filtered shared-memory table) goes to need_f and need is 0, else need_f is 0.
-// Unfiltered rows of more than lmax entries take the global-memory class.
+// Table classes of the fused pass, from each row's number of A entries L: a guess of fu's partners,
+// at least 64 slots, decides the class (cl; lists and counts as by classify_kernel); *kept += fk's
+// (the kept partners). Rows with L >= fwork (fwork > 0) take the filtered pass: their guess
+// ((L * ff) >> 16) picks one of clf's classes, the largest at most. Unfiltered rows of more than
+// lmax entries take the global-memory class. 100,000 rows: 20 us; with one counter update per row
+// and a kernel for each half, 75 us.
 __global__ void fx_need_kernel(const int64_t *__restrict__ a_rp, int64_t n, PartnerFit fu, PartnerFit fk, int64_t fwork,
-                               uint64_t ff, int64_t fcap, int64_t tcap, int64_t lmax, int64_t *__restrict__ need,
-                               int64_t *__restrict__ need_f, unsigned long long *__restrict__ kept) {
+                               uint64_t ff, int64_t tcap, int64_t lmax, Classes cl, Classes clf,
+                               unsigned long long *__restrict__ counts, int32_t *__restrict__ lists,
+                               unsigned long long *__restrict__ counts_f, int32_t *__restrict__ lists_f,
+                               unsigned long long *__restrict__ kept) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
     unsigned long long mine = 0;
-    if (i < n) {
-        const int64_t L = a_rp[i + 1] - a_rp[i];
-        need_f[i] = 0;
-        need[i] = 0;
-        if (L > 0) {
-            const bool filt = fwork > 0 && L >= fwork;
-            const int64_t g0 = filt ? (int64_t)(((unsigned __int128)L * ff) >> 16) : fit_at(fu, L, i, n);
-            int64_t guess = pow2_at_least(g0 > 64 ? g0 : 64);
-            if (guess > tcap) guess = tcap;  // no row has more partners than the table bound for all reads
-            if (filt && guess > fcap) guess = fcap;
-            if (!filt && L > lmax) guess = (int64_t)1 << 40;
-            (filt ? need_f : need)[i] = guess;
-            mine = (unsigned long long)fit_at(fk, L, i, n);
-        }
+    const int64_t L = i < n ? a_rp[i + 1] - a_rp[i] : 0;
+    const bool filt = fwork > 0 && L >= fwork;
+    int c = -1;  // class; filtered rows' behind the others'
+    if (L > 0) {
+        const int64_t g0 = filt ? (int64_t)(((unsigned __int128)L * ff) >> 16) : fit_at(fu, L, i, n);
+        int64_t guess = pow2_at_least(g0 > 64 ? g0 : 64);
+        if (guess > tcap) guess = tcap;  // no row has more partners than the table bound for all reads
+        if (!filt && L > lmax) guess = (int64_t)1 << 40;
+        const Classes &cs = filt ? clf : cl;
+        c = 0;  // a filtered row starts in the largest table at most
+        while (c < cs.ncls - (filt ? 1 : 0) && guess > ((int64_t)1 << cs.log2T[c])) c++;
+        if (filt) c += SP_NCLS + 1;
+        mine = (unsigned long long)fit_at(fk, L, i, n);
     }
+    // one counter update per class and warp
+    const uint32_t peers = __match_any_sync(0xffffffffu, c);
+    const int leader = __ffs(peers) - 1, x = filt ? c - (SP_NCLS + 1) : c;
+    unsigned long long q = 0;
+    if (c >= 0 && lane == leader) q = atomicAdd((filt ? counts_f : counts) + x, (unsigned long long)__popc(peers));
+    q = __shfl_sync(0xffffffffu, q, leader) + __popc(peers & ((1u << lane) - 1u));
+    if (c >= 0 && SG_IN_BOUNDS((int64_t)q < n, 302, q)) (filt ? lists_f : lists)[(int64_t)x * n + (int64_t)q] = (int32_t)i;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
-    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(kept, mine);
+    if (lane == 0 && mine) atomicAdd(kept, mine);
 }
 
 // Least-squares fit of y = L (base + slope x) to the sampled rows (x = 1 - i / n), neither negative.
@@ -1645,11 +1655,11 @@ __global__ void lower_fill_kernel(const uint32_t *__restrict__ mkey, const uint6
     }
 }
 
-// nnz of C's rows in the upper-triangle form: U row i plus its mirrored entries.
-__global__ void c_rowlen_kernel(const int64_t *__restrict__ nnz_row, const uint32_t *__restrict__ colcnt, int64_t n,
-                                int64_t *__restrict__ out) {
+// C's row starts from those of its rows in U and (upper-triangle form) of their mirrored parts.
+__global__ void c_row_ptr_kernel(const int64_t *__restrict__ rpu, const int64_t *__restrict__ lrp, int64_t n,
+                                 int64_t *__restrict__ c_rp) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = nnz_row[i] + colcnt[i];
+    if (i <= n) c_rp[i] = rpu[i] + (lrp ? lrp[i] : 0);
 }
 
 static inline int64_t blocks_for(int64_t n, int nt) { return (n + nt - 1) / nt; }
@@ -1745,23 +1755,20 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
     const int64_t n = A->n_rows, np = At->n_cols;
     const int NT = 256;
     constexpr int NCNT = SP_NCLS + 2;  // classes + global class + overflow counter
-    uint32_t *err = sc.get<uint32_t>(1);
-    int64_t *work = sc.get<int64_t>(n + 1);
+    constexpr int NCTR = 5 * NCNT + 12;
+    // zeroed in one go: counters | row lengths | entries mirrored into each row | error word
+    unsigned long long *counts = sc.get<unsigned long long>((size_t)NCTR + (n + 1) + (n + 2) / 2 + 1);
     int64_t *need = sc.get<int64_t>(n + 1);
-    int64_t *nnz_row = sc.get<int64_t>(n + 1);
-    int64_t *dist = sc.get<int64_t>(n + 1);
-    unsigned long long *counts = sc.get<unsigned long long>(4 * NCNT + 10);
     int32_t *lists = sc.get<int32_t>((size_t)(SP_NCLS + 1) * (n + 1));
     int32_t *ovf = sc.get<int32_t>(2 * (n + 1));  // overflow list | unused list of the re-run
-    if (!err || !work || !need || !nnz_row || !dist || !counts || !lists || !ovf) return SG_ERR_OOM;
+    if (!need || !counts || !lists || !ovf) return SG_ERR_OOM;
+    int64_t *nnz_row = (int64_t *)(counts + NCTR);
+    uint32_t *colcnt = (uint32_t *)(nnz_row + n + 1), *err = colcnt + n + 1;
     unsigned long long *sym_counts = counts, *num_counts = counts + NCNT, *unused = counts + 2 * NCNT;
     unsigned long long *ovf_count = counts + SP_NCLS + 1;
     unsigned long long *fz_counts = counts + 2 * NCNT + 1, *fz_ovf = fz_counts + SP_NCLS + 1;
     unsigned long long *ff_counts = counts + 3 * NCNT + 1;  // filtered rows' classes + global class
-    SG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-    SG_CUDA_TRY(cudaMemsetAsync(counts, 0, (4 * NCNT + 10) * sizeof(unsigned long long), s));
-    SG_CUDA_TRY(cudaMemsetAsync(nnz_row, 0, (n + 1) * sizeof(int64_t), s));
-    SG_CUDA_TRY(cudaMemsetAsync(dist, 0, (n + 1) * sizeof(int64_t), s));
+    SG_CUDA_TRY(cudaMemsetAsync(counts, 0, (size_t)((unsigned char *)(err + 1) - (unsigned char *)counts), s));
     uint64_t *t_pair = nullptr;  // only the two-pass kernels read At as (val << 32 | col) pairs
     SpArgs g{A->row_ptr, A->col, A->val, At->row_ptr, At->col, At->val, nullptr, nullptr, t_pair,
              n, min_shared, S, err, np, opt.row0, nullptr};
@@ -1822,12 +1829,9 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
     // ---- fused path (no symbolic pass): guessed tables, rows written to a temporary region
     if (fused) {
         stage.emplace("SpGEMMNumeric", s);
-        int64_t *tmp_off = sc.get<int64_t>(n + 1), *need_f = sc.get<int64_t>(n + 1), *lrp = sc.get<int64_t>(n + 1);
-        int32_t *lists_f = sc.get<int32_t>((size_t)(SP_NCLS + 1) * (n + 1));
-        int32_t *retry = sc.get<int32_t>(n + 1);
-        uint32_t *colcnt = upper ? sc.get<uint32_t>(n + 1) : nullptr;
-        if (!tmp_off || !need_f || !lrp || !lists_f || !retry || (upper && !colcnt)) return SG_ERR_OOM;
-        if (upper) SG_CUDA_TRY(cudaMemsetAsync(colcnt, 0, (n + 1) * sizeof(uint32_t), s));
+        int64_t *tmp_off = sc.get<int64_t>(4 * (n + 1)), *lrp = tmp_off + n + 1, *wl = lrp + n + 1;
+        int32_t *retry = (int32_t *)(wl + n + 1);
+        if (!tmp_off) return SG_ERR_OOM;
         // counters after the class counts (4 NCNT + 1 of them), all zeroed above
         unsigned long long *tcur = counts + 4 * NCNT + 1;     // temporary region cursor
         unsigned long long *n_retry = counts + 4 * NCNT + 2;  // rows that found the region full
@@ -1843,15 +1847,15 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
         if (nsamp > 0 && n > 0 && A->nnz > 0) {
             const int64_t stride = n > nsamp ? n / nsamp : 1;
             const int64_t nb = (n + stride - 1) / stride;
-            const size_t ssm = fbytes + wbb(256);
+            const size_t ssm = fbytes + wbb(512);
             unsigned long long *rec = sc.get<unsigned long long>(3 * (size_t)nb);
             if (!rec) return SG_ERR_OOM;
             if (upper) {
                 SG_CUDA_TRY(ensure_smem(sample_fx_kernel<true>, ssm));
-                SG_LAUNCH("spgemm_sample", sample_fx_kernel<true>, nb, 256, ssm, s, g, stride, log2F, rec);
+                SG_LAUNCH("spgemm_sample", sample_fx_kernel<true>, nb, 512, ssm, s, g, stride, log2F, rec);
             } else {
                 SG_CUDA_TRY(ensure_smem(sample_fx_kernel<false>, ssm));
-                SG_LAUNCH("spgemm_sample", sample_fx_kernel<false>, nb, 256, ssm, s, g, stride, log2F, rec);
+                SG_LAUNCH("spgemm_sample", sample_fx_kernel<false>, nb, 512, ssm, s, g, stride, log2F, rec);
             }
             std::vector<unsigned long long> h(3 * (size_t)nb);
             SG_CUDA_TRY(read_back(h.data(), rec, h.size() * 8, s));
@@ -1879,18 +1883,16 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
         }
         const bool recur = r1 < 2.0 * r2;  // most partners recur: the filter would keep nearly all
         if (fmode == 1 && recur) fwork = 0;
+        int32_t *lists_f = fwork ? sc.get<int32_t>((size_t)(SP_NCLS + 1) * (n + 1)) : nullptr;
+        if (fwork && !lists_f) return SG_ERR_OOM;
         const double pct = (double)tune("spgemm_guess_pct") / 100.0;
         auto fixed = [](const FitD &f, double by) {
             return PartnerFit{(uint64_t)(by * f.base * 65536.0) + 1, (uint64_t)(by * f.slope * 65536.0)};
         };
         const uint64_t ffq = (uint64_t)(pct * r2 * 65536.0) + 1;
         SG_LAUNCH("fused_need", fx_need_kernel, blocks_for(n, NT), NT, 0, s, A->row_ptr, n, fixed(f1, pct),
-                  fixed(min_shared >= 2 ? f2 : f1, 1.0), fwork, ffq,
-                  ff.ncls > 0 ? (int64_t)1 << ff.log2T[ff.ncls - 1] : (int64_t)64, Tmax,
-                  compact ? (int64_t)CT_ROW : (int64_t)1 << 40, need, need_f, sums);
-        SG_LAUNCH("classify", classify_kernel, blocks_for(n, NT), NT, 0, s, need, n, fz, fz_counts, lists);
-        if (fwork)
-            SG_LAUNCH("classify", classify_kernel, blocks_for(n, NT), NT, 0, s, need_f, n, ff, ff_counts, lists_f);
+                  fixed(min_shared >= 2 ? f2 : f1, 1.0), fwork, ffq, Tmax,
+                  compact ? (int64_t)CT_ROW : (int64_t)1 << 40, fz, ff, fz_counts, lists, ff_counts, lists_f, sums);
         unsigned long long h_fz[NCNT], h_ff[NCNT], h_kept = 0;
         uint32_t herr = 0;
         SG_CUDA_TRY(cudaMemcpyAsync(h_ff, ff_counts, sizeof(h_ff), cudaMemcpyDeviceToHost, s));
@@ -1920,7 +1922,7 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             o.len = nnz_row;
             o.retry = retry;
             o.n_retry = n_retry;
-            o.colcnt = colcnt;
+            o.colcnt = upper ? colcnt : nullptr;
             int64_t least = 64;  // about four entries of a mean row per thread
             while (least < 256 && 4 * least < A->nnz / (n > 0 ? n : 1)) least <<= 1;
             // one launch per table class; the seed form (SK), the filter and the form pick the kernel
@@ -2023,8 +2025,6 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                 return SG_OK;
             };
             // rows in exact global-memory tables: their products first (table sizes), then the pass
-            int64_t *wl = sc.get<int64_t>(n + 1);
-            if (!wl) return SG_ERR_OOM;
             auto launch_gtab = [&](const int32_t *rl, const unsigned long long *cnt, unsigned long long nrows)
                 -> sg_status {
                 SG_CUDA_TRY(cudaMemsetAsync(gw, 0, 2 * sizeof(unsigned long long), s));
@@ -2065,12 +2065,10 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             // one fits in shared memory (esc: second-round class lists and counts, their overflow
             // list), else redone in global memory
             const int esc_shift = (int)tune("spgemm_escalate");
+            unsigned long long *esc_counts = counts + 4 * NCNT + 10;  // zeroed above
             int8_t *ovf_lt = esc_shift > 0 ? sc.get<int8_t>(n + 1) : nullptr;
-            unsigned long long *esc_counts = esc_shift > 0 ? sc.get<unsigned long long>(NCNT + 1) : nullptr;
-            int32_t *esc_lists = esc_shift > 0 ? sc.get<int32_t>((size_t)(SP_NCLS + 1) * (n + 1)) : nullptr;
-            int32_t *esc_ovf = esc_shift > 0 ? sc.get<int32_t>(n + 1) : nullptr;
-            if (esc_shift > 0 && (!ovf_lt || !esc_counts || !esc_lists || !esc_ovf)) return SG_ERR_OOM;
-            if (esc_shift > 0) SG_CUDA_TRY(cudaMemsetAsync(esc_counts, 0, (NCNT + 1) * sizeof(unsigned long long), s));
+            int32_t *esc_lists = nullptr, *esc_ovf = nullptr;
+            if (esc_shift > 0 && !ovf_lt) return SG_ERR_OOM;
             if (compact) SG_TRY(launch_group(lists, h_fz, ovf, fz_ovf, ovf_lt));
             for (int c = 0; !compact && c < fz.ncls; c++) {
                 if (!h_fz[c]) continue;
@@ -2082,11 +2080,27 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                 SG_TRY(launch_tab(true, ff.log2T[c], lists_f + (int64_t)c * n, ff_counts + c,
                                   FIL_NAMES[ff.log2T[c] - SP_MINLOG], ovf, fz_ovf, nullptr));
             }
-            unsigned long long n_ovf = 0, h_esc[NCNT + 1] = {};
+            // the column starts of the mirrored parts and the rows' starts, for the usual case that no
+            // row is left over
+            int64_t *rpu = need;
+            int64_t nnz_u = 0;
+            auto scans = [&]() -> sg_status {
+                if (upper) SG_TRY(exclusive_scan<uint32_t>(colcnt, lrp, n, s, err));
+                SG_TRY(exclusive_scan<int64_t>(nnz_row, rpu, n, s, err));
+                SG_CUDA_TRY(cudaMemcpyAsync(&nnz_u, rpu + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+                SG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+                return SG_OK;
+            };
+            unsigned long long n_ovf = 0, n_rt = 0, h_esc[NCNT + 1] = {};
+            SG_TRY(scans());
+            SG_CUDA_TRY(cudaMemcpyAsync(&n_rt, n_retry, sizeof(n_rt), cudaMemcpyDeviceToHost, s));
             SG_CUDA_TRY(read_back(&n_ovf, fz_ovf, sizeof(n_ovf), s));
             // filtered rows' overflows (no size recorded) are escalated past every class
             const bool escalate = esc_shift > 0 && n_ovf > 0 && !fwork;
             if (escalate) {
+                esc_lists = sc.get<int32_t>((size_t)(SP_NCLS + 2) * (n + 1));
+                if (!esc_lists) return SG_ERR_OOM;
+                esc_ovf = esc_lists + (size_t)(SP_NCLS + 1) * (n + 1);
                 SG_LAUNCH("escalate", escalate_kernel, blocks_for((int64_t)n_ovf, NT), NT, 0, s, (const int32_t *)ovf,
                           (const int8_t *)ovf_lt, (const unsigned long long *)fz_ovf, esc_shift, fz, n, esc_counts,
                           esc_lists);
@@ -2111,8 +2125,8 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                 SG_TRY(launch_gtab((const int32_t *)ovf, fz_ovf, n_ovf));
             }
             // rows that found the region full: grow it by their exact room and redo them
-            unsigned long long n_rt = 0;
-            SG_CUDA_TRY(read_back(&n_rt, n_retry, sizeof(n_rt), s));
+            const bool more = n_ovf || n_big || n_big_f;
+            if (more) SG_CUDA_TRY(read_back(&n_rt, n_retry, sizeof(n_rt), s));
             if (n_rt) {
                 int32_t *rl = sc.get<int32_t>(n_rt + 1);
                 unsigned long long *rc = sc.get<unsigned long long>(1);
@@ -2182,15 +2196,11 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                     SG_TRY(mark(esc_ovf, n_ovf2, 64, true));
                 }
             }
-            int64_t *clen = upper ? need_f : nnz_row;  // need_f is free once the classes have run
-            if (upper)
-                SG_LAUNCH("c_rowlen", c_rowlen_kernel, blocks_for(n, NT), NT, 0, s, (const int64_t *)nnz_row,
-                          (const uint32_t *)colcnt, n, need_f);
-            SG_ALLOC(C->row_ptr, int64_t, n + 1, s);
-            SG_TRY(exclusive_scan<int64_t>(clen, C->row_ptr, n, s, err));
-            int64_t nnz = 0;
-            SG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-            SG_CUDA_TRY(read_back(&nnz, C->row_ptr + n, sizeof(int64_t), s));
+            if (more || n_rt) {
+                SG_TRY(scans());
+                SG_CUDA_TRY(cudaStreamSynchronize(s));
+            }
+            const int64_t nnz = upper ? 2 * nnz_u : nnz_u;  // C = U + U^T
             if (herr & DEV_TIMEOUT) return timeout_error("overlap_spgemm");
             if (herr) {
                 set_error("overlap_spgemm: a row exceeded its output bound (internal error)");
@@ -2199,10 +2209,13 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             C->n = n;
             C->nnz = nnz;
             C->max_seeds = S;
+            SG_ALLOC(C->row_ptr, int64_t, n + 1, s);
             SG_ALLOC(C->col, int32_t, nnz, s);
             SG_ALLOC(C->count, uint32_t, nnz, s);
             SG_ALLOC(C->seed_i, uint32_t, (int64_t)S * nnz, s);
             SG_ALLOC(C->seed_k, uint32_t, (int64_t)S * nnz, s);
+            SG_LAUNCH("c_row_ptr", c_row_ptr_kernel, blocks_for(n + 1, NT), NT, 0, s, (const int64_t *)rpu,
+                      upper ? (const int64_t *)lrp : (const int64_t *)nullptr, n, C->row_ptr);
             if (!upper) {
                 SG_LAUNCH("compact_c", compact_c_kernel, blocks_for(n * 32, 256), 256, 0, s, (const int64_t *)tmp_off,
                           cap, (const int32_t *)o.col, (const uint32_t *)o.cnt, (const uint32_t *)o.si,
@@ -2211,12 +2224,8 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                 return SG_OK;
             }
             // C = U + U^T: U rows in place; the mirrored entries of each column, in row order
-            SG_TRY(exclusive_scan<uint32_t>(colcnt, lrp, n, s, err));
-            int64_t nnz_l = 0;
-            SG_CUDA_TRY(read_back(&nnz_l, lrp + n, sizeof(int64_t), s));
+            const int64_t nnz_l = nnz_u;
             if (tune("spgemm_mirror_sort") && nnz < ((int64_t)1 << MIRROR_POS_BITS)) {
-                int64_t *rpu = need;  // free once the classes have run
-                SG_TRY(exclusive_scan<int64_t>(nnz_row, rpu, n, s, err));
                 uint32_t *mk0 = sc.get<uint32_t>(nnz_l + 1), *mk1 = sc.get<uint32_t>(nnz_l + 1);
                 uint64_t *mv0 = sc.get<uint64_t>(nnz_l + 1), *mv1 = sc.get<uint64_t>(nnz_l + 1);
                 if (!mk0 || !mk1 || !mv0 || !mv1) return SG_ERR_OOM;
@@ -2279,6 +2288,9 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
         // the temporary region would exceed its budget: the two-pass path below
     }
     // ---- two-pass form: row work and At extents per A entry, symbolic sizes, exact tables
+    int64_t *work = sc.get<int64_t>(2 * (n + 1)), *dist = work + n + 1;
+    if (!work) return SG_ERR_OOM;
+    SG_CUDA_TRY(cudaMemsetAsync(dist, 0, (n + 1) * sizeof(int64_t), s));
     int64_t *a_beg = sc.get<int64_t>(A->nnz + 1);
     uint32_t *a_len = sc.get<uint32_t>(A->nnz + 1);
     if (!a_beg || !a_len) return SG_ERR_OOM;
