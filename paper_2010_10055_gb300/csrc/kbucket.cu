@@ -244,13 +244,16 @@ __global__ void __launch_bounds__(PK_NT) kb_pack_kernel(const uint8_t *__restric
             M[2] = (uint32_t)hi;
             M[3] = (uint32_t)(hi >> 32);
         }
-        if (tb > 0 && !jp.jpos) {
+        // a group inside one read set: its prefix once
+        const uint32_t job = jp.jpos ? (uint32_t)(jc.prefix(qs) >> jp.kbits) : 0u;
+        if (tb > 0 && (!jp.jpos || qs + 32 <= jc.jhi)) {
+            const uint32_t jb = job << tb;
 #pragma unroll
             for (int j = 0; j < 32; j++) {
                 if (!((vm >> j) & 1u)) continue;
                 const uint32_t fw = __funnelshift_l(B[j / 16 + 1], B[j / 16], 2 * (j % 16)) >> (32 - tb);
                 const uint32_t rc = ~__funnelshift_r(M[j / 16], M[j / 16 + 1], 2 * (j % 16)) & tmask;
-                atomicAdd(pk_hist + (fw < rc ? fw : rc), 1u);
+                atomicAdd(pk_hist + (jb | (fw < rc ? fw : rc)), 1u);
             }
         } else {
 #pragma unroll 1
