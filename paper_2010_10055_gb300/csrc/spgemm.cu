@@ -76,7 +76,8 @@ struct SpArgs {
 
 // One At row as a 32-byte record: its start in At, its length and, when it has at most AT_INL
 // entries, their reads. An A entry's products then cost one aligned 32-byte load -- one DRAM
-// sector -- instead of a row-pointer gather plus a gather of the row.
+// sector -- instead of a row-pointer gather plus a gather of the row. A longer row's record holds
+// the reads at AT_INL even steps instead (at_step), which stand in for the first loads of a search.
 constexpr int AT_INL = 5;
 struct __align__(32) AtRec {
     int64_t b;
@@ -85,18 +86,31 @@ struct __align__(32) AtRec {
 };
 static_assert(sizeof(AtRec) == 32, "one sector per record");
 
+// One 32-byte load: 32 lanes with 32 records are 32 look-ups in L1, as two 16-byte loads 64.
 __device__ __forceinline__ AtRec load_rec(const AtRec *p) {
-    const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p));
-    const uint4 y = __ldg(reinterpret_cast<const uint4 *>(p) + 1);
+    uint64_t w0, w1, w2, w3;
+    asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(w0), "=l"(w1), "=l"(w2), "=l"(w3) : "l"(p));
     AtRec r;
-    r.b = (int64_t)(((uint64_t)x.y << 32) | x.x);
-    r.len = x.z;
-    r.r[0] = (int32_t)x.w;
-    r.r[1] = (int32_t)y.x;
-    r.r[2] = (int32_t)y.y;
-    r.r[3] = (int32_t)y.z;
-    r.r[4] = (int32_t)y.w;
+    r.b = (int64_t)w0;
+    r.len = (uint32_t)w1;
+    r.r[0] = (int32_t)(w1 >> 32);
+    r.r[1] = (int32_t)(uint32_t)w2;
+    r.r[2] = (int32_t)(w2 >> 32);
+    r.r[3] = (int32_t)(uint32_t)w3;
+    r.r[4] = (int32_t)(w3 >> 32);
     return r;
+}
+
+// r[t] of a row of more than AT_INL entries: the read at entry (t + 1) at_step(len).
+__device__ __forceinline__ uint32_t at_step(uint32_t len) { return len / (AT_INL + 1); }
+// The entries that may hold the last read <= k of such a row: [*lo, *hi); *lo does unless it is 0.
+__device__ __forceinline__ void at_narrow(const AtRec &r, int32_t k, uint32_t *lo, uint32_t *hi) {
+    const uint32_t st = at_step(r.len);
+    uint32_t t = 0;
+#pragma unroll
+    for (int q = 0; q < AT_INL; q++) t += r.r[q] <= k ? 1u : 0u;
+    *lo = t * st;
+    *hi = t < AT_INL ? *lo + st : r.len;
 }
 
 // One thread per row j of At: its record.
@@ -111,7 +125,10 @@ __global__ void at_rec_kernel(const int64_t *__restrict__ t_rp, const int32_t *_
     x.z = len > 0xFFFFFFFFll ? 0xFFFFFFFFu : (uint32_t)len;
     int32_t r[AT_INL];
 #pragma unroll
-    for (int t = 0; t < AT_INL; t++) r[t] = (len <= AT_INL && t < len) ? t_col[b + t] : -1;
+    for (int t = 0; t < AT_INL; t++) {
+        const int64_t e = len <= AT_INL ? t : (t + 1) * (int64_t)at_step(x.z);
+        r[t] = e < len ? t_col[b + e] : -1;
+    }
     x.w = (uint32_t)r[0];
     y.x = (uint32_t)r[1];
     y.y = (uint32_t)r[2];
@@ -582,11 +599,13 @@ __global__ void __launch_bounds__(1024) numeric_kernel(SpArgs g, const int32_t *
 // j = a_col[a] after read gi (UPPER), or the whole row (gi itself is skipped by the caller). With
 // records, a row of at most AT_INL entries is read from its record: *rec receives it and *t0 the
 // index of the first product within it; *t0 = -1 otherwise (the products are read from t_col).
+// A long row's extent may begin with up to AT_SKIP reads that are not past gi (no search).
+constexpr uint32_t AT_SKIP = 12;
 template <bool UPPER>
 __device__ __forceinline__ void at_extent(const SpArgs &g, int64_t a, int32_t gi, int64_t &beg, uint32_t &len,
                                           AtRec *rec = nullptr, int *t0 = nullptr) {
     const int32_t j = g.a_col[a];
-    int64_t b, e;
+    int64_t b, e, lo, hi = 0;
     if (g.t_rec) {
         const AtRec r = load_rec(g.t_rec + j);
         b = r.b;
@@ -603,15 +622,20 @@ __device__ __forceinline__ void at_extent(const SpArgs &g, int64_t a, int32_t gi
             if (t0) *t0 = t;
             return;
         }
+        lo = b;
         e = b + (int64_t)r.len;
+        if (UPPER) {
+            uint32_t s0, s1;
+            at_narrow(r, gi, &s0, &s1);
+            lo = b + s0;
+            hi = s1 - s0 <= AT_SKIP ? lo : b + s1;  // a few reads up to gi are left to the caller
+        }
     } else {
-        b = g.t_rp[j];
-        e = g.t_rp[j + 1];
+        lo = b = g.t_rp[j];
+        hi = e = g.t_rp[j + 1];
     }
     if (t0) *t0 = -1;
-    int64_t lo = b;
     if (UPPER) {
-        int64_t hi = e;
         while (lo < hi) {  // first entry of At row j with read > gi
             const int64_t mid = (lo + hi) >> 1;
             if (g.t_col[mid] <= gi) lo = mid + 1; else hi = mid;
@@ -622,7 +646,7 @@ __device__ __forceinline__ void at_extent(const SpArgs &g, int64_t a, int32_t gi
 }
 
 // Products of row i (read id gi): f(k, idx, ok) by every lane of the warp, for every product (ok): k =
-// the partner, idx = index of the A entry within the row; k == gi is no product. Warp-cooperative: a warp
+// the partner, idx = index of the A entry within the row; others are no products. Warp-cooperative: a warp
 // takes 32 consecutive entries of A's row, finds their extents, scans their lengths (32-bit) and
 // walks the flattened products TU_U x 32 at a time, each lane finding its entry by a 5-step
 // shuffle search; the gathers of the next step are issued before the current step's table
@@ -699,7 +723,7 @@ __device__ __forceinline__ void enum_fused(const SpArgs &g, int32_t gi, int64_t 
             }
             if (base + 32 * TU_U < total) gather(base + 32 * TU_U);
 #pragma unroll
-            for (int u = 0; u < TU_U; u++) f(k_cur[u], i_cur[u], k_cur[u] != gi);
+            for (int u = 0; u < TU_U; u++) f(k_cur[u], i_cur[u], UPPER ? k_cur[u] > gi : k_cur[u] != gi);
         }
     }
 }
@@ -743,6 +767,11 @@ __device__ __forceinline__ void seeds_of(const SpArgs &g, int64_t a0, int64_t a1
                 for (int t = 1; t < AT_INL; t++)
                     if (t < (int)rr[q].len && rr[q].r[t] <= k) at[q] = b[q] + t;
                 len[q] = 0;  // found
+            } else {
+                uint32_t s0, s1;
+                at_narrow(rr[q], k, &s0, &s1);
+                b[q] += s0;
+                len[q] = s1 - s0;
             }
         }
     } else {
