@@ -1027,13 +1027,17 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     // rows of one bucket: at most 2^12, a slot each
     const int rest = rbits - pb1, b2min = two && rest > 12 ? rest - 12 : 0;
     KbPlan pl;
-    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, kb_target<K>(), b2min, sc));
+    // a bucket is a range of (read, column): some rows, or a part of one. Where a mean row is nearly a
+    // block's records, half of them would not fit: two parts each (12 Mbp, k = 31, rows of 7,200: 4.6 ms
+    // -> 3.7; rows of 4,400, 100 Mbp: parts 31 ms, rows 22)
+    const int target = nnz / n > kb_target<K>() / 4 * 3 ? kb_target<K>() / 2 : kb_target<K>();
+    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, target, b2min, sc));
     const int64_t ntiles = blocks_for(nnz, TILE);
     int32_t *tcol = sc.get<int32_t>(ntiles);
     typename K::T *r0 = sc.get<typename K::T>(nnz), *r1 = two ? sc.get<typename K::T>(nnz) : nullptr;
     if (!tcol || !r0 || (two && !r1)) return SG_ERR_OOM;
-    SG_LAUNCH("a_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, kb_target<K>(),
-              two ? std::min(KB_MAXB2, rest) : 0, b2min, KB_CHUNK_TILES * TILE);
+    SG_LAUNCH("a_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, target,
+              two ? std::min(KB_MAXB2, pl.rem) : 0, b2min, KB_CHUNK_TILES * TILE);
     SG_LAUNCH("a_tile_col", tile_col_kernel<TILE>, blocks_for(m, 256), 256, 0, s, At->row_ptr, m, tcol);
     const size_t sm = scatter_smem_bytes<K, true>(pl.nb1);
     SG_CUDA_TRY(ensure_smem(at_scatter_kernel<K>, sm));
@@ -1064,8 +1068,8 @@ sg_status transpose_impl(const sg_csr_u32 *At, sg_csr_u32 *A, int pbits, cudaStr
     const int rbits = bits_for(n), cbits = std::max(bits_for(m), 1);
     // one level while a row group of 2^(rbits - pb1) rows fits a block on average
     int want = 0;  // bits of the buckets wanted
-    while (want < rbits && (nnz >> want) > kb_target<KeyN>() / 2) want++;
-    const bool two = want > 10 || rbits - std::min(want, rbits) > 12;
+    while (want < rbits + cbits && (nnz >> want) > kb_target<KeyN>() / 2) want++;
+    const bool two = want > 10 || want > rbits || rbits - want > 12;
     // a second level splits by at most 11 bits and leaves at most 12 bits of rows to a bucket
     const int pb1 = std::min(rbits, two ? std::max((std::min(want, 20) + 1) / 2, std::max(6, rbits - 23)) : want);
     const KeyBits kb{0, pbits};
