@@ -123,11 +123,31 @@ class ClockSampler:
 # --------------------------------------------------------------------------- roofline
 def algorithmic_bytes(kernel: str, sz: dict) -> float | None:
     """Bytes the method must move per step in `kernel` (inputs read once, outputs written once),
-    from the per-unit figures: a 4-byte filter hash and 2 bits of packed base per position,
-    4-byte filter words (a touch is a read and a write), 8-byte keys, 24-byte C entries."""
+    from the per-unit figures: in the bucketed k-mer stage half a byte of packed base, mask and
+    read per position and a record per window; in the general one a 4-byte filter hash and 2
+    bits of packed base per position, 4-byte filter words (a touch is a read and a write) and
+    8-byte keys; 24-byte C entries."""
+    k = sz.get("kstats") or {}
+    if k and k.get("sort_passes") == 0 and k.get("candidates"):  # bucketed k-mer stage: a record per window
+        rec, cand, nnz = float(k["sort_key_bytes"]), k["candidates"], k["nnz"]
+        bucketed = {
+            "pack": 1.5 * sz["total"],                           # bases in; packed bases, masks, reads out
+            "kmer_scatter1": 0.5 * sz["total"] + rec * cand,     # those in, records out
+            "kmer_hist2": rec * cand,
+            "kmer_scatter2": 2.0 * rec * cand,
+            "kmer_finish": rec * (cand + nnz),                   # records in, kept ones out
+            "emit_at": (rec + 8.0) * nnz + 16.0 * k["m"],        # kept records in; At and codes out
+            "a_scatter1": 16.0 * nnz + 8.0 * k["m"],             # At in, 8-byte records out
+            "a_hist2": 8.0 * nnz,
+            "a_scatter2": 16.0 * nnz,
+            "a_rows": 16.0 * nnz,                                # records in, A out
+        }
+        if kernel in bucketed:
+            return bucketed[kernel]
+    if kernel == "at_records":                                 # At's rows in, 32-byte records out
+        return 40.0 * sz["m"] + 4.0 * sz["nnzA"]
     if kernel == "pack":
         return 1.0 * sz["total"] + 4.25 * sz["total"]          # bases in; hash + packed base out
-    k = sz.get("kstats") or {}
     if kernel == "bloom_insert" and k.get("bloom_bins"):      # shared-memory bins: binned hashes in, B2 out
         return 4.0 * sz["windows"] + k["bloom_b2_bytes"]
     if kernel == "bloom_bin_scatter":                         # hashes in, binned hashes out

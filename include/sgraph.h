@@ -445,12 +445,13 @@ void sg_debug_record_classes(int on);
 int64_t sg_debug_spgemm_classes(int32_t *host_out, int64_t n);
 
 /* Sizes of the calling thread's last k-mer matrix build (sg_build_kmer_matrix or a batch), for
- * profiling: windows = sequence positions, candidates = windows that passed the Bloom filters and
- * were sorted, sort_key_bytes / sort_val_bytes = bytes per candidate through each radix pass
- * (val 0 when the window rides in the key), sort_passes = 8-bit passes over the candidates,
- * a_sort_passes = passes of the (read, entry) sort that forms A, m and nnz as in the outputs,
- * bloom_bins = shared-memory filter bins (0: the filters were sliced global-memory arrays),
- * bloom_b2_bytes = size of the seen-twice filter. */
+ * profiling: windows = sequence positions, candidates = windows that were counted exactly (bucketed
+ * form: every valid window; general form: those that passed the Bloom filters and were sorted),
+ * sort_key_bytes / sort_val_bytes = bytes per candidate through each grouping or radix pass (val 0
+ * when the window rides in the key), sort_passes = 8-bit radix passes over the candidates (0 in the
+ * bucketed form), a_sort_passes = 0 (A is formed by grouping), m and nnz as in the outputs,
+ * bloom_bins = shared-memory filter bins (0: none, or sliced global-memory arrays), bloom_b2_bytes =
+ * size of the seen-twice filter. */
 typedef struct {
     int64_t windows, candidates, m, nnz;
     int32_t sort_key_bytes, sort_val_bytes, sort_passes, a_sort_passes;
@@ -471,6 +472,10 @@ sg_status sg_memory_stats(uint64_t *reserved, uint64_t *in_use, uint64_t *in_use
 void sg_memory_reset_peak(void);
 
 /* Tunable launch parameters (used by the autotuner; results never depend on them):
+ *   kmer_bucketed         1: every window grouped by its code and counted in shared memory, where
+ *                         that form applies (hi up to 1024, k of 11 or more, no prefix that holds
+ *                         much of the input, records that fit the device); 0: the general form
+ *                         (filters and radix sort), which the next tunables are about (1)
  *   bloom_bits            bits of the first-level Bloom filter per window (8): fewer bits, fewer
  *                         slices but more false positives (singletons that reach the exact count)
  *   bloom_slice_mb        megabytes of the first-level Bloom filter updated per launch (64)
@@ -493,28 +498,39 @@ void sg_memory_reset_peak(void);
  *   spgemm_fused          1: C in one numeric pass whose tables are sized from a guess (rows that
  *                         overflow are redone in exact-size global-memory tables) and whose rows
  *                         go to a temporary region; 0: symbolic pass (exact sizes), then numeric (1)
- *   spgemm_sample_rows    rows sampled before the fused pass when nnz(A) >= spgemm_sample_min_nnz
- *                         (2^26) (256): their partners per product
- *                         (distinct, and seen at least twice) scale every row's table guess, and
- *                         the seen-twice filter is used only where it keeps under half the
- *                         partners; 0: no sample, guesses by the shifts below
- *   spgemm_guess_pct      sampled guess = pct / 100 x partners per product x products (300)
- *   num_guess_shift       fused numeric table guess without a sample = products >> shift (2)
+ *   spgemm_upper          1: the fused pass tabulates partners k > i only and mirrors them (1)
+ *   spgemm_at_records     1: the fused pass reads At rows as 32-byte records (1)
+ *   spgemm_sample_rows    rows sampled before the fused pass (256): their partners per entry of A
+ *                         (distinct, and seen at least twice) give every row's table guess; 0: no
+ *                         sample, a partner per entry
+ *   spgemm_guess_pct      guess = pct / 100 x the partners fitted to the sample (180)
+ *   spgemm_escalate       log2 of the growth of a guessed table that overflowed, tried once more in
+ *                         shared memory; 0: straight to an exact table in global memory (2)
+ *   spgemm_tmp_pct        temporary region of the fused pass, % of the kept partners fitted (125)
  *   spgemm_fused_max_mb   largest temporary region of the fused pass, MB (65536); above it, or
  *                         above half the device memory free at the call, the two-pass form runs
- *   spgemm_filter_mode    seen-twice filter for fused rows of spgemm_filter_work products or
+ *   spgemm_mirror_sort    1: mirrored entries ordered by a radix sort by column; 0: scattered by
+ *                         atomics and sorted per row (1); spgemm_mirror_rec 1: through 32-byte
+ *                         records of the upper triangle, for max_seeds <= 3 (1); spgemm_lower_smem:
+ *                         (mirror_sort 0) parts up to this long are sorted in shared memory (4096)
+ *   spgemm_filter_mode    seen-twice filter for fused rows of spgemm_filter_work entries of A or
  *                         more: they first mark, in two bit filters, the partners seen once and
  *                         seen twice, and tabulate only the latter (count-1 partners cannot reach C
- *                         when min_shared >= 2). 0 never, 1 when the row sample finds that fewer
- *                         than half the partners recur (1), 2 always
- *   spgemm_filter_work    rows with at least this many products may be filtered; 0: none (2048)
- *   spgemm_filter_shift   table guess of those rows without a sample = products >> shift (2)
+ *                         when min_shared >= 2). 0 never (0), 1 when the row sample finds that fewer
+ *                         than half the partners recur, 2 always
+ *   spgemm_filter_work    rows with at least this many entries may be filtered; 0: none (1024)
  *   spgemm_filter_log2    bits per filter: one per read up to 2^this, hashed beyond (17)
  *   sym_guess_shift       symbolic hash table guess = products of the row >> shift (2)
- *   spgemm_blocks_per_sm  blocks per SM of each SpGEMM class launch (16)
- *   spgemm_big_threads    threads per numeric block for tables of 4 K slots or more: 512 or 1024
- *                         (1024)
+ *   spgemm_blocks_per_sm  blocks per SM of each SpGEMM launch, at most (256)
+ *   spgemm_tab_warps      warps per SM wanted of a launch's resident blocks (64);
+ *                         spgemm_tab_warps_big: for tables of 4 K slots and more (64)
+ *   spgemm_smem_carveout  shared-memory carveout of the fused pass, % (-1: the driver's)
+ *   spgemm_big_threads    threads per numeric block for tables of 4 K slots or more where
+ *                         spgemm_tab_warps is 0: 512 or 1024 (1024)
  *   tr_blocks_per_sm      blocks per SM of the min-plus launch (32)
+ *   tr_warp_rows          1: rows of up to 128 entries reduced by a warp each; 0: by blocks (1)
+ *   batch_alone_kb        batched items of this many kilobases or more run on their own (64000); the
+ *                         others share unions of at most batch_group_kb (250000)
  *   pool_cross_stream_reuse  1: the library's memory pool may reuse memory freed on one stream for
  *                         another (read once, when the pool is created) (1)
  * sg_tune_set returns 1 if the name is known and the value in range, else 0 (no change).

@@ -21,15 +21,15 @@ SPACE = {
     "bloom_bits": [6, 8, 10, 12],
     "radix_lookback": [4, 8],
     "spgemm_upper": [0, 1],
-    "spgemm_guess_pct": [150, 200, 250, 300],
-    "spgemm_escalate": [0, 1],
+    "spgemm_guess_pct": [130, 150, 180, 200, 250],
+    "spgemm_escalate": [0, 1, 2],
     "spgemm_filter_mode": [0, 1],
     "spgemm_tab_warps": [32, 48, 64],
     "spgemm_tab_warps_big": [16, 32, 64],
     "spgemm_mirror_rec": [0, 1],
     "kmer_direct_seg": [0, 1],
     "spgemm_tmp_pct": [110, 125, 200],
-    "spgemm_blocks_per_sm": [4, 8, 16],
+    "spgemm_blocks_per_sm": [16, 64, 256],
     "tr_blocks_per_sm": [8, 16, 32],
     "tr_warp_rows": [0, 1],
 }

@@ -5,7 +5,9 @@
 // (KeyW) where the bits do not fit. Records are moved by at most two grouping passes:
 //  1. by the top pb1 bits of the code (a prefix p; those bits leave the record);
 //  2. within p, by the next b2[p] bits, b2 chosen from p's exact record count so that a bucket
-//     holds at most about 7/8 of what one block can finish in shared memory.
+//     holds at most 10/11 of what one block can finish in shared memory. (Any number of equal parts
+//     instead of 2^b2 fills the buckets better, but a part's first code costs a division and
+//     leaves fewer slots per record: the finishing pass of 4.1e9 records 52 -> 55 ms.)
 // Grouping is unordered (one atomic per tile and bin reserves a run), since the pass that finishes
 // a bucket orders its records itself: it counts them by slot -- the bucket's next code bits, about
 // as many slots as records -- places them by slot and ranks each among the few of its slot by full
@@ -115,7 +117,8 @@ inline size_t scatter_smem_bytes(int nb) {
 // The second half of a grouping pass, on records held in registers: br[u] = bin << 16 | rank in
 // the bin within the tile, or 0xFFFFFFFF for no record; cnt[] holds the tile's counts. Orders the
 // tile by bin in shared memory and writes every bin's run at a place reserved on cur[bin]
-// (positions are absolute). binof(key) recovers a record's bin unless BINARR keeps it; then() runs
+// (positions are absolute; the lanes of a warp reserve on consecutive words, one request: cursors 32
+// or 128 bytes apart cost 3 and 15 % of the pass). binof(key) recovers a record's bin unless BINARR keeps it; then() runs
 // once the records are in shared memory.
 struct NoOp {
     __device__ void operator()() const {}
@@ -185,7 +188,8 @@ __device__ __forceinline__ void scatter_layout(unsigned char *raw, int nb, Scatt
 __global__ void __launch_bounds__(1024) kb_plan_kernel(const unsigned long long *__restrict__ hist, KbPlan pl,
                                                       int target, int b2max, int b2min, int chunk);
 
-// Level-2 counts: a chunk of one prefix's records per block.
+// Level-2 counts: a chunk of one prefix's records per block. Bound by memory: 4.1e9 records of 8 bytes
+// 4.5 ms, 7.3 TB/s.
 template <class K>
 __global__ void __launch_bounds__(KB_NT) kb_hist2_kernel(KbPlan pl, const typename K::T *__restrict__ in,
                                                         int lowbits) {

@@ -17,7 +17,11 @@
 // windows are singletons and cost one random probe per window; here a singleton costs its share of
 // three or four streaming passes, and drops out when its slot counts one record.
 //
-// 4.1 G windows (100 Mbp at 40x): see the figures at the kernels.
+// 4.1 G windows, 1.77 G entries of A (100 Mbp at 40x, k = 17), ms: pack 3.8, scatter1 25, hist2 4.5,
+// scatter2 18.5, finish 52, emit 8.6, A 44 (scatter1 11.7, hist2 2, scatter2 7, rows 22.4): 157 in all,
+// against 387 for filters, sorts and segment passes (the general form in kmer.cu with a radix sort of
+// A). 154 M windows (5 Mbp at 30x): 4.7 against 5.9; k = 31, 300 M windows: 24.8 against 58 (16-byte
+// records, eight radix passes).
 #include <algorithm>
 #include <vector>
 
@@ -150,6 +154,8 @@ __device__ __forceinline__ void pack4(uint32_t w, uint32_t &code, uint32_t &ok) 
 // One group of 32 bases per lane, lane 31 only as the next group of lane 30 (a window needs up to
 // 31 bases past its group): a warp handles 31 groups per step, in consecutive steps, so that the
 // read of a group is found from the previous step's by a short gallop. P, VM and RG as in WindowSrc.
+// Bound by the prefix counts' shared-memory atomics and their code arithmetic, unrolled so that shifts
+// are immediates: 4.1e9 windows 3.8 ms (1.6 TB/s); a rolling encode and hash per window took 12.
 constexpr int PK_NT = 256;
 constexpr int PK_G = 31;
 
@@ -297,7 +303,8 @@ struct WindowSrc {
 
 // KK > 0: k as a compile-time constant. JOBS: a batch. A warp's groups are described in shared memory,
 // so that a window costs two broadcast loads and 32-bit operations (by shuffles: 26.0 ms instead of 25.2
-// for 4.1e9 windows).
+// for 4.1e9 windows). Bound by shared memory: a window is counted, placed with its bin, read back and
+// written in runs of about eight records (1.3 TB/s written).
 template <class K, int KK, bool JOBS>
 __global__ void __launch_bounds__(KB_NT, 2) kb_scatter1_kernel(WindowSrc w, KbPlan pl,
                                                               typename K::T *__restrict__ out) {
@@ -405,6 +412,10 @@ struct FinishArgs {
 // [c0, cend), at most 2^ls << sh wide: slot = (code - c0) >> sh. Returns the number of records
 // written, from base on. All threads call it. Loops over a thread's records end, for the whole
 // block, where its records do.
+// Bound by its chain of shared-memory phases, about 12 ps a record (4.1e9 records 52 ms): load and count
+// 11 ms, slot starts 5, placing 10, ranking within a slot 11.5, codes 3, keeping 5, writing 6. Blocks of
+// 256 threads with half the records 57 ms; the next bucket's records prefetched 60. Counting first drops
+// the records that are alone in their slot, so a singleton is neither placed nor ranked.
 template <class K, bool COUNT>
 __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const FinishArgs &a, int p,
                                                  typename K::T (&key)[K::ITEMS], int n, uint64_t c0,
@@ -795,7 +806,8 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const
 
 // ----------------------------------------------------------------------------------- emit
 // Kept records (in order within each bucket) -> At and the column codes. One warp per bucket: an
-// entry's column is the bucket's first column plus the codes started up to it (ballots).
+// entry's column is the bucket's first column plus the codes started up to it (ballots). Bound by
+// memory: 1.77 G entries 8.6 ms, 3.4 TB/s (a read search per kept entry in the sorted form took 35).
 template <class K>
 __global__ void __launch_bounds__(256) kb_emit_kernel(KbPlan pl, KeyBits kb, const typename K::T *__restrict__ in,
                                                      const int64_t *__restrict__ pseg,
@@ -888,7 +900,9 @@ __global__ void __launch_bounds__(512) read_hist_kernel(const int32_t *__restric
 }
 
 // At's entries as records (read below the prefix << cbits | column, position, strand), grouped by
-// the read's prefix. A tile's columns: its first entry's, plus the row starts up to an entry.
+// the read's prefix. A tile's columns: its first entry's, plus the row starts up to an entry. With the
+// pass that orders the rows and one between them 44 ms for 1.77 G entries; a radix sort of
+// (read, entry) pairs in three passes took 106 with what came around it.
 template <class K>
 __global__ void __launch_bounds__(KB_NT, 2) at_scatter_kernel(const int64_t *__restrict__ at_rp,
                                                              const int32_t *__restrict__ at_col,

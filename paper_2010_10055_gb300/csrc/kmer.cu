@@ -7,7 +7,10 @@
 // Sec. IV-D: A_ij holds the position of k-mer j in read i (here: pos | strand << 31 at the
 // lowest such position).
 //
-// Pipeline (all on `stream`):
+// Default: the bucketed form (kbucket.cu), which groups every window by its code and counts in
+// shared memory. The general form below takes what that form leaves: reliable ranges past 1,024,
+// k-mers of fewer than 11 bases, inputs of which one code prefix holds a large part, and inputs
+// whose records would not fit the device. Its pipeline (all on `stream`):
 //  0. pack           one walk over the reads packs the bases (2 bits each) and stores each
 //                    window's 32-bit filter hash (H_NONE where no valid window starts); later
 //                    passes recompute a window's canonical code and strand from two packed words.
@@ -27,8 +30,7 @@
 //     position: those entries are At's row, already sorted by read. For position-and-code keys
 //     this runs on the sorted keys themselves (seg_mark, scans of its tile totals, seg_emit,
 //     which resolves the kept windows to (read, pos)); other key forms are unpacked first.
-//  6. A = At transposed by a stable radix sort on the read id (columns stay ascending); its last
-//     pass writes A's column and value arrays.
+//  6. A = At transposed by grouping its entries by read (kbucket.cu).
 #include <optional>
 #include <type_traits>
 
