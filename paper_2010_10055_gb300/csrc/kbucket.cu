@@ -804,6 +804,16 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const
     }
 }
 
+__global__ void kb_totals_kernel(const int64_t *__restrict__ pseg, KbPlan pl, const uint32_t *__restrict__ err,
+                                 int64_t *__restrict__ out) {
+    if (threadIdx.x == 0) {
+        out[0] = pseg[pl.nsub_max];
+        out[1] = pseg[2 * pl.nsub_max];
+        out[2] = pl.start1[pl.nb1];
+        out[3] = (int64_t)*err;
+    }
+}
+
 // ----------------------------------------------------------------------------------- emit
 // Kept records (in order within each bucket) -> At and the column codes. One warp per bucket: an
 // entry's column is the bucket's first column plus the codes started up to it (ballots). Bound by
@@ -825,7 +835,7 @@ __global__ void __launch_bounds__(256) kb_emit_kernel(KbPlan pl, KeyBits kb, con
     const uint32_t le = lane == 31 ? 0xffffffffu : (2u << lane) - 1u;
     if (blockIdx.x == 0 && threadIdx.x == 0) at_rp[m] = nnz;
     for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nsub; b += nwarps) {
-        const int64_t o0 = pkeep[b], cnt = pkeep[b + 1] - o0;
+        const int64_t o0 = pkeep[b] - m, cnt = pkeep[b + 1] - m - o0;
         if (cnt == 0) continue;
         int64_t col0 = pseg[b] - 1;
         const int64_t s0 = start[b];
@@ -1143,10 +1153,10 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
         dst = r0;
     }
     uint32_t *nseg = sc.get<uint32_t>(2 * (size_t)pl.nsub_max);
-    int64_t *pseg = sc.get<int64_t>(2 * ((size_t)pl.nsub_max + 1));
+    int64_t *pseg = sc.get<int64_t>(2 * (size_t)pl.nsub_max + 1 + 4);
     if (!nseg || !pseg) return SG_ERR_OOM;
     uint32_t *nkeep = nseg + pl.nsub_max;
-    int64_t *pkeep = pseg + pl.nsub_max + 1;
+    int64_t *pkeep = pseg + pl.nsub_max, *totals = pseg + 2 * pl.nsub_max + 1;
     if (q.two) SG_CUDA_TRY(cudaMemsetAsync(nseg, 0, 2 * (size_t)pl.nsub_max * 4, s));  // past the last bucket
     FinishArgs a{};
     a.pl = pl;
@@ -1159,20 +1169,18 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
     a.nseg = nseg;
     a.nkeep = nkeep;
     SG_TRY(finish_launch<K>(a, true, src, dst, "kmer_finish", s));
-    SG_TRY(exclusive_scan<uint32_t>(nseg, pseg, pl.nsub_max, s, err));
-    SG_TRY(exclusive_scan<uint32_t>(nkeep, pkeep, pl.nsub_max, s, err));
-    int64_t sizes[3] = {0, 0, 0};  // m, nnz, records
-    uint32_t herr = 0;
-    SG_CUDA_TRY(cudaMemcpyAsync(&sizes[0], pseg + pl.nsub_max, 8, cudaMemcpyDeviceToHost, s));
-    SG_CUDA_TRY(cudaMemcpyAsync(&sizes[1], pkeep + pl.nsub_max, 8, cudaMemcpyDeviceToHost, s));
-    SG_CUDA_TRY(cudaMemcpyAsync(&sizes[2], pl.start1 + pl.nb1, 8, cudaMemcpyDeviceToHost, s));
-    SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));
+    // both totals in one scan (nkeep follows nseg): bucket b's kept records start at pkeep[b] - m
+    SG_TRY(exclusive_scan<uint32_t>(nseg, pseg, 2 * pl.nsub_max, s, err));
+    int64_t sizes[4] = {0, 0, 0, 0};  // m, m + nnz, records, error word: one copy, since each waits
+    SG_LAUNCH("kmer_totals", kb_totals_kernel, 1, 32, 0, s, (const int64_t *)pseg, pl, (const uint32_t *)err, totals);
+    SG_CUDA_TRY(read_back(sizes, totals, sizeof(sizes), s));
+    const uint32_t herr = (uint32_t)sizes[3];
     if (herr & DEV_TIMEOUT) return timeout_error("build_kmer_matrix");
     if (herr) {  // the passes above stayed in bounds; their results are discarded
         set_error("build_kmer_matrix: offsets are not a valid partition of the sequence");
         return SG_ERR_INVALID;
     }
-    const int64_t m = sizes[0], nnz = sizes[1];
+    const int64_t m = sizes[0], nnz = sizes[1] - m;
     if (m >= ((int64_t)1 << 31)) {
         set_error("build_kmer_matrix: %lld reliable k-mers exceed the int32 column range", (long long)m);
         return SG_ERR_OVERFLOW;

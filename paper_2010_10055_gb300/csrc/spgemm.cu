@@ -31,6 +31,7 @@
 // scans their At row lengths in registers, and walks the flattened product list 32 at a time,
 // each lane finding its entry with a 5-step shuffle search.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <optional>
 #include <vector>
@@ -1806,20 +1807,24 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
     const int64_t n = A->n_rows, np = At->n_cols;
     const int NT = 256;
     constexpr int NCNT = SP_NCLS + 2;  // classes + global class + overflow counter
-    constexpr int NCTR = 5 * NCNT + 12;
-    // zeroed in one go: counters | row lengths | entries mirrored into each row | error word
-    unsigned long long *counts = sc.get<unsigned long long>((size_t)NCTR + (n + 1) + (n + 2) / 2 + 1);
-    int64_t *need = sc.get<int64_t>(n + 1);
+    constexpr int NCTR = 5 * NCNT + 13;
+    // one block: starts of U's rows, the last of them beside the counters so that one copy reads both
+    // back (a copy to the host waits for the stream, about 8 us each); zeroed in one go from there:
+    // counters, the error word last | row lengths | entries mirrored into each row
+    int64_t *need = sc.get<int64_t>((n + 1) + (size_t)NCTR + (n + 1) + (n + 2) / 2);
     int32_t *lists = sc.get<int32_t>((size_t)(SP_NCLS + 1) * (n + 1));
     int32_t *ovf = sc.get<int32_t>(2 * (n + 1));  // overflow list | unused list of the re-run
-    if (!need || !counts || !lists || !ovf) return SG_ERR_OOM;
+    if (!need || !lists || !ovf) return SG_ERR_OOM;
+    unsigned long long *counts = (unsigned long long *)(need + n + 1);
     int64_t *nnz_row = (int64_t *)(counts + NCTR);
-    uint32_t *colcnt = (uint32_t *)(nnz_row + n + 1), *err = colcnt + n + 1;
+    uint32_t *colcnt = (uint32_t *)(nnz_row + n + 1), *err = (uint32_t *)(counts + NCTR - 1);
+    unsigned long long h_end[NCTR + 1] = {}, *h_cnt = h_end + 1;  // need[n] | counters
+    auto h_of = [&](const unsigned long long *c) { return h_cnt + (c - counts); };
     unsigned long long *sym_counts = counts, *num_counts = counts + NCNT, *unused = counts + 2 * NCNT;
     unsigned long long *ovf_count = counts + SP_NCLS + 1;
     unsigned long long *fz_counts = counts + 2 * NCNT + 1, *fz_ovf = fz_counts + SP_NCLS + 1;
     unsigned long long *ff_counts = counts + 3 * NCNT + 1;  // filtered rows' classes + global class
-    SG_CUDA_TRY(cudaMemsetAsync(counts, 0, (size_t)((unsigned char *)(err + 1) - (unsigned char *)counts), s));
+    SG_CUDA_TRY(cudaMemsetAsync(counts, 0, (size_t)((unsigned char *)(colcnt + n + 1) - (unsigned char *)counts), s));
     uint64_t *t_pair = nullptr;  // only the two-pass kernels read At as (val << 32 | col) pairs
     SpArgs g{A->row_ptr, A->col, A->val, At->row_ptr, At->col, At->val, nullptr, nullptr, t_pair,
              n, min_shared, S, err, np, opt.row0, nullptr};
@@ -1946,10 +1951,11 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                   compact ? (int64_t)CT_ROW : (int64_t)1 << 40, fz, ff, fz_counts, lists, ff_counts, lists_f, sums);
         unsigned long long h_fz[NCNT], h_ff[NCNT], h_kept = 0;
         uint32_t herr = 0;
-        SG_CUDA_TRY(cudaMemcpyAsync(h_ff, ff_counts, sizeof(h_ff), cudaMemcpyDeviceToHost, s));
-        SG_CUDA_TRY(cudaMemcpyAsync(h_fz, fz_counts, sizeof(h_fz), cudaMemcpyDeviceToHost, s));
-        SG_CUDA_TRY(cudaMemcpyAsync(&h_kept, sums, sizeof(h_kept), cudaMemcpyDeviceToHost, s));
-        SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));
+        SG_CUDA_TRY(read_back(h_cnt, counts, NCTR * sizeof(unsigned long long), s));
+        memcpy(h_ff, h_of(ff_counts), sizeof(h_ff));
+        memcpy(h_fz, h_of(fz_counts), sizeof(h_fz));
+        h_kept = *h_of(sums);
+        herr = (uint32_t)h_cnt[NCTR - 1];
         if (herr & DEV_TIMEOUT) return timeout_error("overlap_spgemm");
         // the temporary region: the kept partners fitted to the sample (at least twice for
         // min_shared >= 2), with room to spare; rows that find it full are redone in a grown one
@@ -2138,14 +2144,15 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             auto scans = [&]() -> sg_status {
                 if (upper) SG_TRY(exclusive_scan<uint32_t>(colcnt, lrp, n, s, err));
                 SG_TRY(exclusive_scan<int64_t>(nnz_row, rpu, n, s, err));
-                SG_CUDA_TRY(cudaMemcpyAsync(&nnz_u, rpu + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-                SG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+                SG_CUDA_TRY(read_back(h_end, rpu + n, sizeof(h_end), s));
+                nnz_u = (int64_t)h_end[0];
+                herr = (uint32_t)h_cnt[NCTR - 1];
                 return SG_OK;
             };
             unsigned long long n_ovf = 0, n_rt = 0, h_esc[NCNT + 1] = {};
             SG_TRY(scans());
-            SG_CUDA_TRY(cudaMemcpyAsync(&n_rt, n_retry, sizeof(n_rt), cudaMemcpyDeviceToHost, s));
-            SG_CUDA_TRY(read_back(&n_ovf, fz_ovf, sizeof(n_ovf), s));
+            n_rt = *h_of(n_retry);
+            n_ovf = *h_of(fz_ovf);
             // filtered rows' overflows (no size recorded) are escalated past every class
             const bool escalate = esc_shift > 0 && n_ovf > 0 && !fwork;
             if (escalate) {
@@ -2247,10 +2254,7 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                     SG_TRY(mark(esc_ovf, n_ovf2, 64, true));
                 }
             }
-            if (more || n_rt) {
-                SG_TRY(scans());
-                SG_CUDA_TRY(cudaStreamSynchronize(s));
-            }
+            if (more || n_rt) SG_TRY(scans());
             const int64_t nnz = upper ? 2 * nnz_u : nnz_u;  // C = U + U^T
             if (herr & DEV_TIMEOUT) return timeout_error("overlap_spgemm");
             if (herr) {
