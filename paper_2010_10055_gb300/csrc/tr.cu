@@ -550,24 +550,26 @@ sg_status tr_impl(const sg_graph_csr *R, uint32_t fuzz, int mode, sg_graph_csr *
     const int64_t n = R->n, nnz0 = R->nnz;
     StageScope stage("TrReduction", s);
     Scratch sc(s);
-    uint32_t *err = sc.get<uint32_t>(1);
+    // row pointers of a round's result, each with an error word behind its last, so that one copy reads
+    // both back (a copy to the host waits for the stream); the first round takes rp[1] and validates
+    int64_t *rp[2] = {nullptr, sc.get<int64_t>(2 * (n + 2))};
     uint8_t *keep = sc.get<uint8_t>(nnz0 + 1);
     int64_t *kept = sc.get<int64_t>(n + 1);
-    if (!err || !keep || !kept) return SG_ERR_OOM;
+    if (!rp[1] || !keep || !kept) return SG_ERR_OOM;
+    rp[0] = rp[1] + n + 2;
+    uint32_t *const err = (uint32_t *)(rp[1] + n + 1), *const errs[2] = {(uint32_t *)(rp[0] + n + 1), err};
     TrWork wk;
     SG_TRY(tr_work_alloc(&wk, n, nnz0, (mode & 1) != SG_TR_DIRMATCH, sc));
     // the rounds' graphs: each reads one buffer and compacts into the other (the first reads the
-    // caller's arrays beside buffer 0); row pointers of a round's result
+    // caller's arrays beside buffer 0)
     TrBuf buf[2];
-    int64_t *rp[2];
     for (int b = 0; b < 2; b++) {
         buf[b].p = sc.get<uint64_t>(nnz0 + 1);
         buf[b].row = sc.get<uint4>(n + 1);
-        rp[b] = sc.get<int64_t>(n + 1);
-        if (!buf[b].p || !buf[b].row || !rp[b]) return SG_ERR_OOM;
+        if (!buf[b].p || !buf[b].row) return SG_ERR_OOM;
     }
     const TrGraph in{R->row_ptr, R->col, R->suffix, R->dir, n};
-    SG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
+    SG_CUDA_TRY(cudaMemsetAsync(err, 0, (size_t)(n + 3) * 8, s));  // both error words and what lies between
     SG_LAUNCH("validate_graph", validate_graph_kernel, blocks_for((n + 1) * 32, 256), 256, 0, s, in, nnz0, buf[0], err);
     TrPacked g{nullptr, buf[0].p, buf[0].row, n, in};
     const int64_t *grp = R->row_ptr;
@@ -584,11 +586,11 @@ sg_status tr_impl(const sg_graph_csr *R, uint32_t fuzz, int mode, sg_graph_csr *
         if (job_ro)
             SG_LAUNCH("tr_job_changes", job_changes_kernel, blocks_for(n, 256), 256, 0, s, grp,
                       (const int64_t *)kept, n, job_ro, njobs, it, job_last);
-        SG_TRY(exclusive_scan<int64_t>(kept, rp[nxt], n, s, err));
-        int64_t nnz2 = 0;
-        uint32_t herr = 0;
-        SG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        SG_CUDA_TRY(read_back(&nnz2, rp[nxt] + n, sizeof(int64_t), s));
+        SG_TRY(exclusive_scan<int64_t>(kept, rp[nxt], n, s, errs[nxt]));
+        int64_t end[2] = {0, 0};
+        SG_CUDA_TRY(read_back(end, rp[nxt] + n, sizeof(end), s));
+        const int64_t nnz2 = end[0];
+        const uint32_t herr = (uint32_t)end[1];
         if (herr & DEV_TIMEOUT) return timeout_error("transitive_reduce");
         if (herr) {
             set_error("graph does not satisfy the CSR contract (sorted unique columns, no diagonal, suffix < 2^30, dir <= 3)");
