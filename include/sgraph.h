@@ -410,7 +410,7 @@ void sg_free(void *d_ptr, sg_stream_t stream);
 const char *sg_last_error(void);
 
 /* Optional device allocator (e.g. a framework's caching allocator). alloc returns NULL on
- * failure, else a pointer aligned to 256 bytes as cudaMalloc's are (the kernels use 16-byte
+ * failure, else a pointer aligned to 256 bytes as cudaMalloc's are (the kernels use up to 32-byte
  * vector accesses; a less aligned pointer fails the call with SG_ERR_OOM and a message). Pass
  * NULLs to restore cudaMallocAsync / cudaFreeAsync. Not thread-safe to change while calls are
  * running. */
