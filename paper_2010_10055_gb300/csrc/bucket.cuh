@@ -98,6 +98,10 @@ struct KbPlan {
     uint32_t *count2;             // [nsub_max + 1]
     int64_t nsub_max;
     int64_t cap;                  // records a buffer holds
+    // error word of the call. The bucket ranges come from a scan whose waits are bounded: when one has run
+    // out they overlap and a bucket holds records of others, whose bits are no indices any more, so
+    // every kernel that uses the ranges returns where the word is set.
+    const uint32_t *err;
     // the bucket's prefix, its first code (below the prefix) and its code bits
     __device__ __forceinline__ int prefix(int64_t b) const { return two ? (int)sub2p[b] : (int)b; }
 };
@@ -247,6 +251,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter2_kernel(KbPlan pl, const 
         }
     };
     load(a0);
+    if (*pl.err) return;  // tested behind the loads: their latency hides its own
     for (int64_t t0 = a0; t0 < a1; t0 += TILE) {
         for (int i = threadIdx.x; i < nb; i += KB_NT) cnt[i] = 0;
         __syncthreads();

@@ -767,6 +767,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const
     FinishSmem<K> &sm = *reinterpret_cast<FinishSmem<K> *>(kb_raw);
     constexpr int TILE = kb_tile<K>();
     const KbPlan &pl = a.pl;
+    if (*pl.err) return;
     const int64_t nsub = pl.two ? (int64_t)pl.sb[pl.nb1] : (int64_t)pl.nb1;
     const int64_t *start = pl.two ? pl.start2 : pl.start1;
     if (!COUNT && blockIdx.x == 0 && threadIdx.x == 0) a.rp[a.n_rows] = a.nnz;
@@ -985,7 +986,8 @@ static int bits_for(int64_t n) {  // bits of the ids 0 .. n - 1
 // A plan for `records` records with code bits `cb` above the prefix's end: prefix bits, whether a
 // second level is needed, and the device arrays (one allocation).
 static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t records, int tile, int target, int b2min,
-                           Scratch &sc) {
+                           Scratch &sc, const uint32_t *err) {
+    pl.err = err;
     pl.nb1 = 1 << pb1;
     pl.rem = cb - pb1;
     pl.two = two ? 1 : 0;
@@ -1055,7 +1057,7 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     // block's records, half of them would not fit: two parts each (12 Mbp, k = 31, rows of 7,200: 4.6 ms
     // -> 3.7; rows of 4,400, 100 Mbp: parts 31 ms, rows 22)
     const int target = nnz / n > kb_target<K>() / 4 * 3 ? kb_target<K>() / 2 : kb_target<K>();
-    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, target, b2min, sc));
+    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, target, b2min, sc, err));
     const int64_t ntiles = blocks_for(nnz, TILE);
     int32_t *tcol = sc.get<int32_t>(ntiles);
     typename K::T *r0 = sc.get<typename K::T>(nnz), *r1 = two ? sc.get<typename K::T>(nnz) : nullptr;
@@ -1128,7 +1130,7 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
     using T = typename K::T;
     constexpr int TILE = kb_tile<K>();
     KbPlan pl;
-    SG_TRY(make_plan(pl, q.pb1, q.cb, q.two, q.total, TILE, kb_target<K>(), 0, sc));
+    SG_TRY(make_plan(pl, q.pb1, q.cb, q.two, q.total, TILE, kb_target<K>(), 0, sc, err));
     SG_LAUNCH("kmer_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, kb_target<K>(),
               q.two ? std::min(KB_MAXB2, pl.rem) : 0, 0, KB_CHUNK_TILES * TILE);
     T *r0 = sc.get<T>(q.total), *r1 = sc.get<T>(q.total);
