@@ -421,11 +421,11 @@ void sg_set_allocator(sg_alloc_fn alloc, sg_free_fn release, void *ctx);
 /* Test hook: make the n-th device allocation from now fail (n >= 1); 0 disables. */
 void sg_debug_fail_alloc_after(int64_t n);
 
-/* Test hook for the bounded waits between thread blocks. While on, every scan of more than one
- * tile has its first tile withhold its prefix: the waits of the later tiles give up after their
- * poll limit (well under a second each), set the call's device error word, and the call returns
- * SG_ERR_TIMEOUT with its outputs freed. Nothing hangs and the context stays usable. Off by
- * default; affects all threads. */
+/* Test hook for the bounded waits between thread blocks. While on, every scan and every radix sort
+ * pass of more than one tile has its first tile withhold its prefix: the waits of the later tiles give
+ * up after their poll limit (well under a second each), set the call's device error word, and the
+ * call returns SG_ERR_TIMEOUT with its outputs freed. Nothing hangs and the context stays usable.
+ * Off by default; affects all threads. */
 void sg_debug_stall_lookback(int on);
 
 /* Checked builds (compiled with -DSG_CHECKED): the first out-of-bounds index any kernel detected

@@ -553,13 +553,17 @@ struct BucketStarts {
     int shift;
 };
 
+// The kernels below use bits of sorted keys, or scanned counts, as indices before the host has seen the
+// call's error word: a sort or scan whose wait ran out leaves words that nobody wrote, so they return where
+// the word is set.
+
 // After a keys-only sort (PK_POS, PK_IDX): the code, and the window resolved to its read.
 __global__ void unpack_kernel(const uint64_t *__restrict__ packed, const uint64_t *__restrict__ vals, int64_t nc,
                               int mode, int pb, BucketStarts bs, const int64_t *__restrict__ off, int64_t n,
                               const int32_t *__restrict__ lut, int64_t nb, uint64_t *__restrict__ key,
-                              uint64_t *__restrict__ val) {
+                              uint64_t *__restrict__ val, const uint32_t *__restrict__ err) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
+    if (i >= nc || *err) return;
     const uint64_t p = packed[i];
     const uint64_t low = p & ((1ull << pb) - 1);
     uint64_t b = 0;  // the bucket's bits above the sorted code bits
@@ -576,9 +580,9 @@ __global__ void unpack_kernel(const uint64_t *__restrict__ packed, const uint64_
 
 // After the pairs sort: val = q | strand << 63  ->  read << 32 | pos | strand << 31.
 __global__ void resolve_kernel(uint64_t *__restrict__ val, int64_t nc, const int64_t *__restrict__ off, int64_t n,
-                               const int32_t *__restrict__ lut, int64_t nb) {
+                               const int32_t *__restrict__ lut, int64_t nb, const uint32_t *__restrict__ err) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
+    if (i >= nc || *err) return;
     val[i] = resolve_pos(val[i], off, n, lut, nb);
 }
 
@@ -603,9 +607,9 @@ __global__ void seg_start_kernel(const uint32_t *__restrict__ head, const int64_
 __global__ void seg_reliable_kernel(const int64_t *__restrict__ seg_start, const int64_t *__restrict__ nseg_p,
                                     uint32_t lo, uint32_t hi, const uint64_t *__restrict__ key,
                                     const uint32_t *__restrict__ lohi, int kbits, int64_t nc,
-                                    uint32_t *__restrict__ rel) {
+                                    uint32_t *__restrict__ rel, const uint32_t *__restrict__ err) {
     int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s > nc) return;
+    if (s > nc || *err) return;
     int64_t nseg = *nseg_p;
     if (s >= nseg) {  // slots past the last segment still feed the scan below: make them 0
         rel[s] = 0u;
@@ -623,9 +627,9 @@ __global__ void seg_reliable_kernel(const int64_t *__restrict__ seg_start, const
 // keep[i]: i lies in a reliable segment and is the first (lowest position) entry of its read.
 __global__ void keep_kernel(const uint32_t *__restrict__ head, const int64_t *__restrict__ seg_excl,
                             const uint32_t *__restrict__ rel, const uint64_t *__restrict__ val, int64_t nc,
-                            uint32_t *__restrict__ keep) {
+                            uint32_t *__restrict__ keep, const uint32_t *__restrict__ err) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
+    if (i >= nc || *err) return;
     int64_t s = seg_excl[i] + head[i] - 1;
     bool first = head[i] || ((val[i] >> 32) != (val[i - 1] >> 32));
     keep[i] = (rel[s] && first) ? 1u : 0u;
@@ -673,8 +677,10 @@ constexpr int PK_SHIFT = 31;
 // scan.
 __global__ void seg_flags_kernel(const uint64_t *__restrict__ key, const uint64_t *__restrict__ val, int64_t nc,
                                  uint32_t lo, uint32_t hi, const uint32_t *__restrict__ lohi, int kbits, int hmax,
-                                 uint64_t *__restrict__ packed, unsigned long long *__restrict__ nkeep) {
+                                 uint64_t *__restrict__ packed, unsigned long long *__restrict__ nkeep,
+                                 const uint32_t *__restrict__ err) {
     __shared__ unsigned int s_kept;
+    if (*err) return;
     if (threadIdx.x == 0) s_kept = 0u;
     __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -848,6 +854,7 @@ struct SegArgs {
     int64_t n;
     const int32_t *lut;
     int64_t nb;
+    const uint32_t *err;
 };
 
 __global__ void __launch_bounds__(DS_NT) seg_mark_kernel(SegArgs a, uint32_t *__restrict__ flags,
@@ -857,6 +864,7 @@ __global__ void __launch_bounds__(DS_NT) seg_mark_kernel(SegArgs a, uint32_t *__
     const int64_t tile = blockIdx.x, base = tile * DS_TILE;
     stage_keys(sk, a.packed, base, a.nc);
     __syncthreads();
+    if (*a.err) return;
     // indices below are local: candidate base - DS_HALO + x is staged at sk[ds_pad(x)]
     const int l0 = DS_HALO + threadIdx.x * DS_ITEMS;
     const int64_t g0 = base - DS_HALO;
@@ -1359,7 +1367,8 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
             uint32_t *tcount = sc.get<uint32_t>(2 * ntiles);
             dpre = sc.get<int64_t>(2 * (ntiles + 1));
             if (!dflags || !tcount || !dpre) return SG_ERR_OOM;
-            dargs = SegArgs{sorted, nc, pb, bs, lo, hi, lohi, 2 * k, (int)hmax, off, n, (const int32_t *)lut, nlut};
+            dargs = SegArgs{sorted, nc, pb, bs, lo, hi, lohi, 2 * k, (int)hmax, off, n, (const int32_t *)lut, nlut,
+                            (const uint32_t *)err};
             SG_LAUNCH("seg_mark", seg_mark_kernel, ntiles, DS_NT, 0, s, dargs, dflags, tcount, tcount + ntiles);
             SG_TRY(exclusive_scan<uint32_t>(tcount, dpre, ntiles, s, err));
             SG_TRY(exclusive_scan<uint32_t>(tcount + ntiles, dpre + ntiles + 1, ntiles, s, err));
@@ -1373,7 +1382,8 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
             val1 = sc.get<uint64_t>(nc);
             if (!val1) return SG_ERR_OOM;
             SG_LAUNCH("unpack", unpack_kernel, blocks_for(nc, NT), NT, 0, s, (const uint64_t *)ks,
-                      (const uint64_t *)val0, nc, mode, pb, bs, off, n, (const int32_t *)lut, nlut, kfree, val1);
+                      (const uint64_t *)val0, nc, mode, pb, bs, off, n, (const int32_t *)lut, nlut, kfree, val1,
+                      (const uint32_t *)err);
             key = kfree;
             val = val1;
             sc.release(ks);
@@ -1386,7 +1396,7 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         sc.release(alt ? key0 : key1);
         sc.release(alt ? val0 : val1);
         SG_LAUNCH("resolve", resolve_kernel, blocks_for(nc, NT), NT, 0, s, val, nc, off, n, (const int32_t *)lut,
-                  nlut);
+                  nlut, (const uint32_t *)err);
     }
 
     // segments -> exact frequency -> reliable -> columns; kept entries -> At
@@ -1403,7 +1413,7 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         if (!pre || !nkeep) return SG_ERR_OOM;
         SG_CUDA_TRY(cudaMemsetAsync(nkeep, 0, sizeof(unsigned long long), s));
         SG_LAUNCH("seg_flags", seg_flags_kernel, blocks_for(nc, NT), NT, 0, s, key, (const uint64_t *)val, nc, lo, hi,
-                  lohi, 2 * k, (int)hmax, pre, nkeep);
+                  lohi, 2 * k, (int)hmax, pre, nkeep, (const uint32_t *)err);
         unsigned long long hk = 0;
         SG_CUDA_TRY(read_back(&hk, nkeep, sizeof(hk), s));
         if (hk >= (1ull << PK_SHIFT)) {  // too many kept entries for the packed scan
@@ -1435,9 +1445,10 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         SG_LAUNCH("seg_start", seg_start_kernel, blocks_for(nc, NT), NT, 0, s, head, seg_excl, nc, seg_start);
         // number of segments lives on the device at seg_excl[nc]; launch over the upper bound nc
         SG_LAUNCH("seg_reliable", seg_reliable_kernel, blocks_for(nc, NT), NT, 0, s, seg_start, seg_excl + nc, lo,
-                  hi, key, lohi, 2 * k, nc, rel);
+                  hi, key, lohi, 2 * k, nc, rel, (const uint32_t *)err);
         SG_TRY(exclusive_scan<uint32_t>(rel, col_of_seg, nc, s, err));
-        SG_LAUNCH("keep", keep_kernel, blocks_for(nc, NT), NT, 0, s, head, seg_excl, rel, val, nc, keep);
+        SG_LAUNCH("keep", keep_kernel, blocks_for(nc, NT), NT, 0, s, head, seg_excl, rel, val, nc, keep,
+                  (const uint32_t *)err);
         SG_TRY(exclusive_scan<uint32_t>(keep, out_pos, nc, s, err));
         // m = reliable segments = col_of_seg[nc] (rel is 0 past the last segment)
         SG_CUDA_TRY(cudaMemcpyAsync(&sizes[0], col_of_seg + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));

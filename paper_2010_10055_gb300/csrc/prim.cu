@@ -59,23 +59,32 @@ struct RsSmem {
     uint32_t tstart[RS_RADIX];
     uint32_t tmp[RS_WARPS + 1];
     unsigned int tile;
+    uint32_t stop;
 };
 
 // ghist: this pass's 256 digit totals; status: [ntiles][256] look-back words, zeroed; tile_ctr:
 // zeroed. Without values (HAS_V == false) vin / vout are not touched.
+// A wait that runs out leaves places of the output unwritten; within the pass every place stays in
+// range, but a later pass would count digits that the totals do not know. So a tile that finds the error
+// word set returns, and whoever reads the sorted arrays has to look at the word first.
+// stall != 0 (test hook, sg_debug_stall_lookback): tile 0 withholds its counts.
 template <class K, class V, bool HAS_V, bool MATCH>
 __global__ void __launch_bounds__(RS_NT, HAS_V ? 3 : 4) radix_onesweep_kernel(const K *__restrict__ kin, const V *__restrict__ vin,
                                                               K *__restrict__ kout, V *__restrict__ vout,
                                                               int64_t n, int shift,
                                                               const unsigned long long *__restrict__ ghist,
                                                               unsigned long long *status, unsigned int *tile_ctr,
-                                                              uint32_t *err, int lbw) {
+                                                              uint32_t *err, int lbw, int stall) {
     extern __shared__ __align__(16) unsigned char rs_raw[];
     RsSmem<K, V, HAS_V> &sm = *reinterpret_cast<RsSmem<K, V, HAS_V> *>(rs_raw);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) sm.tile = atomicAdd(tile_ctr, 1u);
+    if (threadIdx.x == 0) {
+        sm.tile = atomicAdd(tile_ctr, 1u);
+        sm.stop = err ? *(volatile uint32_t *)err : 0u;
+    }
     for (int i = threadIdx.x; i < RS_WARPS * RS_RADIX; i += RS_NT) (&sm.wcnt[0][0])[i] = 0;
     __syncthreads();
+    if (sm.stop) return;
     const int64_t tile = sm.tile;
     const int64_t tbase = tile * RS_TILE;
     const int64_t wbase = tbase + (int64_t)w * 32 * RS_ITEMS;
@@ -126,7 +135,7 @@ __global__ void __launch_bounds__(RS_NT, HAS_V ? 3 : 4) radix_onesweep_kernel(co
     unsigned long long *mine = status + tile * RS_RADIX + d;
     int64_t excl = 0;
     if (tile == 0) {
-        lb_store(mine, LB_P | tot);
+        if (!stall) lb_store(mine, LB_P | tot);
     } else {
         lb_store(mine, LB_A | tot);
         // walk back lbw predecessors at a time: their words are read together, and only a word not
@@ -215,12 +224,12 @@ static sg_status radix_sort_impl(K *k0, V *v0, K *k1, V *v1, int64_t n, int lo_b
             SG_LAUNCH("radix_onesweep", (radix_onesweep_kernel<K, V, HAS_V, true>), ntiles, RS_NT, smem, s,
                       (const K *)ki, (const V *)vi, ko, vo, n, lo_bit + RS_BITS * p,
                       (const unsigned long long *)(ghist + p * RS_RADIX), status + (size_t)p * ntiles * RS_RADIX,
-                      ctr + p, err, lbw);
+                      ctr + p, err, lbw, debug_stall_lookback());
         else
             SG_LAUNCH("radix_onesweep", (radix_onesweep_kernel<K, V, HAS_V, false>), ntiles, RS_NT, smem, s,
                       (const K *)ki, (const V *)vi, ko, vo, n, lo_bit + RS_BITS * p,
                       (const unsigned long long *)(ghist + p * RS_RADIX), status + (size_t)p * ntiles * RS_RADIX,
-                      ctr + p, err, lbw);
+                      ctr + p, err, lbw, debug_stall_lookback());
         K *tk = ki; ki = ko; ko = tk;
         V *tv = vi; vi = vo; vo = tv;
         *in_alt = !*in_alt;

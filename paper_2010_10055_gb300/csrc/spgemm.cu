@@ -1661,9 +1661,9 @@ __global__ void lower_rec_kernel(const uint64_t *__restrict__ mval, int64_t nu, 
                                  const int64_t *__restrict__ c_rp, int64_t n, int64_t nnz, int S,
                                  int32_t *__restrict__ c_col, uint32_t *__restrict__ c_cnt,
                                  uint32_t *__restrict__ c_si, uint32_t *__restrict__ c_sk,
-                                 const MirrorRec *__restrict__ mrec) {
+                                 const MirrorRec *__restrict__ mrec, const uint32_t *__restrict__ err) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nu) return;
+    if (q >= nu || *err) return;  // a sort that timed out leaves words that are no list
     const uint64_t v = mval[q];
     const int64_t k = (int64_t)(v >> pb), p = (int64_t)(v & ((1ull << pb) - 1));
     if (!SG_IN_BOUNDS(k < n && p < nu, 312, q)) return;
@@ -1688,9 +1688,10 @@ __global__ void lower_rec_kernel(const uint64_t *__restrict__ mval, int64_t nu, 
 __global__ void lower_fill_kernel(const uint32_t *__restrict__ mkey, const uint64_t *__restrict__ mval, int64_t nu,
                                   const int64_t *__restrict__ lrp, const int64_t *__restrict__ c_rp, int64_t n,
                                   int64_t nnz, int S, int32_t *__restrict__ c_col, uint32_t *__restrict__ c_cnt,
-                                  uint32_t *__restrict__ c_si, uint32_t *__restrict__ c_sk) {
+                                  uint32_t *__restrict__ c_si, uint32_t *__restrict__ c_sk,
+                                  const uint32_t *__restrict__ err) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nu) return;
+    if (q >= nu || *err) return;
     const uint32_t k = mkey[q];
     const uint64_t v = mval[q];
     const int64_t i = (int64_t)(v >> MIRROR_POS_BITS), p = (int64_t)(v & ((1ull << MIRROR_POS_BITS) - 1));
@@ -2304,13 +2305,13 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                     SG_LAUNCH("lower_fill", lower_rec_kernel, blocks_for(nnz_l, 256), 256, 0, s,
                               (const uint64_t *)(alt ? mv1 : mv0), nnz_l, pb, (const int64_t *)lrp,
                               (const int64_t *)C->row_ptr, n, nnz, S, C->col, C->count, C->seed_i, C->seed_k,
-                              (const MirrorRec *)mrec);
+                              (const MirrorRec *)mrec, (const uint32_t *)err);
                 } else {
                     SG_TRY((radix_sort_pairs<uint32_t, uint64_t>(mk0, mv0, mk1, mv1, nnz_l, kbits, &alt, s, err)));
                     SG_LAUNCH("lower_fill", lower_fill_kernel, blocks_for(nnz_l, 256), 256, 0, s,
                               (const uint32_t *)(alt ? mk1 : mk0), (const uint64_t *)(alt ? mv1 : mv0), nnz_l,
                               (const int64_t *)lrp, (const int64_t *)C->row_ptr, n, nnz, S, C->col, C->count, C->seed_i,
-                              C->seed_k);
+                              C->seed_k, (const uint32_t *)err);
                 }
                 SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));  // the sort waits between tiles
                 if (herr & DEV_TIMEOUT) return timeout_error("overlap_spgemm");

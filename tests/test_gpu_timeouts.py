@@ -1,11 +1,13 @@
-"""A bounded wait that runs out inside the bucketed k-mer stage, without faulting the GPU: the bucket
-ranges come from a multi-tile scan, and nothing may work on them once the scan has given up. With the test
-hook on, the call ends in SG_ERR_TIMEOUT; the same call is right again afterwards."""
+"""Bounded waits that run out in scans and radix sorts whose outputs later kernels of the call use as
+indices, without faulting the GPU: nothing may work on them once a wait has given up. With the test hook on,
+the call ends in SG_ERR_TIMEOUT; the same call is right again afterwards."""
 import numpy as np
 import pytest
 import torch
 
 import paper_2010_10055_gb300 as sg
+import synth
+from tests.gpu_util import dev
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +54,32 @@ def test_bucket_ranges_of_rows():
     off = torch.full((n + 1,), total, dtype=torch.int64, device="cuda")
     off[:401] = torch.arange(0, total + 1, 1000, device="cuda")
     _stalled_then_exact(lambda: _tensors(sg.build_kmer_matrix(seq, off, 17, 2, 8)))
+
+
+@pytest.fixture
+def tuned():
+    saved = sg.tunables()
+    yield lambda **kw: [sg.tune(name, v) for name, v in kw.items()]
+    for name, v in saved.items():
+        sg.tune(name, v)
+
+
+# sorted windows by position, by index and in pairs; segments from the sorted keys, from unpacked ones and
+# (hi beyond the walk bound) without the packed flags
+@pytest.mark.parametrize("k,hi,cfg", [(17, 8, {}), (17, 8, {"kmer_direct_seg": 0}), (17, 5000, {}), (31, 8, {}),
+                                      (23, 8, {"kmer_sort_buckets": 0}), (23, 5000, {"kmer_sort_buckets": 0})])
+def test_radix_of_windows(tuned, k, hi, cfg):
+    tuned(kmer_bucketed=0, **cfg)
+    seq = _bases(3, 100_000).repeat(2)
+    off = torch.arange(0, 200_001, 2000, device="cuda")
+    _stalled_then_exact(lambda: _tensors(sg.build_kmer_matrix(seq, off, k, 2, hi)))
+
+
+@pytest.mark.parametrize("rec", [0, 1])
+def test_radix_of_the_mirror(tuned, rec):
+    """Fewer than 4,096 reads (single-tile scans), more than 4,096 mirrored entries."""
+    tuned(spgemm_mirror_rec=rec)
+    d = synth.make(synth.BACTERIAL.scaled(0.1))
+    km = sg.build_kmer_matrix(dev(d["seq"], np.uint8), dev(d["offsets"], np.int64), 17, 2, 20)
+    assert km.A.shape[0] < 4096 and sg.overlap_spgemm(km, 2, 2).nnz > 3 * 4096
+    _stalled_then_exact(lambda: [t.clone() for t in sg.overlap_spgemm(km, 2, 2).tensors().values()])
