@@ -31,10 +31,11 @@ struct KeyBits {
     __host__ __device__ int low() const { return rbits + pbits + 1; }
 };
 
-// The low 32 bits of x >> s (0 <= s < 64), in two instructions where s is the same for all lanes.
+// The low 32 bits of x >> s (0 <= s <= 64; 64: a prefix that is not split, of records that fill their
+// word), in two instructions where s is the same for all lanes. The clamped shift is defined at 32.
 __device__ __forceinline__ uint32_t low_bits_at(uint64_t x, int s) {
     const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
-    return s < 32 ? __funnelshift_r(lo, hi, s) : hi >> (s - 32);
+    return s < 32 ? __funnelshift_r(lo, hi, s) : __funnelshift_rc(hi, 0u, s - 32);
 }
 
 struct KeyN {  // one word: code << low | read << (pbits + 1) | pos << 1 | strand
