@@ -99,10 +99,13 @@ struct KbPlan {
     uint32_t *count2;             // [nsub_max + 1]
     int64_t nsub_max;
     int64_t cap;                  // records a buffer holds
-    // error word of the call. The bucket ranges come from a scan whose waits are bounded: when one has run
-    // out they overlap and a bucket holds records of others, whose bits are no indices any more, so
-    // every kernel that uses the ranges returns where the word is set.
-    const uint32_t *err;
+    // Two words: the call's errors, and whether a bucket holds more than `limit` records. The bucket ranges
+    // come from a scan whose waits are bounded: when one has run out they overlap and a bucket holds records
+    // of others, whose bits are no indices any more. Every kernel that uses the ranges returns where
+    // either is set.
+    uint32_t *stop;
+    int64_t limit;
+    __device__ __forceinline__ bool stopped() const { return (stop[0] | stop[1]) != 0; }
     // the bucket's prefix, its first code (below the prefix) and its code bits
     __device__ __forceinline__ int prefix(int64_t b) const { return two ? (int)sub2p[b] : (int)b; }
 };
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter2_kernel(KbPlan pl, const 
         }
     };
     load(a0);
-    if (*pl.err) return;  // tested behind the loads: their latency hides its own
+    if (pl.stopped()) return;  // tested behind the loads: their latency hides its own
     for (int64_t t0 = a0; t0 < a1; t0 += TILE) {
         for (int i = threadIdx.x; i < nb; i += KB_NT) cnt[i] = 0;
         __syncthreads();
@@ -279,8 +282,17 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter2_kernel(KbPlan pl, const 
 __device__ __forceinline__ int slot_pad(int w) { return w + (w >> 4) * 4; }
 constexpr int KB_SLOT_WORDS = (1 << (KB_NS - 1)) + (1 << (KB_NS - 3)) + 8;
 
-constexpr int KB_STACK = 8;    // nested refinements of an oversized bucket (13 code bits each)
-constexpr int KB_GROUPS = 64;  // slot ranges taken from one count of an oversized bucket
+constexpr int KB_PIECE_BITS = 13;  // code bits by which a piece too large for a block is split, at most
+constexpr int KB_PIECES = 112;     // pending pieces of an oversized bucket
+
+// Records [off, off + len) of an oversized bucket with codes in [c0, cend), in the bucket's range of the
+// input (where == 0) or of the other buffer. len above a block's records: they agree in the code bits
+// from `bits` on; split: they are in order of the next KB_PIECE_BITS already.
+struct KbPiece {
+    uint64_t c0, cend;
+    uint32_t off, len;
+    uint8_t bits, where, split;
+};
 
 template <class K>
 struct FinishSmem {
@@ -290,12 +302,9 @@ struct FinishSmem {
     uint32_t heads[KB_NT * K::ITEMS / 32 + 2];   // bit i + 32: record i of sk starts a slot
     uint32_t codes[KB_NT * K::ITEMS / 32 + 2];   // ... (in order) a code
     uint32_t tmp[KB_NT / 32 + 1];
-    uint32_t nseg, nst;
-    uint64_t f_base[KB_STACK];  // refinement frames: codes with code >> f_bits == f_base, from slot f_a
-    int f_bits[KB_STACK];
-    int f_a[KB_STACK];
-    int g_a[KB_GROUPS], g_z[KB_GROUPS];
-    int ng, child;
+    uint32_t nseg;
+    int npiece;
+    KbPiece piece[KB_PIECES];
 };
 
 }  // namespace sg

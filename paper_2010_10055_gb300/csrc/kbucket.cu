@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(1024) kb_plan_kernel(const unsigned long long 
         const int64_t st = s_base + block_exclusive_scan<1024, int64_t>(c, t64, &tot);
         const uint32_t sub = s_sub + block_exclusive_scan<1024, uint32_t>(p < pl.nb1 ? 1u << b : 0u, t32, &stot);
         const uint32_t chk = s_chk + block_exclusive_scan<1024, uint32_t>(nch, t32, &ctot);
+        if (!pl.two && c > pl.limit) pl.stop[1] = 1;
         if (p < pl.nb1) {
             pl.start1[p] = st;
             pl.cur1[p] = (unsigned long long)st;
@@ -86,6 +87,14 @@ __global__ void kb_sub2p_kernel(KbPlan pl) {
     for (uint32_t x = pl.sb[p] + (threadIdx.x & 31); x < pl.sb[p + 1]; x += 32)
         if (SG_IN_BOUNDS((int64_t)x < pl.nsub_max, 701, x)) pl.sub2p[x] = (uint16_t)p;
     for (uint32_t x = pl.chunk2[p] + (threadIdx.x & 31); x < pl.chunk2[p + 1]; x += 32) pl.chunk2p[x] = (uint16_t)p;
+}
+
+// Level-2 write cursors, and whether a bucket is too large for one block.
+__global__ void kb_cursors_kernel(KbPlan pl) {
+    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= pl.nsub_max) return;
+    pl.cur2[b] = (unsigned long long)pl.start2[b];
+    if ((int64_t)pl.count2[b] > pl.limit) pl.stop[1] = 1;
 }
 
 // ----------------------------------------------------------------------------------- pack
@@ -637,137 +646,173 @@ __device__ __forceinline__ uint32_t finish_group(FinishSmem<K> &sm, const Finish
     }
 }
 
-// A bucket of more records than a block holds: its codes are split into ranges that fit, counted
-// over the whole bucket (13 code bits at a time, refined where one slot alone is too full) and
-// finished in code order. A single code with more records than a block holds is skipped: in the
-// count pass its frequency is above every hi taken here, and A's (read, column) pairs are distinct.
+// A bucket of more records than a block holds, split by its block: the records are ordered by their next
+// code bits (counted, then moved to the same range of the other buffer), runs of slots that fit are finished
+// in code order, and a slot that does not fit is split again the same way, back and forth between the
+// buffers. Every level reads the records twice and writes them once, whatever their number (choosing the
+// runs from counts alone and searching the whole bucket for each run's records read a bucket of n records
+// n / 8192 times: a contig of 8 Mbp among reads 7.7 s instead of 20 ms). Results go to the front of the
+// bucket's own range of `out`, which may be `alt`: no more are written than records taken. A single code
+// with more records than a block holds is skipped: in the count pass its frequency is above every hi taken
+// here, and A's (read, column) pairs are distinct.
+template <class K> __device__ __forceinline__ typename K::T load_moved(const typename K::T *p);
+template <> __device__ __forceinline__ uint64_t load_moved<KeyN>(const uint64_t *p) {
+    return *reinterpret_cast<const volatile uint64_t *>(p);
+}
+template <> __device__ __forceinline__ U128 load_moved<KeyW>(const U128 *p) {
+    const volatile uint64_t *q = reinterpret_cast<const volatile uint64_t *>(p);
+    return U128{q[0], q[1]};
+}
+
 template <class K, bool COUNT>
-__device__ __noinline__ uint2 finish_big(FinishSmem<K> &sm, const FinishArgs &a, int p,
-                                         const typename K::T *__restrict__ in, int64_t n, uint64_t c0, int bits,
-                                         int64_t base, typename K::T *__restrict__ out) {
+__device__ __noinline__ uint2 finish_big(FinishSmem<K> &sm, const FinishArgs &a, int p, typename K::T *in,
+                                         typename K::T *alt, int64_t n, uint64_t c0, int bits, int64_t base,
+                                         typename K::T *out) {
     using T = typename K::T;
-    constexpr int TILE = kb_tile<K>();
-    const int lowbits = a.kb.low();
+    constexpr int TILE = kb_tile<K>(), U = 8;  // loads in flight
+    const int lowbits = a.kb.low(), tid = threadIdx.x, lane = tid & 31;
     uint32_t done = 0, segs = 0;
-    uint32_t *cnt = sm.slots;  // [2^13 + 1], exclusive prefixes after the scan
-    if (threadIdx.x == 0) {
-        sm.nst = 1;
-        sm.f_base[0] = bits < 64 ? c0 >> bits : 0;
-        sm.f_bits[0] = bits;
-        sm.f_a[0] = 0;
+    uint32_t *first = sm.slots;                                // [2^13 + 1] first record of each slot
+    uint32_t *cur = reinterpret_cast<uint32_t *>(sm.sk);       // [2^13] where its next record goes
+    static_assert(sizeof(sm.sk) >= sizeof(uint32_t) << KB_PIECE_BITS, "cursors in the records' place");
+    if (tid == 0) {
+        sm.piece[0] = KbPiece{c0, c0 + (1ull << bits), 0u, (uint32_t)n, (uint8_t)bits, 0, 0};
+        sm.npiece = 1;
     }
     __syncthreads();
     for (;;) {
-        const int top = (int)sm.nst - 1;
+        const int top = sm.npiece - 1;
         if (top < 0) break;
-        const uint64_t fb = sm.f_base[top];
-        const int fbits = sm.f_bits[top], fa = sm.f_a[top];
-        const int ls = fbits < 13 ? fbits : 13, sh = fbits - ls, NS = 1 << ls;
+        const KbPiece w = sm.piece[top];
+        T *src = (w.where ? alt : in) + w.off;
         __syncthreads();
-        if (fa >= NS) {
-            if (threadIdx.x == 0) sm.nst--;
-            __syncthreads();
-            continue;
-        }
-        for (int i = threadIdx.x; i <= NS; i += KB_NT) cnt[i] = 0;
-        __syncthreads();
-        auto in_frame = [&](uint64_t c) { return fbits >= 64 || (c >> fbits) == fb; };
-        auto slot_of = [&](uint64_t c) { return (int)((c >> sh) & (uint64_t)(NS - 1)); };
-        for (int64_t i = threadIdx.x; i < n; i += KB_NT) {
-            const uint64_t c = K::code(K::load(in + i), lowbits);
-            if (in_frame(c)) atomicAdd(cnt + slot_of(c), 1u);
-        }
-        __syncthreads();
-        {
-            const int per = (NS + KB_NT - 1) / KB_NT, i0 = threadIdx.x * per;
-            uint32_t s = 0, tot;
-            for (int i = i0; i < i0 + per && i < NS; i++) s += cnt[i];
-            uint32_t ex = block_exclusive_scan<KB_NT>(s, sm.tmp, &tot);
-            for (int i = i0; i < i0 + per && i < NS; i++) {
-                const uint32_t c = cnt[i];
-                cnt[i] = ex;
-                ex += c;
+        if (w.len <= (uint32_t)TILE) {
+            if (tid == 0) {
+                sm.npiece = top;
+                sm.nseg = 0;
             }
-            if (threadIdx.x == 0) cnt[NS] = tot;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int x = fa, ng = 0;
-            sm.child = -1;
-            while (x < NS && ng < KB_GROUPS) {
-                if (cnt[x + 1] - cnt[x] > (uint32_t)TILE) {
-                    if (sh == 0) {  // one code
-                        x++;
-                        continue;
-                    }
-                    if (ng == 0) sm.child = x++;
-                    break;
-                }
-                int lo = x + 1, hi = NS;  // largest z with the records of [x, z) fitting
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (cnt[mid] - cnt[x] <= (uint32_t)TILE) lo = mid; else hi = mid - 1;
-                }
-                sm.g_a[ng] = x;
-                sm.g_z[ng] = lo;
-                ng++;
-                x = lo;
-            }
-            sm.ng = ng;
-            sm.f_a[top] = x;
-            if (sm.child >= 0) {
-                sm.f_base[top + 1] = (fb << ls) | (uint64_t)sm.child;
-                sm.f_bits[top + 1] = sh;
-                sm.f_a[top + 1] = 0;
-                sm.nst++;
-            }
-        }
-        __syncthreads();
-        const int ng = sm.ng;
-        for (int g = 0; g < ng; g++) {
-            const int ga = sm.g_a[g], gz = sm.g_z[g];
-            if (threadIdx.x == 0) sm.nseg = 0;
-            __syncthreads();
-            // the range's records into shared memory, in any order, then into registers
-            for (int64_t i = threadIdx.x; i < n; i += KB_NT) {
-                const T k = K::load(in + i);
-                const uint64_t c = K::code(k, lowbits);
-                if (!in_frame(c)) continue;
-                const int s = slot_of(c);
-                if (s < ga || s >= gz) continue;
-                const uint32_t q = atomicAdd(&sm.nseg, 1u);
-                if (q < (uint32_t)TILE) sm.sk[q] = k;  // the counts say it fits
-            }
-            __syncthreads();
-            const int m = sm.nseg < (uint32_t)TILE ? (int)sm.nseg : TILE;
             T key[K::ITEMS];
 #pragma unroll
             for (int u = 0; u < K::ITEMS; u++) {
-                const int i = u * KB_NT + threadIdx.x;
-                key[u] = i < m ? sm.sk[i] : K::none();
+                const uint32_t i = u * KB_NT + tid;
+                key[u] = i < w.len ? load_moved<K>(src + i) : K::none();
             }
             __syncthreads();
-            const uint64_t r0 = ((fb << ls) | (uint64_t)ga) << sh;
-            const uint64_t width = (uint64_t)(gz - ga) << sh;
             int wb = 0;  // slots: the range's codes at up to 2^14 steps
-            while (((uint64_t)1 << wb) < width) wb++;
+            while (((uint64_t)1 << wb) < w.cend - w.c0) wb++;
             const int sh2 = wb > KB_NS ? wb - KB_NS : 0;
-            done += finish_group<K, COUNT>(sm, a, p, key, m, r0, r0 + width, sh2, wb - sh2, base + done, out);
+            done += finish_group<K, COUNT>(sm, a, p, key, (int)w.len, w.c0, w.cend, sh2, wb - sh2, base + done, out);
             segs += sm.nseg;
             __syncthreads();
+            continue;
         }
+        const int ls = w.bits < KB_PIECE_BITS ? w.bits : KB_PIECE_BITS, sh = w.bits - ls, NS = 1 << ls;
+        auto slot_of = [&](uint64_t c) { return (uint32_t)(c >> sh) & (uint32_t)(NS - 1); };
+        for (int i = tid; i <= NS; i += KB_NT) first[i] = 0;
+        __syncthreads();
+        for (uint32_t i = tid; i < w.len; i += U * KB_NT) {
+            T k[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) k[u] = i + u * KB_NT < w.len ? load_moved<K>(src + i + u * KB_NT) : K::none();
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (i + u * KB_NT < w.len) atomicAdd(first + slot_of(K::code(k[u], lowbits)), 1u);
+        }
+        __syncthreads();
+        {
+            const int per = (NS + KB_NT - 1) / KB_NT, i0 = tid * per;
+            uint32_t s = 0, tot;
+            for (int i = i0; i < i0 + per && i < NS; i++) s += first[i];
+            uint32_t ex = block_exclusive_scan<KB_NT>(s, sm.tmp, &tot);
+            for (int i = i0; i < i0 + per && i < NS; i++) {
+                const uint32_t c = first[i];
+                first[i] = ex;
+                cur[i] = ex;
+                ex += c;
+            }
+            if (tid == 0) first[NS] = tot;
+        }
+        __syncthreads();
+        if (!w.split) {
+            T *dst = (w.where ? in : alt) + w.off;
+            for (uint32_t i0 = 0; i0 < w.len; i0 += U * KB_NT) {
+                T k[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const uint32_t i = i0 + u * KB_NT + tid;
+                    k[u] = i < w.len ? load_moved<K>(src + i) : K::none();
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const bool have = i0 + u * KB_NT + tid < w.len;
+                    const uint32_t s = have ? slot_of(K::code(k[u], lowbits)) : ~0u;
+                    // the lanes that share the first lane's slot take one place together: a slot that
+                    // holds most of the records would serialise the warp
+                    const uint32_t s0 = __shfl_sync(0xffffffffu, s, 0);
+                    const uint32_t m = __ballot_sync(0xffffffffu, have && s == s0);
+                    if (m == 0) continue;  // no records (lane 0 has the first)
+                    uint32_t q = 0;
+                    if (lane == 0) q = atomicAdd(cur + s0, (uint32_t)__popc(m));
+                    q = __shfl_sync(0xffffffffu, q, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (!have) continue;
+                    if (s != s0) q = atomicAdd(cur + s, 1u);
+                    if (SG_IN_BOUNDS(q < w.len, 713, q)) dst[q] = k[u];
+                }
+            }
+            __syncthreads();
+        }
+        if (tid == 0) {  // the pieces, in code order from the top of the stack down
+            const uint8_t at = w.split ? w.where : (uint8_t)(1 - w.where);
+            // each level below may need a few
+            const int room = KB_PIECES - 4 * ((sh + KB_PIECE_BITS - 1) / KB_PIECE_BITS) - 1;
+            const uint64_t f0 = w.c0 >> w.bits << w.bits;  // slot 0's first code
+            int q = top, x = (int)slot_of(w.c0);
+            while (x < NS) {
+                const uint32_t b = first[x];
+                if (q >= room) {  // what is left, later
+                    sm.piece[q++] = KbPiece{f0 + ((uint64_t)x << sh), w.cend, w.off + b, w.len - b, w.bits, at, 1};
+                    break;
+                }
+                int z = x + 1;
+                if (first[z] - b > (uint32_t)TILE) {
+                    if (sh > 0)
+                        sm.piece[q++] = KbPiece{f0 + ((uint64_t)x << sh), f0 + ((uint64_t)z << sh), w.off + b,
+                                                first[z] - b, (uint8_t)sh, at, 0};
+                    x = z;
+                    continue;
+                }
+                int hi = NS;  // largest z with the records of [x, z) fitting
+                while (z < hi) {
+                    const int mid = (z + hi + 1) >> 1;
+                    if (first[mid] - b <= (uint32_t)TILE) z = mid; else hi = mid - 1;
+                }
+                // rows of A may start where there are no records
+                if (!COUNT || first[z] > b)
+                    sm.piece[q++] = KbPiece{f0 + ((uint64_t)x << sh), f0 + ((uint64_t)z << sh), w.off + b, first[z] - b,
+                                            0, at, 0};
+                x = z;
+            }
+            for (int i = top, j = q - 1; i < j; i++, j--) {
+                const KbPiece t = sm.piece[i];
+                sm.piece[i] = sm.piece[j];
+                sm.piece[j] = t;
+            }
+            sm.npiece = q;
+        }
+        __syncthreads();
     }
     return make_uint2(done, segs);
 }
 
+// alt: where the kept records go (COUNT); in either form a buffer of the plan's size that oversized buckets
+// may use beside `in`.
 template <class K, bool COUNT>
-__global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const typename K::T *__restrict__ in,
-                                                            typename K::T *__restrict__ out) {
+__global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, typename K::T *in, typename K::T *alt) {
     extern __shared__ __align__(16) unsigned char kb_raw[];
     FinishSmem<K> &sm = *reinterpret_cast<FinishSmem<K> *>(kb_raw);
     constexpr int TILE = kb_tile<K>();
     const KbPlan &pl = a.pl;
-    if (*pl.err) return;
+    if (pl.stopped()) return;
     const int64_t nsub = pl.two ? (int64_t)pl.sb[pl.nb1] : (int64_t)pl.nb1;
     const int64_t *start = pl.two ? pl.start2 : pl.start1;
     if (!COUNT && blockIdx.x == 0 && threadIdx.x == 0) a.rp[a.n_rows] = a.nnz;
@@ -779,7 +824,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const
         const uint64_t c0 = pl.two && bits < 64 ? (uint64_t)(b - pl.sb[p]) << bits : 0ull;
         uint32_t kept = 0, segs = 0;
         if (n > TILE) {
-            const uint2 r = finish_big<K, COUNT>(sm, a, p, in + s0, n, c0, bits, s0, out);
+            const uint2 r = finish_big<K, COUNT>(sm, a, p, in + s0, alt + s0, n, c0, bits, s0, alt);
             kept = r.x;
             segs = r.y;
         } else if (n > 0 || !COUNT) {
@@ -794,7 +839,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_finish_kernel(FinishArgs a, const
             if (!COUNT && lm < bits - a.cbits) lm = bits - a.cbits;
             const int ls = bits < lm ? bits : lm;
             kept = finish_group<K, COUNT>(sm, a, p, key, (int)n, c0, c0 + ((uint64_t)1 << bits), bits - ls, ls, s0,
-                                          out);
+                                          alt);
             segs = sm.nseg;
             __syncthreads();
         }
@@ -812,6 +857,7 @@ __global__ void kb_totals_kernel(const int64_t *__restrict__ pseg, KbPlan pl, co
         out[1] = pseg[2 * pl.nsub_max];
         out[2] = pl.start1[pl.nb1];
         out[3] = (int64_t)*err;
+        out[4] = (int64_t)pl.stop[1];
     }
 }
 
@@ -985,9 +1031,15 @@ static int bits_for(int64_t n) {  // bits of the ids 0 .. n - 1
 
 // A plan for `records` records with code bits `cb` above the prefix's end: prefix bits, whether a
 // second level is needed, and the device arrays (one allocation).
+// One block finishes a bucket at about 6 ns a record above its shared memory's (the whole device: 37 ps for
+// the windows, 25 for A's entries; the general form 95 and 60). Up to this limit the largest bucket costs
+// less than the general form does; beyond it the call takes that form.
+static int64_t bucket_limit(int64_t records) { return records / 128 + ((int64_t)1 << 15); }
+
 static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t records, int tile, int target, int b2min,
-                           Scratch &sc, const uint32_t *err) {
-    pl.err = err;
+                           Scratch &sc, uint32_t *stop) {
+    pl.stop = stop;
+    pl.limit = bucket_limit(records);
     pl.nb1 = 1 << pb1;
     pl.rem = cb - pb1;
     pl.two = two ? 1 : 0;
@@ -1022,7 +1074,7 @@ static sg_status second_level(KbPlan &pl, const typename K::T *in, typename K::T
     SG_LAUNCH("kmer_buckets", kb_sub2p_kernel, blocks_for((int64_t)pl.nb1 * 32, 256), 256, 0, s, pl);
     SG_LAUNCH(hname, kb_hist2_kernel<K>, nch, KB_NT, 0, s, pl, in, lowbits);
     SG_TRY(exclusive_scan<uint32_t>(pl.count2, pl.start2, pl.nsub_max, s, err));
-    SG_CUDA_TRY(cudaMemcpyAsync(pl.cur2, pl.start2, (size_t)pl.nsub_max * 8, cudaMemcpyDeviceToDevice, s));
+    SG_LAUNCH("kmer_buckets", kb_cursors_kernel, blocks_for(pl.nsub_max, 256), 256, 0, s, pl);
     const size_t sm = scatter_smem_bytes<K, false>(KB_MAXBINS);
     SG_CUDA_TRY(ensure_smem(kb_scatter2_kernel<K>, sm));
     SG_LAUNCH(sname, kb_scatter2_kernel<K>, nch, KB_NT, sm, s, pl, in, out, lowbits);
@@ -1030,23 +1082,23 @@ static sg_status second_level(KbPlan &pl, const typename K::T *in, typename K::T
 }
 
 template <class K>
-static sg_status finish_launch(const FinishArgs &a, bool count, const typename K::T *in, typename K::T *out,
+static sg_status finish_launch(const FinishArgs &a, bool count, typename K::T *in, typename K::T *alt,
                                const char *name, cudaStream_t s) {
     const size_t sm = sizeof(FinishSmem<K>);
     const int64_t grid = std::min<int64_t>(a.pl.nsub_max, (int64_t)sm_count() * 2);
     if (count) {
         SG_CUDA_TRY(ensure_smem(kb_finish_kernel<K, true>, sm));
-        SG_LAUNCH(name, (kb_finish_kernel<K, true>), grid, KB_NT, sm, s, a, in, out);
+        SG_LAUNCH(name, (kb_finish_kernel<K, true>), grid, KB_NT, sm, s, a, in, alt);
     } else {
         SG_CUDA_TRY(ensure_smem(kb_finish_kernel<K, false>, sm));
-        SG_LAUNCH(name, (kb_finish_kernel<K, false>), grid, KB_NT, sm, s, a, in, out);
+        SG_LAUNCH(name, (kb_finish_kernel<K, false>), grid, KB_NT, sm, s, a, in, alt);
     }
     return SG_OK;
 }
 
 template <class K>
 static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, bool two, int cbits, int rbits,
-                               KeyBits kb, const unsigned long long *hist, cudaStream_t s, uint32_t *err) {
+                               KeyBits kb, const unsigned long long *hist, cudaStream_t s, uint32_t *stop) {
     constexpr int TILE = kb_tile<K>();
     const int64_t m = At->n_rows, n = At->n_cols, nnz = At->nnz;
     Scratch sc(s);
@@ -1057,11 +1109,11 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     // block's records, half of them would not fit: two parts each (12 Mbp, k = 31, rows of 7,200: 4.6 ms
     // -> 3.7; rows of 4,400, 100 Mbp: parts 31 ms, rows 22)
     const int target = nnz / n > kb_target<K>() / 4 * 3 ? kb_target<K>() / 2 : kb_target<K>();
-    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, target, b2min, sc, err));
+    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, target, b2min, sc, stop));
     const int64_t ntiles = blocks_for(nnz, TILE);
     int32_t *tcol = sc.get<int32_t>(ntiles);
-    typename K::T *r0 = sc.get<typename K::T>(nnz), *r1 = two ? sc.get<typename K::T>(nnz) : nullptr;
-    if (!tcol || !r0 || (two && !r1)) return SG_ERR_OOM;
+    typename K::T *r0 = sc.get<typename K::T>(nnz), *r1 = sc.get<typename K::T>(nnz);
+    if (!tcol || !r0 || !r1) return SG_ERR_OOM;
     SG_LAUNCH("a_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, target,
               two ? std::min(KB_MAXB2, pl.rem) : 0, b2min, KB_CHUNK_TILES * TILE);
     SG_LAUNCH("a_tile_col", tile_col_kernel<TILE>, blocks_for(m, 256), 256, 0, s, At->row_ptr, m, tcol);
@@ -1069,7 +1121,7 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     SG_CUDA_TRY(ensure_smem(at_scatter_kernel<K>, sm));
     SG_LAUNCH("a_scatter1", at_scatter_kernel<K>, ntiles, KB_NT, sm, s, At->row_ptr, At->col, At->val, m, nnz,
               (const int32_t *)tcol, rest, cbits, kb, pl, r0);
-    if (two) SG_TRY(second_level<K>(pl, r0, r1, nnz, kb.low(), "a_hist2", "a_scatter2", s, err));
+    if (two) SG_TRY(second_level<K>(pl, r0, r1, nnz, kb.low(), "a_hist2", "a_scatter2", s, stop));
     FinishArgs a{};
     a.pl = pl;
     a.kb = kb;
@@ -1079,13 +1131,57 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     a.col = A->col;
     a.val = A->val;
     a.rp = A->row_ptr;
-    SG_TRY(finish_launch<K>(a, false, two ? r1 : r0, nullptr, "a_rows", s));
+    SG_TRY(finish_launch<K>(a, false, two ? r1 : r0, two ? r0 : r1, "a_rows", s));
+    return SG_OK;
+}
+
+// At's entries with their columns, for a sort by read: a thread per column.
+__global__ void at_pairs_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
+                                const uint32_t *__restrict__ val, int64_t m, uint32_t *__restrict__ key,
+                                uint64_t *__restrict__ pv) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= m) return;
+    for (int64_t e = rp[j], e1 = rp[j + 1]; e < e1; e++) {
+        key[e] = (uint32_t)col[e];
+        pv[e] = ((uint64_t)j << 32) | val[e];
+    }
+}
+
+// Sorted pairs -> A's columns and values, and the row pointers where a read's entries begin.
+__global__ void a_from_pairs_kernel(const uint32_t *__restrict__ key, const uint64_t *__restrict__ pv, int64_t nnz,
+                                    int64_t n, int32_t *__restrict__ col, uint32_t *__restrict__ val,
+                                    int64_t *__restrict__ rp, const uint32_t *__restrict__ err) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e > nnz || *err) return;  // a sort that timed out leaves words that are no reads
+    const int64_t prev = e == 0 ? -1 : (int64_t)key[e - 1], cur = e == nnz ? n : (int64_t)key[e];
+    for (int64_t r = prev + 1; r <= cur; r++) rp[r] = e;
+    if (e == nnz) return;
+    const uint64_t x = pv[e];
+    col[e] = (int32_t)(x >> 32);
+    val[e] = (uint32_t)x;
+}
+
+// A by a stable radix sort of At's entries by read (columns stay ascending): 24 bytes an entry of work
+// memory whatever the rows, 60 ps an entry against 25 by grouping. For rows that grouping cannot split
+// over enough blocks: one read of 8 Mbp among 160,000 of 1 kbp, 144 M entries, its row in two buckets: 26 ms by
+// grouping, 10 by sorting.
+sg_status transpose_sorted(const sg_csr_u32 *At, sg_csr_u32 *A, cudaStream_t s, uint32_t *err) {
+    const int64_t m = At->n_rows, n = At->n_cols, nnz = At->nnz;
+    Scratch sc(s);
+    uint32_t *k0 = sc.get<uint32_t>(nnz), *k1 = sc.get<uint32_t>(nnz);
+    uint64_t *v0 = sc.get<uint64_t>(nnz), *v1 = sc.get<uint64_t>(nnz);
+    if (!k0 || !k1 || !v0 || !v1) return SG_ERR_OOM;
+    SG_LAUNCH("at_pairs", at_pairs_kernel, blocks_for(m, 256), 256, 0, s, At->row_ptr, At->col, At->val, m, k0, v0);
+    bool alt = false;
+    SG_TRY((radix_sort_pairs<uint32_t, uint64_t>(k0, v0, k1, v1, nnz, bits_for(n), &alt, s, err)));
+    SG_LAUNCH("a_rows", a_from_pairs_kernel, blocks_for(nnz + 1, 256), 256, 0, s, (const uint32_t *)(alt ? k1 : k0),
+              (const uint64_t *)(alt ? v1 : v0), nnz, n, A->col, A->val, A->row_ptr, (const uint32_t *)err);
     return SG_OK;
 }
 
 // A = At transposed into A's arrays (allocated, nnz entries): rows ascending, columns ascending in
-// a row. pbits: bits of a position.
-sg_status transpose_impl(const sg_csr_u32 *At, sg_csr_u32 *A, int pbits, cudaStream_t s, uint32_t *err) {
+// a row. pbits: bits of a position. stop[1]: set where a bucket is too large (A is left unwritten).
+sg_status transpose_impl(const sg_csr_u32 *At, sg_csr_u32 *A, int pbits, cudaStream_t s, uint32_t *stop) {
     const int64_t m = At->n_rows, n = At->n_cols, nnz = At->nnz;
     if (nnz == 0) {
         SG_CUDA_TRY(cudaMemsetAsync(A->row_ptr, 0, (size_t)(n + 1) * 8, s));
@@ -1105,8 +1201,8 @@ sg_status transpose_impl(const sg_csr_u32 *At, sg_csr_u32 *A, int pbits, cudaStr
     SG_CUDA_TRY(cudaMemsetAsync(hist, 0, (size_t)8 << pb1, s));
     const int64_t hg = std::min<int64_t>(blocks_for(nnz, 4096), (int64_t)sm_count() * 4);
     SG_LAUNCH("a_hist1", read_hist_kernel, hg, 512, (size_t)4 << pb1, s, At->col, nnz, rbits - pb1, 1 << pb1, hist);
-    if (rbits - pb1 + cbits + kb.low() <= 64) return transpose_run<KeyN>(At, A, pb1, two, cbits, rbits, kb, hist, s, err);
-    return transpose_run<KeyW>(At, A, pb1, two, cbits, rbits, kb, hist, s, err);
+    if (rbits - pb1 + cbits + kb.low() <= 64) return transpose_run<KeyN>(At, A, pb1, two, cbits, rbits, kb, hist, s, stop);
+    return transpose_run<KeyW>(At, A, pb1, two, cbits, rbits, kb, hist, s, stop);
 }
 
 // ---------------------------------------------------------------------------- k-mer stage
@@ -1126,7 +1222,7 @@ struct KbBuild {
 template <class K>
 static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, cudaStream_t s,
                         Scratch &sc, uint32_t *err, const uint64_t *P, const uint32_t *VM, const int32_t *RG,
-                        int64_t ngroups, JobPos jp, const unsigned long long *hist, Scratch &early) {
+                        int64_t ngroups, JobPos jp, const unsigned long long *hist, Scratch &early, bool *taken) {
     using T = typename K::T;
     constexpr int TILE = kb_tile<K>();
     KbPlan pl;
@@ -1147,15 +1243,14 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
                        : run(kb_scatter1_kernel<K, decltype(kc)::value, false>);
     }));
     for (const void *p : {(const void *)P, (const void *)VM, (const void *)RG}) early.release(p);
-    const T *src = r0;
-    T *dst = r1;
+    T *src = r0, *dst = r1;
     if (q.two) {
         SG_TRY(second_level<K>(pl, r0, r1, q.total, q.kb.low(), "kmer_hist2", "kmer_scatter2", s, err));
         src = r1;
         dst = r0;
     }
     uint32_t *nseg = sc.get<uint32_t>(2 * (size_t)pl.nsub_max);
-    int64_t *pseg = sc.get<int64_t>(2 * (size_t)pl.nsub_max + 1 + 4);
+    int64_t *pseg = sc.get<int64_t>(2 * (size_t)pl.nsub_max + 1 + 5);
     if (!nseg || !pseg) return SG_ERR_OOM;
     uint32_t *nkeep = nseg + pl.nsub_max;
     int64_t *pkeep = pseg + pl.nsub_max, *totals = pseg + 2 * pl.nsub_max + 1;
@@ -1173,7 +1268,7 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
     SG_TRY(finish_launch<K>(a, true, src, dst, "kmer_finish", s));
     // both totals in one scan (nkeep follows nseg): bucket b's kept records start at pkeep[b] - m
     SG_TRY(exclusive_scan<uint32_t>(nseg, pseg, 2 * pl.nsub_max, s, err));
-    int64_t sizes[4] = {0, 0, 0, 0};  // m, m + nnz, records, error word: one copy, since each waits
+    int64_t sizes[5] = {0, 0, 0, 0, 0};  // m, m + nnz, records, the stop words: one copy, since each waits
     SG_LAUNCH("kmer_totals", kb_totals_kernel, 1, 32, 0, s, (const int64_t *)pseg, pl, (const uint32_t *)err, totals);
     SG_CUDA_TRY(read_back(sizes, totals, sizeof(sizes), s));
     const uint32_t herr = (uint32_t)sizes[3];
@@ -1182,6 +1277,8 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
         set_error("build_kmer_matrix: offsets are not a valid partition of the sequence");
         return SG_ERR_INVALID;
     }
+    if (sizes[4]) return SG_OK;  // not taken
+    *taken = true;
     const int64_t m = sizes[0], nnz = sizes[1] - m;
     if (m >= ((int64_t)1 << 31)) {
         set_error("build_kmer_matrix: %lld reliable k-mers exceed the int32 column range", (long long)m);
@@ -1208,9 +1305,10 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
 }
 
 // *taken is false where the general form has to run: a reliable range above KB_HMAX (records of
-// one code are ranked against each other), k-mers too short to spread over buckets, one prefix
-// holding a large part of a large input (a nearly constant sequence: one block would finish it
-// alone), or records that would not fit the device.
+// one code are ranked against each other), k-mers too short to spread over buckets, one prefix or one
+// bucket holding a large part of the input (low-complexity sequence: one block would finish it alone; the
+// general form then costs what it always does, after a tenth of it spent here), or records that would
+// not fit the device.
 constexpr uint32_t KB_HMAX = 1024;
 constexpr int KB_MIN_CODE = 22;
 
@@ -1287,12 +1385,11 @@ sg_status build_bucketed(const uint8_t *seq, const int64_t *off, int64_t n, int6
         const unsigned long long mx = *std::max_element(h.begin(), h.end());
         if (mx > (unsigned long long)std::max<int64_t>(total / 16, (int64_t)1 << 23)) return SG_OK;
     }
-    *taken = true;
     *pbits = q.kb.pbits;
     if (fits)
-        SG_TRY(kb_run<KeyN>(q, At, codes_out, s, sc, err, P, VM, RG, ngroups, jp, hist, early));
+        SG_TRY(kb_run<KeyN>(q, At, codes_out, s, sc, err, P, VM, RG, ngroups, jp, hist, early, taken));
     else
-        SG_TRY(kb_run<KeyW>(q, At, codes_out, s, sc, err, P, VM, RG, ngroups, jp, hist, early));
+        SG_TRY(kb_run<KeyW>(q, At, codes_out, s, sc, err, P, VM, RG, ngroups, jp, hist, early, taken));
     return SG_OK;
 }
 

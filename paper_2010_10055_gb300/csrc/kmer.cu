@@ -1076,7 +1076,7 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
                      cudaStream_t s, Scratch &sc, JobMap jm, const uint32_t *lohi,
                      unsigned long long *job_ncols, uint32_t hmax) {
     const int NT = 256;
-    uint32_t *err = sc.get<uint32_t>(4);  // error word | longest read (u64 at [2])
+    uint32_t *err = sc.get<uint32_t>(4);  // error word | a bucket is too large | longest read (u64 at [2])
     if (!err) return SG_ERR_OOM;
     unsigned long long *maxlen = (unsigned long long *)(err + 2);
     SG_CUDA_TRY(cudaMemsetAsync(err, 0, 4 * sizeof(uint32_t), s));
@@ -1088,9 +1088,13 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         SG_ALLOC(A->val, uint32_t, At->nnz, s);
         A->n_rows = n; A->n_cols = At->n_rows; A->nnz = At->nnz;
         SG_TRY(transpose_impl(At, A, pbits, s, err));
-        uint32_t herr = 0;
-        SG_CUDA_TRY(read_back(&herr, err, sizeof(uint32_t), s));
-        return herr ? timeout_error("build_kmer_matrix") : SG_OK;
+        uint32_t herr[2] = {0, 0};
+        SG_CUDA_TRY(read_back(herr, err, sizeof(herr), s));
+        if (!herr[0] && herr[1]) {
+            SG_TRY(transpose_sorted(At, A, s, err));
+            SG_CUDA_TRY(read_back(herr, err, sizeof(uint32_t), s));
+        }
+        return herr[0] ? timeout_error("build_kmer_matrix") : SG_OK;
     };
     {
         bool taken = false;
@@ -1102,6 +1106,7 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
             StageScope mat("CreateSpMat", s);
             return transpose(pbits);
         }
+        SG_CUDA_TRY(cudaMemsetAsync(err + 1, 0, sizeof(uint32_t), s));
     }
 
     const int64_t nblk = blocks_for(total, KM_CHUNK);

@@ -80,14 +80,17 @@ sg_status check_offsets(const int64_t *off, int64_t n, int64_t total, uint32_t *
                         cudaStream_t s);
 
 // The bucketed form (kbucket.cu): At and the column codes, with *pbits = bits of a position in its
-// read. *taken is false where the general form has to run.
+// read. *taken is false where the general form has to run. err[1] (zeroed): set where a bucket was too
+// large for the form.
 sg_status build_bucketed(const uint8_t *seq, const int64_t *off, int64_t n, int64_t total, int k, uint32_t lo,
                          uint32_t hi, sg_csr_u32 *At, uint64_t **codes_out, cudaStream_t s, Scratch &sc, JobMap jm,
                          const uint32_t *lohi, unsigned long long *job_ncols, uint32_t hmax, uint32_t *err,
                          const unsigned long long *maxlen, int *pbits, bool *taken);
 
 // A = At transposed into A's arrays (allocated: n + 1 row pointers, nnz entries): columns ascending
-// in a row. pbits: bits that hold every position (kbucket.cu).
-sg_status transpose_impl(const sg_csr_u32 *At, sg_csr_u32 *A, int pbits, cudaStream_t s, uint32_t *err);
+// in a row. pbits: bits that hold every position. stop: the error word and (zeroed) a word that is set where
+// a row is too long for the form; A is then unwritten, and transpose_sorted does it (kbucket.cu).
+sg_status transpose_impl(const sg_csr_u32 *At, sg_csr_u32 *A, int pbits, cudaStream_t s, uint32_t *stop);
+sg_status transpose_sorted(const sg_csr_u32 *At, sg_csr_u32 *A, cudaStream_t s, uint32_t *err);
 
 }  // namespace sg

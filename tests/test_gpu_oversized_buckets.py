@@ -1,0 +1,118 @@
+"""Buckets far above a block's shared memory, of many distinct codes: low-complexity sequence whose windows
+share a long prefix, and rows of A with millions of entries beside short ones. Bit for bit against the
+general form (radix sorts) or a plain sort, in about its time."""
+import time
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2010_10055_gb300 as sg
+
+pytestmark = pytest.mark.gpu
+
+
+def _gen(seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return g
+
+
+def _ascii(codes):
+    return torch.tensor([65, 67, 71, 84], dtype=torch.uint8, device="cuda")[codes.long()]
+
+
+def _random(seed, n, share_a=None):
+    g = _gen(seed)
+    x = torch.randint(0, 4, (n,), dtype=torch.uint8, device="cuda", generator=g)
+    if share_a is not None:  # most bases are A
+        x[torch.rand(n, device="cuda", generator=g) < share_a] = 0
+    return x
+
+
+def _low_complexity(n, tails):
+    """Uniform bases, then reads of 85 % A: about a fifth of their windows begin with nine A."""
+    return torch.cat([_random(1, n - tails), _random(2, tails, 0.8)])
+
+
+def _build(seq, off, k, lo, hi):
+    km = sg.build_kmer_matrix(seq, off, k, lo, hi)
+    out = [t.clone() for m in (km.A, km.At) for t in m.tensors().values()] + [km.codes().clone()]
+    stats = sg.last_kmer_stats()
+    km.free()
+    return out, stats
+
+
+def _time(f):
+    f()
+    ts = []
+    for _ in range(3):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        f()
+        torch.cuda.synchronize()
+        ts.append(time.perf_counter() - t)
+    return min(ts)
+
+
+def _both_forms(seq, off, k, lo, hi):
+    saved = sg.tunables()["kmer_bucketed"]
+    try:
+        out = {}
+        for form in (1, 0):
+            sg.tune("kmer_bucketed", form)
+            out[form] = (_build(seq, off, k, lo, hi), _time(lambda: sg.build_kmer_matrix(seq, off, k, lo, hi).free()))
+    finally:
+        sg.tune("kmer_bucketed", saved)
+    (got, _), t1 = out[1]
+    (exp, _), t0 = out[0]
+    assert all(torch.equal(a, b) for a, b in zip(got, exp))
+    return t1, t0
+
+
+# 3 to 16 M windows of one- and two-word records, buckets of 60 K to 1 M, finished by one block or left to the
+# general form; either way in about its time, where a search of the bucket per run of codes takes 100 times it
+@pytest.mark.parametrize("k", [17, 21, 31])
+@pytest.mark.parametrize("total,tails", [(3_000_000, 400_000), (16_000_000, 5_000_000)])
+def test_many_codes_of_one_prefix(k, total, tails):
+    seq = _ascii(_low_complexity(total, tails))
+    off = torch.arange(0, total + 1, 1000, device="cuda")
+    t1, t0 = _both_forms(seq, off, k, 2, 30)
+    assert t1 < 2 * t0 + 1e-3, (t1, t0)
+
+
+def test_single_code():
+    """Windows that are nearly all one code, and all one code."""
+    seq = _ascii(_random(3, 8_000_000, 0.999))
+    off = torch.arange(0, 8_000_001, 4000, device="cuda")
+    for k in (17, 31):
+        _both_forms(seq, off, k, 2, 40)
+    seq[:] = 65
+    t1, t0 = _both_forms(seq, off, 17, 1, 1000)
+    assert t1 < 2 * t0 + 1e-3, (t1, t0)
+
+
+@pytest.mark.parametrize("k", [17, 31])
+def test_long_row_among_short_ones(k):
+    """One read of 3 Mbp beside 60,000 reads of 500 bases of the same genome: its row of A has millions of
+    entries, in the same group of rows as a hundred short ones. A against At's entries sorted by read."""
+    G, L, n = 3_000_000, 500, 60_000
+    g = _random(4, G)
+    at = torch.randint(0, G - L, (n,), device="cuda", generator=_gen(5))
+    short = g[(at[:, None] + torch.arange(L, device="cuda")[None, :]).reshape(-1)]
+    seq = _ascii(torch.cat([short[:n // 2 * L], g, short[n // 2 * L:]]))
+    lens = torch.full((n + 1,), L, dtype=torch.int64, device="cuda")
+    lens[n // 2] = G
+    off = torch.cat([torch.zeros(1, dtype=torch.int64, device="cuda"), torch.cumsum(lens, 0)])
+    km = sg.build_kmer_matrix(seq, off, k, 2, 60)
+    A, At = km.A.tensors(), km.At.tensors()
+    assert int((A["row_ptr"][1:] - A["row_ptr"][:-1]).max()) > 2_000_000
+    m = At["row_ptr"].numel() - 1
+    col = torch.repeat_interleave(torch.arange(m, device="cuda"), At["row_ptr"][1:] - At["row_ptr"][:-1])
+    order = torch.argsort(At["col"].long(), stable=True)
+    assert torch.equal(A["col"].long(), col[order])
+    assert torch.equal(A["val"], At["val"][order])
+    counts = torch.bincount(At["col"].long(), minlength=n + 1)
+    assert torch.equal(A["row_ptr"][1:], torch.cumsum(counts, 0))
+    t = _time(lambda: sg.build_kmer_matrix(seq, off, k, 2, 60).free())
+    assert t < 0.05, t  # a second or more where each run of columns searches the bucket
