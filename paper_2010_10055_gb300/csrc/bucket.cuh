@@ -303,6 +303,7 @@ struct FinishSmem {
     uint32_t codes[KB_NT * K::ITEMS / 32 + 2];   // ... (in order) a code
     uint32_t tmp[KB_NT / 32 + 1];
     uint32_t nseg;
+    uint32_t crowd;                              // sum of the placed records' ranks in their slots
     int npiece;
     KbPiece piece[KB_PIECES];
 };
