@@ -1087,10 +1087,12 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         SG_ALLOC(A->col, int32_t, At->nnz, s);
         SG_ALLOC(A->val, uint32_t, At->nnz, s);
         A->n_rows = n; A->n_cols = At->n_rows; A->nnz = At->nnz;
-        SG_TRY(transpose_impl(At, A, pbits, s, err));
+        const sg_status grouped = transpose_impl(At, A, pbits, s, err);
+        if (grouped != SG_ERR_OOM) SG_TRY(grouped);
         uint32_t herr[2] = {0, 0};
         SG_CUDA_TRY(read_back(herr, err, sizeof(herr), s));
-        if (!herr[0] && herr[1]) {
+        // rows too long for the groups, or two-word records (32 bytes an entry) that do not fit
+        if (!herr[0] && (herr[1] || grouped == SG_ERR_OOM)) {
             SG_TRY(transpose_sorted(At, A, s, err));
             SG_CUDA_TRY(read_back(herr, err, sizeof(uint32_t), s));
         }
@@ -1100,13 +1102,22 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         bool taken = false;
         int pbits = 31;
         Scratch sb(s);
-        SG_TRY(build_bucketed(seq, off, n, total, k, lo, hi, At, codes_out, s, sb, jm, lohi, job_ncols, hmax, err,
-                              maxlen, &pbits, &taken));
+        const sg_status st = build_bucketed(seq, off, n, total, k, lo, hi, At, codes_out, s, sb, jm, lohi, job_ncols,
+                                            hmax, err, maxlen, &pbits, &taken);
+        if (st == SG_ERR_OOM) {  // the general form needs less: from the beginning, with this one's memory back
+            sg_free_csr_u32(At, (sg_stream_t)s);
+            dfree(*codes_out, s);
+            *codes_out = nullptr;
+            taken = false;
+        } else {
+            SG_TRY(st);
+        }
         if (taken) {
             StageScope mat("CreateSpMat", s);
             return transpose(pbits);
         }
         SG_CUDA_TRY(cudaMemsetAsync(err + 1, 0, sizeof(uint32_t), s));
+        if (job_ncols) SG_CUDA_TRY(cudaMemsetAsync(job_ncols, 0, (size_t)jm.njobs * sizeof(*job_ncols), s));
     }
 
     const int64_t nblk = blocks_for(total, KM_CHUNK);
