@@ -465,8 +465,8 @@ uint64_t sg_launch_count(void);
 /* Device memory of the library's two pools (temporaries of calls, outputs) on the current device, in
  * bytes, as sums over both: reserved = held by the pools (freed memory stays reserved for reuse),
  * in_use = allocated and not yet freed (library outputs the caller still holds, and work memory of
- * calls in flight), in_use_peak = the largest in_use of each pool since it was created or
- * sg_memory_reset_peak. All 0 while an allocator installed by sg_set_allocator is in use. NULL
+ * calls in flight), in_use_peak = the most that both together have held at one time since the first
+ * allocation or sg_memory_reset_peak (a block counts until its release is enqueued). All 0 while an allocator installed by sg_set_allocator is in use. NULL
  * pointers are skipped. Returns SG_OK, or SG_ERR_CUDA if the pools cannot be queried. */
 sg_status sg_memory_stats(uint64_t *reserved, uint64_t *in_use, uint64_t *in_use_peak);
 void sg_memory_reset_peak(void);

@@ -539,7 +539,7 @@ def last_kmer_stats() -> dict:
 
 
 def memory_stats() -> tuple:
-    """(reserved, in_use, in_use_peak) bytes of the library's device memory pool (see
+    """(reserved, in_use, in_use_peak) bytes of the library's two device memory pools together (see
     sg_memory_stats)."""
     r, u, h = ctypes.c_uint64(), ctypes.c_uint64(), ctypes.c_uint64()
     _check(lib().sg_memory_stats(ctypes.byref(r), ctypes.byref(u), ctypes.byref(h)), "memory_stats")

@@ -3,10 +3,12 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <map>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -81,6 +83,33 @@ static cudaMemPool_t library_pool(int which) {
         }
     }
     return g_pools[dev][which];
+}
+
+// What the pools hold for the library's callers and calls, both together, and its largest value. Each
+// pool has a high-water mark of its own, but the two are not reached at the same time (temporaries in the
+// k-mer stage, outputs at the end), so allocations are counted here: about 0.1 us each.
+static std::mutex g_use_mu;
+struct LiveBlock { size_t bytes; int dev; };
+// never destroyed: outputs may be released while the process ends
+static std::unordered_map<void *, LiveBlock> &g_live = *new std::unordered_map<void *, LiveBlock>();
+static size_t g_use[256], g_use_peak[256];
+
+static void count_alloc(void *p, size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return;
+    bytes = (bytes + 511) & ~(size_t)511;  // the pools' granularity
+    std::lock_guard<std::mutex> lk(g_use_mu);
+    g_live[p] = LiveBlock{bytes, dev};
+    g_use[dev] += bytes;
+    g_use_peak[dev] = std::max(g_use_peak[dev], g_use[dev]);
+}
+
+static void count_free(void *p) {
+    std::lock_guard<std::mutex> lk(g_use_mu);
+    const auto it = g_live.find(p);
+    if (it == g_live.end()) return;
+    g_use[it->second.dev] -= it->second.bytes;
+    g_live.erase(it);
 }
 
 // Bytes of both pools under one attribute; false if it cannot be read.
@@ -175,6 +204,7 @@ void *dalloc(size_t bytes, cudaStream_t s, bool temporary) {
                   bytes, cudaGetErrorString(e), free_b / 1e9, total_b / 1e9, reserved / 1e9, used / 1e9);
         return nullptr;
     }
+    if (pool) count_alloc(p, bytes);
     return p;
 }
 
@@ -184,6 +214,7 @@ void dfree(void *p, cudaStream_t s) {
         g_free(p, (sg_stream_t)s, g_alloc_ctx);
         return;
     }
+    count_free(p);  // before the block can be handed out again
     cudaFreeAsync(p, s);
 }
 
@@ -417,11 +448,16 @@ uint64_t sg_launch_count(void) { return sg::g_launches.load(); }
 
 sg_status sg_memory_stats(uint64_t *reserved, uint64_t *in_use, uint64_t *in_use_peak) {
     uint64_t r = 0, u = 0, h = 0;
-    if (!sg::g_alloc && !(sg::pool_bytes(cudaMemPoolAttrReservedMemCurrent, &r) &&
-                          sg::pool_bytes(cudaMemPoolAttrUsedMemCurrent, &u) &&
-                          sg::pool_bytes(cudaMemPoolAttrUsedMemHigh, &h))) {
+    int dev = 0;
+    if (!sg::g_alloc && !(cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 256 &&
+                          sg::pool_bytes(cudaMemPoolAttrReservedMemCurrent, &r) &&
+                          sg::pool_bytes(cudaMemPoolAttrUsedMemCurrent, &u))) {
         sg::set_error("memory_stats: the pools cannot be queried");
         return SG_ERR_CUDA;
+    }
+    if (!sg::g_alloc) {
+        std::lock_guard<std::mutex> lk(sg::g_use_mu);
+        h = std::max<uint64_t>(sg::g_use_peak[dev], u);
     }
     if (reserved) *reserved = r;
     if (in_use) *in_use = u;
@@ -430,11 +466,10 @@ sg_status sg_memory_stats(uint64_t *reserved, uint64_t *in_use, uint64_t *in_use
 }
 
 void sg_memory_reset_peak(void) {
-    for (int w = 0; w < 2 && !sg::g_alloc; w++) {
-        cudaMemPool_t pool = sg::library_pool(w);
-        uint64_t zero = 0;
-        if (pool && cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero) != cudaSuccess) cudaGetLastError();
-    }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return;
+    std::lock_guard<std::mutex> lk(sg::g_use_mu);
+    sg::g_use_peak[dev] = sg::g_use[dev];
 }
 
 void sg_last_kmer_stats(sg_kmer_stats *out) {
