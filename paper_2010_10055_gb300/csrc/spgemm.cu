@@ -1054,6 +1054,7 @@ struct TabGroup {
     int lT[SP_NCLS], ob[SP_NCLS];
     uint32_t cnt[SP_NCLS];
     const int32_t *rows[SP_NCLS];
+    int8_t *used;  // test hook: log2 of the table that held each row (nullptr: not recorded)
 };
 
 // 32 registers: 64 warps per SM, which the gathers' latency wants (25 Mbp at 40x: 12.3 ms a call; 40
@@ -1190,6 +1191,7 @@ __global__ void __maxnreg__(32) ctab_numeric_kernel(SpArgs g, const __grid_const
             } else {
                 o.off[i] = (int64_t)e0;
                 o.len[i] = nv;
+                if (tg.used) tg.used[i] = (int8_t)lT;
             }
         }
         int nb = 32;
@@ -1992,6 +1994,8 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
             // Mbp: 58 -> 78 ms), or where all rows are within one wave. A launch per class and a
             // second one for its overflows: 5 Mbp at 30x 1.78 ms a call, 25 Mbp at 40x 12.3; now
             // 1.33 and 11.8.
+            int8_t *used = compact && debug_record_classes() ? sc.get<int8_t>(n + 1) : nullptr;
+            if (used) SG_CUDA_TRY(cudaMemsetAsync(used, 0, (size_t)(n + 1), s));
             auto launch_group = [&](const int32_t *ls, const unsigned long long *h_cnt, int32_t *ol,
                                     unsigned long long *oc, int8_t *olt) -> sg_status {
                 struct Shape {
@@ -2016,6 +2020,7 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                     const int nt = lead.threads;
                     TabGroup tg{};
                     tg.shift = (int)tune("spgemm_escalate");
+                    tg.used = used;
                     size_t tsm = 0;
                     uint64_t nrows = 0;
                     for (; c1 >= 0; c1--) {
@@ -2253,6 +2258,14 @@ sg_status overlap_impl(const sg_csr_u32 *A, const sg_csr_u32 *At, uint32_t min_s
                     unsigned long long n_ovf2 = 0;
                     SG_CUDA_TRY(read_back(&n_ovf2, esc_counts + NCNT, sizeof(n_ovf2), s));
                     SG_TRY(mark(esc_ovf, n_ovf2, 64, true));
+                }
+                if (used) {  // rows redone in place, in a larger table of the same launch
+                    std::vector<int8_t> h_used(n);
+                    SG_CUDA_TRY(read_back(h_used.data(), used, (size_t)n, s));
+                    for (int64_t r = 0; r < n; r++)
+                        if (h_used[r] > 0 && (rec[r] < 32 ? rec[r] < h_used[r] : rec[r] < 96 + h_used[r]) &&
+                            (rec[r] < 32 || (rec[r] > 96 && rec[r] < 128)))
+                            rec[r] = 96 + h_used[r];
                 }
             }
             if (more || n_rt) SG_TRY(scans());
