@@ -2,8 +2,11 @@
 
 Coordinate descent: each tunable in turn is set to every candidate value while the others stay
 fixed, one timed call of `step` (after a warm-up call) is taken per candidate and repetition, and
-the fastest median wins. The parameters (Bloom slice size, symbolic table guess, grid sizes) only
-change speed, never results. The chosen values can be cached per GPU and workload signature.
+the fastest median wins, by MARGIN at least. The parameters (form of the k-mer stage, table guesses,
+grid sizes) only change speed, never results. Parameters of the general k-mer form are tried where the
+step runs that form: elsewhere their times differ by noise alone, and a value adopted from noise would
+act on the next input that does run it. The chosen values can be cached per GPU and workload
+signature.
 """
 from __future__ import annotations
 
@@ -14,6 +17,7 @@ import statistics
 import paper_2010_10055_gb300 as sg
 
 SPACE = {
+    "kmer_bucketed": [0, 1],
     "bloom_binned": [0, 1],
     "bloom_bin_kb": [64, 128],
     "bloom_scatter_cfg": [0, 1, 2],
@@ -33,6 +37,9 @@ SPACE = {
     "tr_blocks_per_sm": [8, 16, 32],
     "tr_warp_rows": [0, 1],
 }
+# act on the general k-mer form alone (filters, radix sort of the candidates)
+GENERAL_FORM = ("bloom_binned", "bloom_bin_kb", "bloom_scatter_cfg", "kmer_sort_buckets", "bloom_bits", "kmer_direct_seg")
+MARGIN = 0.005  # a setting is faster when it saves this share of the time: medians of one setting differ by less
 # the batched form adds the planner's thresholds
 BATCH_SPACE = {"batch_alone_kb": [32000, 64000, 128000], "batch_group_kb": [100000, 250000, 500000, 1000000]}
 
@@ -52,18 +59,29 @@ def _time_ms(step, reps: int) -> float:
     return statistics.median(ts)
 
 
-def autotune(step, space: dict | None = None, reps: int = 3, rounds: int = 1, log=None, timer=None) -> dict:
+def general_form_ran() -> bool:
+    """Whether this thread's last k-mer build sorted candidates (the general form)."""
+    return sg.last_kmer_stats()["sort_passes"] > 0
+
+
+def autotune(step, space: dict | None = None, reps: int = 3, rounds: int = 1, log=None, timer=None,
+             used_only: bool | None = None, general=general_form_ran) -> dict:
     """Tunes in place and returns {"params": chosen values, "ms": best step time, "trials": n}.
     timer(step, reps) -> ms times one setting (default: CUDA events around `step`, median of reps
-    after a warm-up call)."""
+    after a warm-up call). used_only: leave out what the step does not use (default: where no space is
+    given); general() -> whether the step just timed ran the general k-mer form."""
+    used_only = space is None if used_only is None else used_only
     space = space or SPACE
     _time = timer or _time_ms
     best = _time(step, reps)
+    best_general = used_only and general()
     trials = 1
     for _ in range(rounds):
         for name, cands in space.items():
+            if used_only and name in GENERAL_FORM and not best_general:
+                continue
             cur = sg.tunables()[name]
-            choice, choice_ms = cur, best
+            choice, choice_ms, choice_general = cur, best, best_general
             for v in cands:
                 if v == cur:
                     continue
@@ -72,10 +90,10 @@ def autotune(step, space: dict | None = None, reps: int = 3, rounds: int = 1, lo
                 trials += 1
                 if log:
                     log(f"{name}={v}: {ms:.3f} ms")
-                if ms < choice_ms:
-                    choice, choice_ms = v, ms
+                if ms < choice_ms - MARGIN * best:
+                    choice, choice_ms, choice_general = v, ms, used_only and general()
             sg.tune(name, choice)
-            best = choice_ms
+            best, best_general = choice_ms, choice_general
     return {"params": sg.tunables(), "ms": best, "trials": trials}
 
 
@@ -163,7 +181,7 @@ def _main():
             sg.transitive_reduce(R, w.fuzz)
     before = sg.tunables()
     space = {**SPACE, **BATCH_SPACE} if a.batched else SPACE
-    res = autotune(step, space=space, reps=a.reps, log=lambda s: print(s, flush=True))
+    res = autotune(step, space=space, reps=a.reps, log=lambda s: print(s, flush=True), used_only=True)
     changed = {k: (before[k], v) for k, v in res["params"].items() if before.get(k) != v}
     print(json.dumps({"signature": signature, "ms": res["ms"], "trials": res["trials"], "changed": changed,
                       "params": res["params"]}), flush=True)
