@@ -1104,7 +1104,9 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
         Scratch sb(s);
         const sg_status st = build_bucketed(seq, off, n, total, k, lo, hi, At, codes_out, s, sb, jm, lohi, job_ncols,
                                             hmax, err, maxlen, &pbits, &taken);
-        if (st == SG_ERR_OOM) {  // the general form needs less: from the beginning, with this one's memory back
+        // The general form needs less, where records are what the memory is for: from the beginning, with
+        // this one's memory back. Below a million windows (16 to 32 MB of them) the two need about the same.
+        if (st == SG_ERR_OOM && total > ((int64_t)1 << 20)) {
             sg_free_csr_u32(At, (sg_stream_t)s);
             dfree(*codes_out, s);
             *codes_out = nullptr;
