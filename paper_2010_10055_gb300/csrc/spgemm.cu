@@ -1423,7 +1423,11 @@ __global__ void fx_need_kernel(const int64_t *__restrict__ a_rp, int64_t n, Part
     if (lane == 0 && mine) atomicAdd(kept, mine);
 }
 
-// Least-squares fit of y = L (base + slope x) to the sampled rows (x = 1 - i / n), neither negative.
+// Fit of y = L (base + slope x) to the sampled rows (x = 1 - i / n), neither negative: least squares of the
+// differences over sqrt(L), so that the fitted partners add up to the sampled ones and the temporary
+// region holds the kept ones whatever the rows are like. (Unweighted, the long rows decide: among reads of
+// which two thirds have 30 entries of many partners each, the region came out too small and rows were
+// computed twice, 87,000 reads 3.7 -> 4.6 ms.)
 struct FitD {
     double base, slope;
 };
@@ -1433,11 +1437,11 @@ static FitD fit_partners(const std::vector<unsigned long long> &rec, int col, in
     for (int64_t b = 0; b < nb; b++) {
         const double L = (double)rec[3 * b], y = (double)rec[3 * b + col];
         const double x = upper ? 1.0 - (double)(b * stride) / (double)n : 0.0;
-        ll += L * L;
-        lx += L * L * x;
-        xx += L * L * x * x;
-        ly += L * y;
-        xy += L * x * y;
+        ll += L;
+        lx += L * x;
+        xx += L * x * x;
+        ly += y;
+        xy += x * y;
     }
     const double det = ll * xx - lx * lx;
     FitD f{ll > 0 ? ly / ll : 0.0, 0.0};
