@@ -1324,7 +1324,10 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
         set_error("build_kmer_matrix: offsets are not a valid partition of the sequence");
         return SG_ERR_INVALID;
     }
-    if (sizes[4]) return SG_OK;  // not taken
+    if (sizes[4]) {  // not taken; A's rows use the word again
+        SG_CUDA_TRY(cudaMemsetAsync(err + 1, 0, sizeof(uint32_t), s));
+        return SG_OK;
+    }
     *taken = true;
     const int64_t m = sizes[0], nnz = sizes[1] - m;
     if (m >= ((int64_t)1 << 31)) {

@@ -1111,6 +1111,7 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
             dfree(*codes_out, s);
             *codes_out = nullptr;
             taken = false;
+            SG_CUDA_TRY(cudaMemsetAsync(err + 1, 0, sizeof(uint32_t), s));
         } else {
             SG_TRY(st);
         }
@@ -1118,8 +1119,6 @@ sg_status build_impl(const uint8_t *seq, const int64_t *off, int64_t n, int64_t 
             StageScope mat("CreateSpMat", s);
             return transpose(pbits);
         }
-        SG_CUDA_TRY(cudaMemsetAsync(err + 1, 0, sizeof(uint32_t), s));
-        if (job_ncols) SG_CUDA_TRY(cudaMemsetAsync(job_ncols, 0, (size_t)jm.njobs * sizeof(*job_ncols), s));
     }
 
     const int64_t nblk = blocks_for(total, KM_CHUNK);
