@@ -81,6 +81,15 @@ def test_many_codes_of_one_prefix(k, total, tails):
     assert t1 < 2 * t0 + 1e-3, (t1, t0)
 
 
+def test_dominating_prefix():
+    """Above 2^24 bases, one of the first level's prefixes holds most windows: found before any are moved."""
+    seq = _ascii(torch.cat([_random(6, 8_000_000), _random(7, 12_000_000, 0.97)]))
+    off = torch.arange(0, 20_000_001, 2000, device="cuda")
+    _, stats = _build(seq, off, 17, 2, 30)
+    assert stats["sort_passes"] > 0  # the general form ran
+    _both_forms(seq, off, 17, 2, 30)
+
+
 def test_single_code():
     """Windows that are nearly all one code, and all one code."""
     seq = _ascii(_random(3, 8_000_000, 0.999))
