@@ -109,6 +109,7 @@ __device__ __forceinline__ void load_chunk(uint32_t *smw, const uint8_t *__restr
 // (window_key). Thread t of block b covers windows and bases b * KM_CHUNK + t * KM_W + j, j < KM_W,
 // reading bases [t * KM_W, t * KM_W + KM_W + k - 1) of the block's chunk. K > 0 makes k a
 // compile-time constant (K == 0: k taken from k_rt).
+constexpr uint64_t WC_STRAND = 1ull << 63;
 constexpr uint32_t H_NONE = 0xFFFFFFFFu;
 constexpr uint32_t B1_SEED = 0x9e3779b9u, B2_SEED = 0x7f4a7c15u;
 static_assert(KM_W == 32, "one packed word per thread");
@@ -181,6 +182,22 @@ __global__ void __launch_bounds__(KM_NT) pack_kernel(const uint8_t *__restrict__
         }
     }
     P[qs >> 5] = pw;
+}
+
+// Key of window q = 32g + lane from P[g] = w0 and P[g + 1] = w1 (a valid window): the canonical
+// code (with the job prefix) | strand << 63. The 2k bits from
+// bit 2 * lane of w1:w0 hold the window's bases, first base lowest; complementing them gives the
+// reverse complement's code (last base's complement highest), and reversing the order of the
+// 2-bit groups gives the forward code (first base highest).
+__device__ __forceinline__ uint64_t window_key(uint64_t w0, uint64_t w1, int lane, int k, JobPosCursor &jc,
+                                               int64_t q) {
+    const int sh = 2 * lane;
+    const uint64_t x = sh ? (w0 >> sh) | (w1 << (64 - sh)) : w0;
+    const uint64_t rc = ~x & ((1ull << (2 * k)) - 1);  // k <= 31
+    uint64_t y = __brevll(x);
+    y = ((y >> 1) & 0x5555555555555555ull) | ((y & 0x5555555555555555ull) << 1);
+    const uint64_t fw = y >> (64 - 2 * k);
+    return jc.prefix(q) | (fw < rc ? fw : rc) | (rc < fw ? WC_STRAND : 0ull);
 }
 
 // One launch per slice [w_lo, w_hi) of B1's words: every launch streams all window hashes but

@@ -7,8 +7,6 @@
 
 namespace sg {
 
-constexpr uint64_t WC_STRAND = 1ull << 63;
-
 // Batches: the job prefix of a window, from the base offset of each job's first read (jpos[b] =
 // off[ro[b]], jpos[njobs] = total). A window lies in the last job b with jpos[b] <= its position
 // (windows never cross reads, and empty jobs start where the next one does). The cursor keeps the
@@ -45,22 +43,6 @@ static __global__ void job_pos_kernel(const int64_t *__restrict__ ro, int64_t nj
     int64_t r = ro[b];
     r = r < 0 ? 0 : (r > n ? n : r);
     jpos[b] = off[r];
-}
-
-// Key of window q = 32g + lane from P[g] = w0 and P[g + 1] = w1 (a valid window): the canonical
-// code (with the job prefix) | strand << 63. The 2k bits from
-// bit 2 * lane of w1:w0 hold the window's bases, first base lowest; complementing them gives the
-// reverse complement's code (last base's complement highest), and reversing the order of the
-// 2-bit groups gives the forward code (first base highest).
-__device__ __forceinline__ uint64_t window_key(uint64_t w0, uint64_t w1, int lane, int k, JobPosCursor &jc,
-                                               int64_t q) {
-    const int sh = 2 * lane;
-    const uint64_t x = sh ? (w0 >> sh) | (w1 << (64 - sh)) : w0;
-    const uint64_t rc = ~x & ((1ull << (2 * k)) - 1);  // k <= 31
-    uint64_t y = __brevll(x);
-    y = ((y >> 1) & 0x5555555555555555ull) | ((y & 0x5555555555555555ull) << 1);
-    const uint64_t fw = y >> (64 - 2 * k);
-    return jc.prefix(q) | (fw < rc ? fw : rc) | (rc < fw ? WC_STRAND : 0ull);
 }
 
 // Runs f with k as a compile-time constant for the common k (17 is the paper's), else 0.
