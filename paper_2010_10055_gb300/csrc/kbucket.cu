@@ -35,22 +35,45 @@ namespace sg {
 static inline int64_t blocks_for(int64_t n, int nt) { return (n + nt - 1) / nt; }
 
 __global__ void __launch_bounds__(1024) kb_plan_kernel(const unsigned long long *__restrict__ hist, KbPlan pl,
-                                                      int target, int b2max, int b2min, int chunk) {
+                                                      int target, int b2max, int b2min, float skew, float skew_max, int pb1,
+                                                      int chunk) {
     __shared__ int64_t t64[33];
     __shared__ uint32_t t32[33];
     __shared__ int64_t s_base;
     __shared__ uint32_t s_sub, s_chk;
+    __shared__ float s_s, s_ss;
     if (threadIdx.x == 0) {
         s_base = 0;
         s_sub = 0;
         s_chk = 0;
+        s_s = s_ss = 0.0f;
     }
     __syncthreads();
+    const int grow_max = skew < 0.0f ? KB_SMALL_GROW : KB_MAXB2;
+    if (skew < 0.0f) {
+        float s = 0.0f, ss = 0.0f;
+        for (int p = threadIdx.x; p < pl.nb1; p += 1024) {
+            const float c = (float)hist[p];
+            s += c;
+            ss += c * c;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&s_s, s);
+            atomicAdd(&s_ss, ss);
+        }
+        __syncthreads();
+        skew = kb_skew(s_s, s_ss, pl.nb1, pb1);
+    }
+    if (threadIdx.x == 0 && skew >= skew_max) pl.stop[1] = 1;
     for (int p0 = 0; p0 < pl.nb1; p0 += 1024) {
         const int p = p0 + threadIdx.x;
         const int64_t c = p < pl.nb1 ? (int64_t)hist[p] : 0;
-        int b = b2min;
-        while (b < b2max && (c >> b) > target) b++;
+        const int b = kb_split(c, target, b2max, b2min, skew, grow_max);
         const uint32_t nch = p < pl.nb1 ? (uint32_t)((c + chunk - 1) / chunk) : 0u;
         int64_t tot;
         uint32_t stot, ctot;
@@ -344,6 +367,7 @@ __global__ void __launch_bounds__(KB_NT, 2) kb_scatter1_kernel(WindowSrc w, KbPl
             s_group[warp][lane] = d;
         }
     }
+    if (pl.stopped()) return;
     for (int i = threadIdx.x; i < nb; i += KB_NT) cnt[i] = 0;
     __syncthreads();
     const uint64_t rmask = (1ull << w.kb.rbits) - 1;
@@ -1083,7 +1107,13 @@ static int bits_for(int64_t n) {  // bits of the ids 0 .. n - 1
 // less than the general form does; beyond it the call takes that form.
 static int64_t bucket_limit(int64_t records) { return records / 128 + ((int64_t)1 << 15); }
 
-static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t records, int tile, int target, int b2min,
+// A prefix of c records splits into fewer than 2 c / target + 1 buckets (2^b2min at least).
+static int64_t split_bound(int64_t records, int target, int pb1, int b2min) {
+    return ((int64_t)1 << (pb1 + b2min)) + 2 * (records / target + 1);
+}
+
+// buckets: their number at most, for a second level.
+static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t records, int tile, int64_t buckets,
                            Scratch &sc, uint32_t *stop) {
     pl.stop = stop;
     pl.limit = bucket_limit(records);
@@ -1091,8 +1121,7 @@ static sg_status make_plan(KbPlan &pl, int pb1, int cb, bool two, int64_t record
     pl.rem = cb - pb1;
     pl.two = two ? 1 : 0;
     pl.cap = records;
-    // a prefix of c records splits into fewer than 2 c / target + 1 buckets (2^b2min at least)
-    pl.nsub_max = two ? ((int64_t)pl.nb1 << b2min) + 2 * (records / target + 1) : pl.nb1;
+    pl.nsub_max = two ? buckets : pl.nb1;
     const size_t nb = (size_t)pl.nb1, ns = two ? (size_t)pl.nsub_max : 0;
     const size_t nc = two ? (size_t)(records / (KB_CHUNK_TILES * (int64_t)tile) + pl.nb1) : 0;  // a partial chunk per prefix
     const size_t words = (nb + 1) + nb + (ns + 1) + ns;  // 8-byte arrays
@@ -1133,13 +1162,13 @@ static sg_status finish_launch(const FinishArgs &a, bool count, typename K::T *i
                                const char *name, cudaStream_t s) {
     const size_t sm = sizeof(FinishSmem<K>);
     const int64_t grid = std::min<int64_t>(a.pl.nsub_max, (int64_t)sm_count() * 2);
-    if (count) {
-        SG_CUDA_TRY(ensure_smem(kb_finish_kernel<K, true>, sm));
-        SG_LAUNCH(name, (kb_finish_kernel<K, true>), grid, KB_NT, sm, s, a, in, alt);
-    } else {
-        SG_CUDA_TRY(ensure_smem(kb_finish_kernel<K, false>, sm));
-        SG_LAUNCH(name, (kb_finish_kernel<K, false>), grid, KB_NT, sm, s, a, in, alt);
-    }
+    auto run = [&](auto kern) -> sg_status {
+        SG_CUDA_TRY(ensure_smem(kern, sm));
+        SG_LAUNCH(name, kern, grid, KB_NT, sm, s, a, in, alt);
+        return SG_OK;
+    };
+    if (count) SG_TRY(run(kb_finish_kernel<K, true>));
+    else SG_TRY(run(kb_finish_kernel<K, false>));
     return SG_OK;
 }
 
@@ -1156,13 +1185,14 @@ static sg_status transpose_run(const sg_csr_u32 *At, sg_csr_u32 *A, int pb1, boo
     // block's records, half of them would not fit: two parts each (12 Mbp, k = 31, rows of 7,200: 4.6 ms
     // -> 3.7; rows of 4,400, 100 Mbp: parts 31 ms, rows 22)
     const int target = nnz / n > kb_target<K>() / 4 * 3 ? kb_target<K>() / 2 : kb_target<K>();
-    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, target, b2min, sc, stop));
+    SG_TRY(make_plan(pl, pb1, rbits + cbits, two, nnz, TILE, split_bound(nnz, target, pb1, b2min), sc, stop));
     const int64_t ntiles = blocks_for(nnz, TILE);
     int32_t *tcol = sc.get<int32_t>(ntiles);
     typename K::T *r0 = sc.get<typename K::T>(nnz), *r1 = sc.get<typename K::T>(nnz);
     if (!tcol || !r0 || !r1) return SG_ERR_OOM;
     SG_LAUNCH("a_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, target,
-              two ? std::min(KB_MAXB2, pl.rem) : 0, b2min, KB_CHUNK_TILES * TILE);
+              two ? std::min(KB_MAXB2, pl.rem) : 0, b2min, 0.0f, 1.0f, pb1,
+              KB_CHUNK_TILES * TILE);
     SG_LAUNCH("a_tile_col", tile_col_kernel<TILE>, blocks_for(m, 256), 256, 0, s, At->row_ptr, m, tcol);
     const size_t sm = scatter_smem_bytes<K, true>(pl.nb1);
     SG_CUDA_TRY(ensure_smem(at_scatter_kernel<K>, sm));
@@ -1264,6 +1294,8 @@ struct KbBuild {
     int cb, job_bits, pb1;
     bool two;
     KeyBits kb;
+    std::vector<unsigned long long> counts;  // large inputs: windows of each prefix
+    float skew, skew_max;                    // of the codes (negative: found on the device); not taken from here on
 };
 
 template <class K>
@@ -1273,9 +1305,15 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
     using T = typename K::T;
     constexpr int TILE = kb_tile<K>();
     KbPlan pl;
-    SG_TRY(make_plan(pl, q.pb1, q.cb, q.two, q.total, TILE, kb_target<K>(), 0, sc, err));
-    SG_LAUNCH("kmer_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, kb_target<K>(),
-              q.two ? std::min(KB_MAXB2, pl.rem) : 0, 0, KB_CHUNK_TILES * TILE);
+    constexpr int TARGET = kb_target<K>();
+    const int b2max = q.two ? std::min(KB_MAXB2, q.cb - q.pb1) : 0;
+    int64_t buckets = 0;  // exactly, where the host has the prefixes' counts
+    for (const unsigned long long c : q.counts)
+        buckets += (int64_t)1 << kb_split((int64_t)c, TARGET, b2max, 0, q.skew, KB_MAXB2);
+    if (q.counts.empty()) buckets = split_bound(q.total, TARGET, q.pb1, 0) << (q.skew < 0.0f ? KB_SMALL_GROW : 0);
+    SG_TRY(make_plan(pl, q.pb1, q.cb, q.two, q.total, TILE, buckets, sc, err));
+    SG_LAUNCH("kmer_plan", kb_plan_kernel, 1, 1024, 0, s, hist, pl, TARGET, b2max, 0, q.skew, q.skew_max,
+              q.pb1, KB_CHUNK_TILES * TILE);
     T *r0 = sc.get<T>(q.total), *r1 = sc.get<T>(q.total);
     if (!r0 || !r1) return SG_ERR_OOM;
     const WindowSrc w{P, VM, RG, q.off, q.n, ngroups, q.k, jp, pl.rem, q.kb};
@@ -1361,6 +1399,14 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
 // not fit the device.
 constexpr uint32_t KB_HMAX = 1024;
 constexpr int KB_MIN_CODE = 22;
+// Skewed codes cost the bucketed form more (buckets of unequal size, records that share slots), the sorts
+// not. Times of both, ms, 120 M windows, k = 17: 60 % A and T 4.9 and 5.6, 65 % 5.4 and 5.8, 70 % 6.4 and
+// 6.2, 75 % 7.8 and 6.9, 80 % 9.8 and 8.2 at 10 % errors; at 1 % 80 % 12.2 and 12.6. With long k-mers, which
+// accurate reads go with, the sorts move pairs and lose: k = 21 at 1 % errors 14.0 and 20.9. Below two
+// million windows launches decide: 1 M windows at 80 % 0.36 and 0.43.
+constexpr float KB_SKEW_MAX = 0.15f;  // about 73 % A and T
+constexpr int KB_SKEW_K = 19;
+constexpr int64_t KB_SKEW_TOTAL = (int64_t)1 << 21;
 
 sg_status build_bucketed(const uint8_t *seq, const int64_t *off, int64_t n, int64_t total, int k, uint32_t lo,
                          uint32_t hi, sg_csr_u32 *At, uint64_t **codes_out, cudaStream_t s, Scratch &sc, JobMap jm,
@@ -1368,7 +1414,11 @@ sg_status build_bucketed(const uint8_t *seq, const int64_t *off, int64_t n, int6
                          const unsigned long long *maxlen, int *pbits, bool *taken) {
     *taken = false;
     if (!tune("kmer_bucketed") || hmax > KB_HMAX || 2 * k < KB_MIN_CODE || total <= 0 || n <= 0) return SG_OK;
-    KbBuild q{seq, off, n, total, k, lo, hi, hmax, lohi, job_ncols, 0, 0, 0, false, {}};
+    KbBuild q{seq, off, n, total, k, lo, hi, hmax, lohi, job_ncols, 0, 0, 0, false, {}, {}, 0.0f, 1.0f};
+    if (!jm.ro && total > KB_SKEW_TOTAL) {  // (prefixes of read sets differ by their sizes)
+        q.skew = -1.0f;
+        if (k <= KB_SKEW_K) q.skew_max = KB_SKEW_MAX;
+    }
     while (jm.ro && ((int64_t)1 << q.job_bits) < jm.njobs) q.job_bits++;
     q.cb = 2 * k + q.job_bits;
     const bool large = total > ((int64_t)1 << 24);
@@ -1430,9 +1480,17 @@ sg_status build_bucketed(const uint8_t *seq, const int64_t *off, int64_t n, int6
     SG_LAUNCH("pack", kb_pack_kernel, blocks_for(blocks_for(steps, (int)spw), PK_NT / 32), PK_NT, (size_t)nb1 * 4, s, seq,
               total, off, n, k, jp, q.pb1, q.job_bits, ngroups, spw, P, VM, RG, hist);
     if (large) {
-        std::vector<unsigned long long> h(nb1);
-        SG_CUDA_TRY(read_back(h.data(), hist, (size_t)nb1 * 8, s));
-        const unsigned long long mx = *std::max_element(h.begin(), h.end());
+        q.counts.resize(nb1);
+        SG_CUDA_TRY(read_back(q.counts.data(), hist, (size_t)nb1 * 8, s));
+        unsigned long long mx = 0;
+        double sum = 0.0, squares = 0.0;
+        for (const unsigned long long c : q.counts) {
+            mx = std::max(mx, c);
+            sum += (double)c;
+            squares += (double)c * (double)c;
+        }
+        if (!jm.ro) q.skew = kb_skew((float)sum, (float)squares, nb1, q.pb1);
+        if (q.skew >= q.skew_max) return SG_OK;
         if (mx > (unsigned long long)std::max<int64_t>(total / 16, (int64_t)1 << 23)) return SG_OK;
     }
     *pbits = q.kb.pbits;
