@@ -473,9 +473,9 @@ void sg_memory_reset_peak(void);
 
 /* Tunable launch parameters (used by the autotuner; results never depend on them):
  *   kmer_bucketed         1: every window grouped by its code and counted in shared memory, where
- *                         that form applies (hi up to 1024, k of 11 or more, no prefix that holds
- *                         much of the input, records that fit the device); 0: the general form
- *                         (filters and radix sort), which the next tunables are about (1)
+ *                         that form applies (hi up to 1024, k of 11 or more, codes not too unequal,
+ *                         records that fit the device); 0: the general form (filters and radix
+ *                         sort), which the next tunables are about (1)
  *   bloom_bits            bits of the first-level Bloom filter per window (8): fewer bits, fewer
  *                         slices but more false positives (singletons that reach the exact count)
  *   bloom_slice_mb        megabytes of the first-level Bloom filter updated per launch (64)

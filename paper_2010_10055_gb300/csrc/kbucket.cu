@@ -17,11 +17,12 @@
 // windows are singletons and cost one random probe per window; here a singleton costs its share of
 // three or four streaming passes, and drops out when its slot counts one record.
 //
-// 4.1 G windows, 1.77 G entries of A (100 Mbp at 40x, k = 17), ms: pack 3.8, scatter1 25, hist2 4.5,
-// scatter2 18.5, finish 52, emit 8.6, A 44 (scatter1 11.7, hist2 2, scatter2 7, rows 22.4): 157 in all,
+// 4.1 G windows, 1.77 G entries of A (100 Mbp at 40x, k = 17), ms: pack 4, scatter1 25, hist2 4.5,
+// scatter2 18, finish 50, emit 8.5, A 43 (scatter1 11.8, hist2 2, scatter2 7, rows 21.5): 154 in all,
 // against 387 for filters, sorts and segment passes (the general form in kmer.cu with a radix sort of
-// A). 154 M windows (5 Mbp at 30x): 4.7 against 5.9; k = 31, 300 M windows: 24.8 against 58 (16-byte
-// records, eight radix passes).
+// A). 154 M windows (5 Mbp at 30x): 4.5 against 5.9; k = 31, 300 M windows: 24 against 58 (16-byte
+// records, eight radix passes). These are uniform sequences; what skewed ones cost is told where the split
+// of the prefixes, the oversized buckets and the crowded slots are dealt with.
 #include <algorithm>
 #include <vector>
 
@@ -485,7 +486,7 @@ __device__ __noinline__ void sort_block(typename K::T *sk, int n) {
 // [c0, cend), at most 2^ls << sh wide: slot = (code - c0) >> sh. Returns the number of records
 // written, from base on. All threads call it. Loops over a thread's records end, for the whole
 // block, where its records do.
-// Bound by its chain of shared-memory phases, about 12 ps a record (4.1e9 records 52 ms): load and count
+// Bound by its chain of shared-memory phases, about 12 ps a record (4.1e9 records 50 ms; when 52): load and count
 // 11 ms, slot starts 5, placing 10, ranking within a slot 11.5, codes 3, keeping 5, writing 6. Blocks of
 // 256 threads with half the records 57 ms; the next bucket's records prefetched 60. Counting first drops
 // the records that are alone in their slot, so a singleton is neither placed nor ranked.
@@ -1395,8 +1396,8 @@ static sg_status kb_run(const KbBuild &q, sg_csr_u32 *At, uint64_t **codes_out, 
 // *taken is false where the general form has to run: a reliable range above KB_HMAX (records of
 // one code are ranked against each other), k-mers too short to spread over buckets, one prefix or one
 // bucket holding a large part of the input (low-complexity sequence: one block would finish it alone; the
-// general form then costs what it always does, after a tenth of it spent here), or records that would
-// not fit the device.
+// general form then costs what it always does, after a tenth of it spent here), short k-mers whose codes are
+// too skewed, or records that would not fit the device.
 constexpr uint32_t KB_HMAX = 1024;
 constexpr int KB_MIN_CODE = 22;
 // Skewed codes cost the bucketed form more (buckets of unequal size, records that share slots), the sorts

@@ -9,8 +9,9 @@
 //
 // Default: the bucketed form (kbucket.cu), which groups every window by its code and counts in
 // shared memory. The general form below takes what that form leaves: reliable ranges past 1,024,
-// k-mers of fewer than 11 bases, inputs of which one code prefix holds a large part, and inputs
-// whose records would not fit the device. Its pipeline (all on `stream`):
+// k-mers of fewer than 11 bases, inputs of which one code prefix or bucket holds a large part, short k-mers
+// of very unequal composition, and inputs whose records do not fit the device. Its pipeline (all on
+// `stream`):
 //  0. pack           one walk over the reads packs the bases (2 bits each) and stores each
 //                    window's 32-bit filter hash (H_NONE where no valid window starts); later
 //                    passes recompute a window's canonical code and strand from two packed words.
